@@ -175,6 +175,10 @@ wf_status wf_level0_schedule(int64_t n, int levels, int64_t k, int32_t* keep);
  * Outputs: idx int32 [B*H][keep[0]] token positions, ascending per unit.
  * level_sets (optional, NULL to skip): int32
  * [B*H][keep[L] + .. + keep[1] + keep[0]] = J_L, .., J_1, mu^0 per unit.
+ * For bf16 keys with head_dim 128 the whole filter is one launch of wf_step's
+ * fused kernel without its attention (one query head per key head) or of its
+ * grouped filter kernel, within those kernels' limits (see wf_step); other
+ * shapes run three kernels a scale.
  * ws: device scratch of at least wf_filter_workspace_bytes() bytes,
  * 256-byte aligned.  Its first 4 bytes are a status word: for bf16 keys with
  * head_dim 128 the scores run on the tensor cores, and a kernel whose bounded

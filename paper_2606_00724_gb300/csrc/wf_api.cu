@@ -139,6 +139,32 @@ wf_status check_attn_args(const wf_tensor* q, const wf_tensor* kv, int k, const 
   return WF_OK;
 }
 
+// The skim and scan of one layer: wf_step's fused kernel without its attention
+// where it applies (one launch; one query head per key head), else the grouped
+// filter kernel, else three kernels a scale.  wf_filter's scratch beyond the
+// status word is used by the last only.  The line lies where the kernels'
+// limits do, because one launch is faster over the whole range: 32 heads x
+// 20K tokens, filter then attention, 152 us with 13 launches for the filter
+// and 69 us with one.
+cudaError_t run_filter(const wf::FilterPlan& p, const void* Q, const wf_tensor& q, const void* coeffs, const void* K,
+                       const wf_tensor& kv, int levels, const int32_t* keep, int32_t* idx, int32_t* level_sets,
+                       void* scratch, int* status, int sms, cudaStream_t s) {
+  if (q.heads == kv.heads) {
+    const wf::FusedPlan fp = wf::plan_fused(q, kv, levels, keep, -1, sms);
+    if (fp.ok) {
+      wf::FusedRange r{};
+      r.lev_top = levels;
+      r.lev_bot = fp.trim ? 0 : 1;
+      r.final_sel = 1;
+      return wf::launch_fused(fp, Q, q, K, nullptr, kv, nullptr, nullptr, nullptr, coeffs, levels, keep, idx,
+                              level_sets, nullptr, q, status, s, &r);
+    }
+  }
+  const wf::GqaPlan gp = wf::plan_gqa(q, kv, levels, keep, sms);
+  if (gp.ok) return wf::launch_gqa_filter(gp, Q, q, K, kv, coeffs, levels, keep, idx, level_sets, status, s);
+  return wf::launch_filter(p, Q, q, coeffs, K, kv, idx, level_sets, scratch, status, s);
+}
+
 }  // namespace
 
 WF_API const char* wf_status_str(int status) {
@@ -258,8 +284,11 @@ WF_API wf_status wf_filter(const void* Q, const wf_tensor* q, const void* coeffs
     return WF_ERR_ALIGN;
   const wf::FilterPlan p = wf::plan_filter(*q, *kv, levels, keep);
   if (ws_bytes < p.total) return WF_ERR_WORKSPACE;
-  return cuda_status(wf::launch_filter(p, Q, *q, coeffs, K, *kv, idx, level_sets, ws, static_cast<int*>(ws),
-                                       static_cast<cudaStream_t>(stream)));
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  int sms = 0;
+  if (!device_sms(&sms)) return WF_ERR_CUDA;
+  return cuda_status(run_filter(p, Q, *q, coeffs, K, *kv, levels, keep, idx, level_sets, ws, static_cast<int*>(ws),
+                                sms, s));
 }
 
 WF_API wf_status wf_wavelet_approx(const void* K, const wf_tensor* kv, const int32_t* cand, int m, int level,
@@ -298,7 +327,7 @@ WF_API wf_status wf_filter_wavelet(const void* Q, const wf_tensor* q, const void
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int sms = 0;
   if (!device_sms(&sms)) return WF_ERR_CUDA;
-  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, 0, nullptr, sms);
+  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, -1, sms);
   if (fp.ok && q->heads == kv->heads)
     return cuda_status(wf::launch_literal_fused(fp, p, Q, *q, top, K, nullptr, *kv, nullptr, nullptr, nullptr,
                                                 wavelet, idx, level_sets, nullptr, nullptr, ws,
@@ -370,25 +399,18 @@ WF_API wf_status wf_step(const void* Q, const wf_tensor* q, const void* K, const
   void* scratch = static_cast<char*>(ws) + kStatusBytes;
   cudaError_t e = cudaSuccess;
   if (refresh_coeffs && (e = wf::launch_dwt(K, *kv, levels, coeffs, s)) != cudaSuccess) return WF_ERR_CUDA;
-  // The fused kernel takes one query head per KV head; grouped heads run the per-stage kernels.
-  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, n_g, n_g > 0 ? g : nullptr, sms);
+  // The fused kernel takes one query head per KV head.
+  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, n_g, sms);
   if (fp.ok && q->heads == kv->heads) {
     e = wf::launch_fused(fp, Q, *q, K, V, *kv, Kg, Vg, n_g > 0 ? g : nullptr, coeffs, levels, keep, idx,
                          level_sets, O, *o, status, s);
     return cuda_status(e);
   }
-  // Grouped query heads: the grouped filter kernel where it applies, else the
-  // per-stage filter; then the per-stage attention.
-  const wf::GqaPlan gp = wf::plan_gqa(*q, *kv, levels, keep, sms);
-  if (gp.ok) {
-    if ((e = wf::launch_gqa_filter(gp, Q, *q, K, *kv, coeffs, levels, keep, idx, level_sets, status, s)) !=
-        cudaSuccess)
-      return WF_ERR_CUDA;
-  } else {
-    const wf::FilterPlan fl = wf::plan_filter(*q, *kv, levels, keep);
-    if ((e = wf::launch_filter(fl, Q, *q, coeffs, K, *kv, idx, level_sets, scratch, status, s)) != cudaSuccess)
-      return WF_ERR_CUDA;
-  }
+  // Otherwise the filter (wf_filter's kernels), then the per-stage attention.
+  const wf::FilterPlan fl = wf::plan_filter(*q, *kv, levels, keep);
+  if ((e = run_filter(fl, Q, *q, coeffs, K, *kv, levels, keep, idx, level_sets, scratch, status, sms, s)) !=
+      cudaSuccess)
+    return WF_ERR_CUDA;
   const wf::AttnPlan ap = wf::plan_attn(*q, keep[0], n_g, group_of(q, kv));
   const float sc = 1.0f / sqrtf((float)q->head_dim);
   e = wf::launch_attn(ap, Q, *q, K, V, *kv, idx, Kg, Vg, n_g > 0 ? g : nullptr, O, *o, sc, scratch, status, s);
@@ -427,7 +449,7 @@ WF_API wf_status wf_step_wavelet(const void* Q, const wf_tensor* q, const void* 
   int* status = static_cast<int*>(ws);
   void* scratch = static_cast<char*>(ws) + kStatusBytes;
   const wf::FilterPlan fl = wf::plan_filter(*q, *kv, levels, keep);
-  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, n_g, n_g > 0 ? g : nullptr, sms);
+  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, n_g, sms);
   if (fp.ok && q->heads == kv->heads)
     return cuda_status(wf::launch_literal_fused(fp, fl, Q, *q, top, K, V, *kv, Kg, Vg, n_g > 0 ? g : nullptr, wavelet,
                                                 idx, level_sets, O, o, scratch, status, s));

@@ -2288,9 +2288,7 @@ int max_active_clusters(int stages, bool wide, int cs, size_t smem) {
 
 }  // namespace
 
-FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g,
-                     const wf_tensor* g, int num_sms) {
-  (void)g;
+FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g, int num_sms) {
   FusedPlan fp{};
   fp.ok = false;
   if (kv.dtype != WF_BF16 || kv.head_dim != D || q.seq > NQ || levels > 10) return fp;
@@ -2301,7 +2299,7 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   for (int l = 0; l <= levels; ++l) kmax = kmax > keep[l] ? kmax : keep[l];
   for (int l = 1; l <= levels; ++l) cmax = cmax > 2 * keep[l] ? cmax : 2 * keep[l];
   if (cmax > kMaxCand || kmax > kMaxCand) return fp;
-  const int total = keep[0] + n_g;
+  const int total = n_g < 0 ? 0 : keep[0] + n_g;  // keys of the attention
   // TMEM columns of one unit's region at cluster size cs: the widest scale
   // slice, or the attention slice plus the O^T accumulator.
   // TMEM tiles of the widest scale slice at cluster size cs.
@@ -2316,7 +2314,7 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   };
   auto unit_cols = [&](int cs) {
     int tmax = scale_tiles(cs);
-    const int ta = ((total + cs - 1) / cs + TM - 1) / TM + 1;
+    const int ta = total > 0 ? ((total + cs - 1) / cs + TM - 1) / TM + 1 : 0;
     tmax = tmax > ta ? tmax : ta;
     return 32 * tmax;
   };

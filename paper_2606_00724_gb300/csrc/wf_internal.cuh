@@ -143,8 +143,8 @@ struct FusedPlan {
   bool trim;
   bool wide;  // one unit per cluster served by both compute warpgroups
 };
-FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g,
-                     const wf_tensor* g, int num_sms);
+// n_g: generation rows of the attention, or -1 for a plan of the filter alone.
+FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g, int num_sms);
 // Part of the chain in one launch (the literal-basis path runs one launch per
 // scale, with the transform of the candidates' blocks between launches):
 // scales lev_top down to lev_bot; the previous selection J_{lev_top+1} as its

@@ -1,0 +1,55 @@
+"""Which kernels wf_filter takes, at the edges of each route: the fused kernel
+without its attention (bf16, head_dim 128, at most 32 query rows, one query
+head a key head), the grouped filter kernel (grouped heads), and the kernels
+per scale past those kernels' 8192 candidates a scale.  Indices and
+level sets bit-exact against the fp64 oracle on planted inputs, which have a
+margin at every Top-K boundary; also for [B, rows, H, d] strides and without
+level sets."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import LibRun, f64
+from paper_2606_00724_gb300 import synth, wf
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+
+def _bshd(t):
+    return t.transpose(1, 2).contiguous().transpose(1, 2)
+
+
+@pytest.mark.parametrize("B,H,group,q,n,L,k,bshd", [
+    (1, 3, 1, 1, 2048, 1, 301, False),    # one query row, one scale, an odd k (token trim), units that pair unevenly
+    (1, 1, 1, 32, 256, 3, 8, True),       # one unit, fewer candidates than one tile
+    (2, 3, 1, 32, 4104, 3, 512, True),    # ragged n, [B, rows, H, d] strides
+    (1, 2, 1, 17, 16384, 1, 4096, False),  # 8192 candidates: the largest list of the fused kernel
+    (1, 1, 1, 17, 16640, 1, 4096, False),  # 8320 candidates: the kernels per scale
+    (1, 2, 4, 32, 4104, 3, 513, True),    # grouped heads, ragged n, token trim
+])
+def test_filter_route(B, H, group, q, n, L, k, bshd):
+    w = synth.Workload("filter_route", B, H, 128, n, q, 1, L, tuple(wf.wf_default_schedule(n, L, k)), "bf16", "iid",
+                       group=group)
+    b = synth.make_batch(w, planted=True, device="cuda", cfg="route")
+    if bshd:
+        b = dataclasses.replace(b, Q=_bshd(b.Q), K=_bshd(b.K), V=_bshd(b.V))
+    run = LibRun(b.Q, b.K, b.V, None, None, L, w.keep).dwt().filter()
+    bare = LibRun(b.Q, b.K, b.V, None, None, L, w.keep, want_sets=False).dwt().filter()
+    torch.cuda.synchronize()
+    assert torch.equal(bare.idx, run.idx)
+    for u in range(w.units):
+        i, h = divmod(u, H)
+        K = f64(b.K[i, h])
+        pyr = oracle.haar_pyramid_spec32(K.astype(np.float32), L, True)
+        mu0, sets = oracle.filter_gqa(f64(b.Q[i, h * group:(h + 1) * group]), pyr, K, n, L, np.array(w.keep),
+                                      want_sets=True)
+        assert np.array_equal(run.idx[u].cpu().numpy(), mu0), f"unit {u}"
+        got = run.level_sets(u)
+        for lev in range(L, -1, -1):
+            assert np.array_equal(got[lev], sets[lev]), f"unit {u} scale {lev}"
