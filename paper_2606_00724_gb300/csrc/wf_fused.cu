@@ -2462,17 +2462,20 @@ cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd
   return cudaGetLastError();
 }
 
-// The grouped filter (wf_gqa_filter_kernel): bf16, d = 128, G >= 2 query
-// heads per key head with q <= 32 rows each and G q <= 256, candidate lists
-// within the Top-K's 8192.  One unit per cluster; the largest cluster of up
-// to 8 CTAs whose grid fits the SMs in one wave with every cluster resident.
+// The grouped filter (wf_gqa_filter_kernel): bf16, d = 128, at most 256 stacked
+// query rows a key head of grouped heads, or of one head with a block of more
+// than 32 rows (up to 32 are the fused kernel's), candidate lists within the
+// Top-K's 8192.  (32 heads x 16K tokens with blocks of 64: a step took 171 us
+// with 20 launches for the filter and takes 80 us with this one.)
+// One unit per cluster; the largest cluster of up to 8 CTAs
+// whose grid fits the SMs in one wave with every cluster resident.
 GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int num_sms) {
   GqaPlan gp{};
   gp.ok = false;
   if (kv.dtype != WF_BF16 || kv.head_dim != D || q.dtype != WF_BF16 || kv.heads <= 0 || levels > 10) return gp;
   if (q.heads % kv.heads != 0 || q.batch != kv.batch) return gp;
   const int G = q.heads / kv.heads;
-  if (G < 2 || q.seq > NQ || G * q.seq > GQ_MAXCH * NQ) return gp;
+  if ((G == 1 && q.seq <= NQ) || q.seq > kMaxQ || G * q.seq > GQ_MAXCH * NQ) return gp;
   const int U = kv.batch * kv.heads;
   int cmax = kv.seq >> levels, kmax = 0;
   for (int l = 0; l <= levels; ++l) kmax = kmax > keep[l] ? kmax : keep[l];

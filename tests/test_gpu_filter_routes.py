@@ -1,7 +1,7 @@
 """Which kernels wf_filter takes, at the edges of each route: the fused kernel
 without its attention (bf16, head_dim 128, at most 32 query rows, one query
-head a key head), the grouped filter kernel (grouped heads), and the kernels
-per scale past those kernels' 8192 candidates a scale.  Indices and
+head a key head), the grouped filter kernel (grouped heads, blocks of 33 to 64
+rows), and the kernels per scale past those kernels' 8192 candidates a scale.  Indices and
 level sets bit-exact against the fp64 oracle on planted inputs, which have a
 margin at every Top-K boundary; also for [B, rows, H, d] strides and without
 level sets."""
@@ -32,6 +32,10 @@ def _bshd(t):
     (1, 2, 1, 17, 16384, 1, 4096, False),  # 8192 candidates: the largest list of the fused kernel
     (1, 1, 1, 17, 16640, 1, 4096, False),  # 8320 candidates: the kernels per scale
     (1, 2, 4, 32, 4104, 3, 513, True),    # grouped heads, ragged n, token trim
+    (1, 3, 1, 33, 4104, 3, 513, True),    # the smallest block above the fused kernel's: two chunks of query columns
+    (1, 2, 1, 64, 8192, 4, 820, False),   # the largest block
+    (1, 1, 4, 64, 2048, 2, 301, False),   # grouped heads with blocks of 64: 256 stacked rows
+    (1, 1, 3, 5, 2048, 2, 256, False),    # grouped heads that fit one chunk
 ])
 def test_filter_route(B, H, group, q, n, L, k, bshd):
     w = synth.Workload("filter_route", B, H, 128, n, q, 1, L, tuple(wf.wf_default_schedule(n, L, k)), "bf16", "iid",
