@@ -175,7 +175,7 @@ wf_status wf_level0_schedule(int64_t n, int levels, int64_t k, int32_t* keep);
  * Outputs: idx int32 [B*H][keep[0]] token positions, ascending per unit.
  * level_sets (optional, NULL to skip): int32
  * [B*H][keep[L] + .. + keep[1] + keep[0]] = J_L, .., J_1, mu^0 per unit.
- * For bf16 keys with head_dim 128 the whole filter is one launch of wf_step's
+ * For bf16 keys the whole filter is one launch of wf_step's
  * fused kernel without its attention (one query head per key head) or of its
  * grouped filter kernel, within those kernels' limits (see wf_step); other
  * shapes run three kernels a scale.
@@ -307,12 +307,12 @@ wf_status wf_noalloc_status(void* stream);
  * NULL) and O exactly as wf_filter + wf_sparse_attn define them.  Same
  * arguments and rules as those calls; ws must hold wf_step_workspace_bytes().
  *
- * For bf16 with head_dim 128, at most 32 query rows and one query head per
+ * For bf16 with at most 32 query rows and one query head per
  * key head, the filter and the attention run as one fused kernel (one
  * thread-block cluster per (batch, head)).  Grouped query heads and blocks of
- * 33 to 64 rows with bf16, head_dim 128 and at most 256 stacked rows a key
+ * 33 to 64 rows with bf16 and at most 256 stacked rows a key
  * head run the grouped filter kernel (one cluster per (batch, key head), the
- * stacked rows as the MMA columns), then the tensor-core attention.
+ * stacked rows as the MMA columns), then the attention of wf_sparse_attn.
  * Other shapes run the per-stage kernels.  The fused kernels' waits
  * (on copies, tensor-core completion and the cluster's exchanges) are
  * bounded: if one gives up (it never should), the kernel returns early,
@@ -338,7 +338,7 @@ wf_status wf_step(const void* Q, const wf_tensor* q, const void* K, const void* 
  * for wf_step; ws: at least wf_step_wavelet_workspace_bytes() bytes, 256-byte
  * aligned, with the status word of wf_step in its first 4 bytes.
  *
- * For bf16 with head_dim 128, at most 32 query rows and one query head per
+ * For bf16 with at most 32 query rows and one query head per
  * key head, every scale runs on wf_step's fused kernel: one launch per scale,
  * after the transform of that scale's candidate blocks, with the previous
  * selection handed over in ws; the last launch also runs the attention.

@@ -403,7 +403,7 @@ WF_API wf_status wf_step(const void* Q, const wf_tensor* q, const void* K, const
   const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, n_g, sms);
   if (fp.ok && q->heads == kv->heads) {
     e = wf::launch_fused(fp, Q, *q, K, V, *kv, Kg, Vg, n_g > 0 ? g : nullptr, coeffs, levels, keep, idx,
-                         level_sets, O, *o, status, s);
+                         level_sets, O, *o, status, s, nullptr);
     return cuda_status(e);
   }
   // Otherwise the filter (wf_filter's kernels), then the per-stage attention.

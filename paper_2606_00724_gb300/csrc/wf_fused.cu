@@ -47,12 +47,25 @@
 #include "wf_internal.cuh"
 #include "wf_sm100.cuh"
 
+// The file is compiled once per head_dim (wf_fused_d64.cu defines 64 and
+// includes it); the entry points live in a namespace of that head_dim.
+#ifndef WF_HEAD_DIM
+#define WF_HEAD_DIM 128
+#endif
+#if WF_HEAD_DIM == 128
+#define WF_HD hd128
+#else
+#define WF_HD hd64
+#endif
+
 namespace wf {
+namespace WF_HD {
 namespace {
 
 using namespace sm100;
 
-constexpr int D = 128;                     // head_dim
+constexpr int D = WF_HEAD_DIM;             // head_dim
+static_assert(D == 64 || D == 128, "a row is one or two 128-byte swizzle rows");
 constexpr int TM = 128;                    // rows per MMA tile (M)
 constexpr int NQ = 32;                     // query rows per MMA (N), zero padded
 constexpr int MAXP = 2;                    // units per cluster
@@ -65,10 +78,19 @@ constexpr int P0 = 32 * (MMA_WARP + 1);    // first producer thread
 constexpr int NT = 32 * (MMA_WARP + 1 + NPW);  // threads per CTA
 constexpr int MAXCS = 8;                   // CTAs per cluster
 constexpr int HALF_BYTES = TM * 128;       // one 64-column half of a tile, 128-byte rows
-constexpr int TILE_BYTES = 2 * HALF_BYTES;
+constexpr int HALVES = D / 64;               // 128-byte halves of a row
+constexpr int TILE_BYTES = HALVES * HALF_BYTES;
+// Ring stages: as many bytes for either head_dim.
+constexpr int MAXS = 4 * 128 / D;          // most stages of an instance
 constexpr int QGRP = (D / 8) * 128;        // bytes per 8-row group of a query tile (core matrices)
 constexpr int Q_BYTES = NQ * D * 2;
-constexpr int P_BYTES = NQ * TM * 2;
+// The attention's P = 2^(s - m) is the bf16 operand of the PV product.  For
+// head_dim 128 P is rounded to bf16.  For head_dim 64 P keeps its 24 bits, as
+// three bf16 terms (each the rounding of what the terms before it leave) that
+// multiply V one after the other into the same fp32 accumulator.
+constexpr int PTERMS = D == 64 ? 3 : 1;
+constexpr int PT_BYTES = NQ * TM * 2;      // one term of one P tile
+constexpr int P_BYTES = PTERMS * PT_BYTES;
 constexpr int MAXCS_PAD_BYTES = 8 * NQ * 4;  // the ragged head-dim slices of a cluster of up to 8 CTAs
 // A unit's P double buffer; also its Top-K scratch and its combine buffer
 // (the partial O rows of this CTA's head-dim slice from every cluster CTA:
@@ -80,7 +102,10 @@ constexpr uint32_t kCsyncId = 1;           // named barriers 1, 2: the compute w
 constexpr uint32_t kSetupSyncId = 3;       // named barrier 3: the set-up threads (all but the producers)
 
 constexpr uint32_t kIdescScore = idesc_bf16(TM, NQ, 0, 0);  // A = rows (K-major), B = Q (K-major)
-constexpr uint32_t kIdescPV = idesc_bf16(D, NQ, 1, 1);      // A = V^T (MN-major), B = P^T (MN-major)
+// A = V^T (MN-major), B = P^T (MN-major).  M is 128 for head_dim 64 too: the
+// upper 64 accumulator rows are products of whatever follows the value tile
+// in shared memory (always inside the CTA's allocation) and nothing reads them.
+constexpr uint32_t kIdescPV = idesc_bf16(128, NQ, 1, 1);
 
 constexpr int MAXT = 16;  // TMEM tiles of one unit's region (512 columns / 32)
 
@@ -99,7 +124,7 @@ struct UnitState {
 };
 
 struct Misc {
-  unsigned long long full[4], empty[4];
+  unsigned long long full[MAXS], empty[MAXS];
   unsigned long long mdone[MAXP], jready[MAXP], xbar[MAXP], kbar[MAXP];
   unsigned long long tdone[MAXP][MAXT];  // scale tile t of a unit scored (one phase per scale)
   unsigned long long pfull[MAXP][2], pempty[MAXP][2], cbar[MAXP], cready[MAXP];
@@ -386,34 +411,35 @@ __host__ __device__ constexpr int topk_run(int m) {
 // Producer warps.
 // ---------------------------------------------------------------------------
 
-// This producer thread's share of one 128-row tile: 16-byte chunk c = pt % 16
-// of rows r0 + RSTEP j (r0 = pt / 16, j < RROWS), written in the
+// This producer thread's share of one 128-row tile: 16-byte chunk c = pt % LPR
+// of rows r0 + RSTEP j (r0 = pt / LPR, j < RROWS), written in the
 // 128-byte-swizzled K-major layout (row r, chunk c at half c/8, byte
-// r*128 + ((c%8) ^ (r%8))*16).  The 16 lanes of a half-warp copy the same
-// rows, so each lane forms one row's index or address per 16 rows and the
-// half-warp shares them by shuffles.  The swizzle term of a thread's rows
-// repeats every 4 rows (RSTEP j mod 8 takes 4 values), so each destination
-// is one add.
-constexpr int RSTEP = NPT / 16;
+// r*128 + ((c%8) ^ (r%8))*16).  The LPR lanes of a row's chunks copy the same
+// rows, so each lane forms one row's index or address per LPR rows and they
+// share them by shuffles.  The swizzle term of a thread's rows repeats every
+// 4 rows (RSTEP j mod 8 takes at most 4 values), so each destination is one
+// add.
+constexpr int LPR = D / 8;                       // lanes (16-byte chunks) a row
+constexpr int RSTEP = NPT / LPR;
 constexpr int RROWS = (TM + RSTEP - 1) / RSTEP;  // most rows of one thread
-static_assert(RSTEP == 6 && RROWS == 22, "the row schedule below assumes 6 rows a step");
+static_assert(RSTEP % 2 == 0 && RROWS <= 2 * LPR, "4 swizzle terms and two resolved rows a lane cover a thread's rows");
 template <int KIND>
 __device__ __forceinline__ void load_share(uint32_t st, int t, const RowSrc& src, int pt) {
-  const int c = pt & 15, r0 = pt >> 4, half = pt & 16;
+  const int c = pt & (LPR - 1), r0 = pt / LPR, grp = pt & (32 - LPR);
   const uint32_t dbase = st + ((c >> 3) << 14) + (uint32_t)r0 * 128u;
   uint32_t xr[4];
 #pragma unroll
   for (int m = 0; m < 4; ++m) xr[m] = (uint32_t)((c ^ (r0 + RSTEP * m)) & 7) << 4;
-  // Rows j = c and j = 16 + c of this half-warp (clamped into the tile).
-  const int ra = t * TM + r0 + RSTEP * c;
-  const int rb = t * TM + min(r0 + RSTEP * min(16 + c, RROWS - 1), TM - 1);
+  // Rows j = c and j = LPR + c of these lanes (clamped into the tile).
+  const int ra = t * TM + min(r0 + RSTEP * min(c, RROWS - 1), TM - 1);
+  const int rb = t * TM + min(r0 + RSTEP * min(LPR + c, RROWS - 1), TM - 1);
   if (KIND <= 1) {
     const char* cb = reinterpret_cast<const char*>(src.base) + c * 16;
     const uint32_t sb = (uint32_t)src.stride * 2u;  // row stride in bytes
     const uint32_t ia = row_index<KIND>(src, ra), ib = row_index<KIND>(src, rb);
 #pragma unroll
     for (int j = 0; j < RROWS; ++j) {
-      const uint32_t idx = __shfl_sync(0xffffffffu, j < 16 ? ia : ib, half | (j & 15));
+      const uint32_t idx = __shfl_sync(0xffffffffu, j < LPR ? ia : ib, grp | (j & (LPR - 1)));
       if (RSTEP * j + RSTEP - 1 < TM || r0 + RSTEP * j < TM)
         cp_async16(dbase + 128u * RSTEP * j + xr[j & 3], cb + (size_t)idx * sb);
     }
@@ -422,7 +448,7 @@ __device__ __forceinline__ void load_share(uint32_t st, int t, const RowSrc& src
     const unsigned long long pb = reinterpret_cast<unsigned long long>(row_ptr<KIND>(src, rb));
 #pragma unroll
     for (int j = 0; j < RROWS; ++j) {
-      const unsigned long long ak = __shfl_sync(0xffffffffu, j < 16 ? pa : pb, half | (j & 15));
+      const unsigned long long ak = __shfl_sync(0xffffffffu, j < LPR ? pa : pb, grp | (j & (LPR - 1)));
       if (RSTEP * j + RSTEP - 1 < TM || r0 + RSTEP * j < TM)
         cp_async16(dbase + 128u * RSTEP * j + xr[j & 3], reinterpret_cast<const bf16*>(ak) + c * 8);
     }
@@ -463,7 +489,7 @@ __device__ void producer_role(const Ctx& c, const FusedParams& p) {
     const bf16* qb = p.Q + (int64_t)(u / p.H) * p.qsb + (int64_t)(u % p.H) * p.qsh;
     const uint32_t sq = smem_u32(c.smem + c.ly.q + pp * Q_BYTES);
     for (int e = pt; e < NQ * (D / 8); e += NPT) {
-      const int rr = e & 7, ch = (e >> 3) & (D / 8 - 1), g = e >> 7;
+      const int rr = e & 7, ch = (e >> 3) & (D / 8 - 1), g = e / D;
       const int i = g * 8 + rr;
       cp_async16_zfill(sq + (uint32_t)(g * QGRP + ch * 128 + rr * 16), qb + (int64_t)min(i, p.q - 1) * p.qss + ch * 8,
                        i < p.q);
@@ -520,7 +546,7 @@ __device__ __forceinline__ void mma_score_tile(const Ctx& c, const FusedParams& 
     tc_fence_after();
     const uint32_t st = smem_u32(c.smem) + s * TILE_BYTES;
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int h = 0; h < HALVES; ++h)
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
         mma_bf16(dcol, smem_desc_sw128(st + h * HALF_BYTES + kk * 32, 16, 1024),
@@ -546,8 +572,11 @@ __device__ __forceinline__ void mma_pv_tile(const Ctx& c, const FusedParams& p, 
     const uint32_t st = smem_u32(c.smem) + s * TILE_BYTES;
 #pragma unroll
     for (int kq = 0; kq < TM / 16; ++kq)
-      mma_bf16(ocol, smem_desc_sw128(st + kq * 2048, HALF_BYTES, 1024),
-               smem_desc(pa + pb * P_BYTES + kq * 1024, 512, 128), kIdescPV, (t > 0 || kq > 0) ? 1u : 0u);
+#pragma unroll
+      for (int e = 0; e < PTERMS; ++e)
+        mma_bf16(ocol, smem_desc_sw128(st + kq * 2048, HALF_BYTES, 1024),
+                 smem_desc(pa + pb * P_BYTES + e * PT_BYTES + kq * 1024, 512, 128), kIdescPV,
+                 (t > 0 || kq > 0 || e > 0) ? 1u : 0u);
   }
   mma_commit(bar_addr(ms.empty[s]));
   mma_commit(bar_addr(ms.pempty[pp][pb]));
@@ -1370,24 +1399,55 @@ __device__ __noinline__ void attn_online(Misc& ms, int* status, float sl2, uint8
         if (lane == 0) wait_or_abort(bar_addr(ms.pempty[pp][pb]), (pn - 1) & 1u, ms, status);
         __syncwarp();
       }
-      uint32_t w[16];
-      if (valid) {
+      // P^T, MN-major core matrices: key group r / 8, query chunk ch.  Rows
+      // past the slice: P = 0.
+      uint8_t* dst = pbase + pb * P_BYTES + (row >> 3) * 512 + (row & 7) * 16;
+      if (PTERMS == 1) {
+        uint32_t w[16];
+        if (valid) {
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const float2 x = up2(fma2(pk2(__uint_as_float(ra[2 * k]), __uint_as_float(ra[2 * k + 1])), s2, nml[k]));
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(ex2(x.x), ex2(x.y));
+            lsum2[k] = add2(lsum2[k], pk2(__low2float(h2), __high2float(h2)));
+            w[k] = *reinterpret_cast<const uint32_t*>(&h2);
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 16; ++k) w[k] = 0u;
+        }
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch)
+          *reinterpret_cast<uint4*>(dst + ch * 128) =
+              make_uint4(w[4 * ch], w[4 * ch + 1], w[4 * ch + 2], w[4 * ch + 3]);
+      } else {
+        // The exponentials take the logits' registers; each term is stored
+        // and taken off what is left.
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
           const float2 x = up2(fma2(pk2(__uint_as_float(ra[2 * k]), __uint_as_float(ra[2 * k + 1])), s2, nml[k]));
-          const __nv_bfloat162 h2 = __floats2bfloat162_rn(ex2(x.x), ex2(x.y));
-          lsum2[k] = add2(lsum2[k], pk2(__low2float(h2), __high2float(h2)));
-          w[k] = *reinterpret_cast<const uint32_t*>(&h2);
+          const float e0 = valid ? ex2(x.x) : 0.f, e1 = valid ? ex2(x.y) : 0.f;
+          lsum2[k] = add2(lsum2[k], pk2(e0, e1));
+          ra[2 * k] = __float_as_uint(e0);
+          ra[2 * k + 1] = __float_as_uint(e1);
         }
-      } else {
 #pragma unroll
-        for (int k = 0; k < 16; ++k) w[k] = 0u;  // rows past the slice: P = 0
+        for (int e = 0; e < PTERMS; ++e)
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch) {
+            uint32_t w[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const int i = 8 * ch + 2 * k;
+              const __nv_bfloat162 h2 =
+                  __floats2bfloat162_rn(__uint_as_float(ra[i]), __uint_as_float(ra[i + 1]));
+              ra[i] = __float_as_uint(__uint_as_float(ra[i]) - __low2float(h2));
+              ra[i + 1] = __float_as_uint(__uint_as_float(ra[i + 1]) - __high2float(h2));
+              w[k] = *reinterpret_cast<const uint32_t*>(&h2);
+            }
+            *reinterpret_cast<uint4*>(dst + e * PT_BYTES + ch * 128) = make_uint4(w[0], w[1], w[2], w[3]);
+          }
       }
-      // P^T, MN-major core matrices: key group r / 8, query chunk ch.
-      uint8_t* dst = pbase + pb * P_BYTES + (row >> 3) * 512 + (row & 7) * 16;
-#pragma unroll
-      for (int ch = 0; ch < 4; ++ch)
-        *reinterpret_cast<uint4*>(dst + ch * 128) = make_uint4(w[4 * ch], w[4 * ch + 1], w[4 * ch + 2], w[4 * ch + 3]);
       fence_proxy_async();
       tc_fence_before();
       __syncwarp();
@@ -1437,7 +1497,7 @@ __device__ __noinline__ void attn_combine(Misc& ms, const FusedParams& p, uint32
   const uint32_t comb_a = smem_u32(comb);
   const uint32_t cbar = bar_addr(ms.cbar[pp]);
   const bool send = !aborted(ms);  // every owner has announced its buffers free
-  if (send) {
+  if (send && tid < D) {
     // Owner of head-dim row d = tid, and the row's place in its buffer.
     int owner = tid * (int)cs / D;
     while (owner + 1 < (int)cs && dlo(owner + 1, cs) <= tid) ++owner;
@@ -1486,22 +1546,21 @@ __device__ __noinline__ void attn_combine(Misc& ms, const FusedParams& p, uint32
       if (r < (int)cs) n = fmaf(lds_f32(comb_a + 4u * (uint32_t)((r * rows + dl) * NQ + qi)), f[r], n);
     return n * inv;
   };
-  // A slice of 32, 64 or 128 rows (clusters of 4, 2, 1): warp w writes rows
-  // [w rows / 4, (w + 1) rows / 4) of its query, 16 bytes a store; otherwise
-  // one element a store.
-  const bool vec = rows % (NCW * 8) == 0 && d0 % 8 == 0 && p.oss % 8 == 0 &&
-                   (reinterpret_cast<uintptr_t>(ob) & 15) == 0;
+  // A slice of a multiple of 8 rows (clusters of a power of two): warp w
+  // writes its quarter of the 8-row pieces of its query, 16 bytes a store;
+  // otherwise one element a store.
+  const bool vec = rows % 8 == 0 && d0 % 8 == 0 && p.oss % 8 == 0 && (reinterpret_cast<uintptr_t>(ob) & 15) == 0;
   if (qi < p.q && vec) {
-    const int per = rows / NCW, db = warp * per;
+    const int np8 = rows / 8;
 #pragma unroll 1
-    for (int c0 = 0; c0 < per; c0 += 8) {
+    for (int c0 = 8 * (warp * np8 / NCW); c0 < 8 * ((warp + 1) * np8 / NCW); c0 += 8) {
       uint32_t w4[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(out(db + c0 + 2 * e), out(db + c0 + 2 * e + 1));
+        const __nv_bfloat162 h = __floats2bfloat162_rn(out(c0 + 2 * e), out(c0 + 2 * e + 1));
         w4[e] = *reinterpret_cast<const uint32_t*>(&h);
       }
-      *reinterpret_cast<uint4*>(ob + (int64_t)qi * p.oss + d0 + db + c0) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+      *reinterpret_cast<uint4*>(ob + (int64_t)qi * p.oss + d0 + c0) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
     }
   } else if (qi < p.q) {
 #pragma unroll 1
@@ -1823,7 +1882,7 @@ __device__ void gqa_producer_role(const Ctx& c, const FusedParams& p) {
   for (int ch = 0; ch < p.nch; ++ch) {
     const uint32_t sq = smem_u32(c.smem + c.ly.q + ch * Q_BYTES);
     for (int e = pt; e < NQ * (D / 8); e += NPT) {
-      const int rr = e & 7, c16 = (e >> 3) & (D / 8 - 1), g8 = e >> 7;
+      const int rr = e & 7, c16 = (e >> 3) & (D / 8 - 1), g8 = e / D;
       const int i = ch * NQ + g8 * 8 + rr;
       const int ic = min(i, nq - 1), hd = ic / p.q, r = ic - hd * p.q;
       const bf16* src = p.Q + b * p.qsb + (h * p.G + hd) * p.qsh + (int64_t)r * p.qss + c16 * 8;
@@ -1883,7 +1942,7 @@ __device__ void gqa_mma_role(const Ctx& c, const FusedParams& p) {
         // One MMA per K step over every query chunk at once (N = 32 nch: the
         // chunks' 8-row groups follow each other at the same stride).
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int h = 0; h < HALVES; ++h)
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
             mma_bf16(c.tmem + (uint32_t)r * rcols, smem_desc_sw128(st + h * HALF_BYTES + kk * 32, 16, 1024),
@@ -2231,9 +2290,10 @@ namespace {
 // long candidate lists run the WIDE instance, whose two warpgroups both serve
 // the unit).
 typedef void (*FusedKernel)(FusedParams);
+constexpr int kStagesMin = D == 64 ? 4 : 3;  // (two units' P terms leave head_dim 64 four stages of 16 KB)
 FusedKernel fused_kernel(int stages, bool wide) {
-  if (stages == 4) return wide ? wf_fused_kernel<4, true> : wf_fused_kernel<4, false>;
-  return wide ? wf_fused_kernel<3, true> : wf_fused_kernel<3, false>;
+  if (stages == MAXS) return wide ? wf_fused_kernel<MAXS, true> : wf_fused_kernel<MAXS, false>;
+  return wide ? wf_fused_kernel<kStagesMin, true> : wf_fused_kernel<kStagesMin, false>;
 }
 
 // The kernel's dynamic shared-memory limit, raised once per device and
@@ -2333,9 +2393,9 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
     size_t smem;
   };
   auto choose = [&](int P) {
-    Choice ch{P, 0, 4, 0};
+    Choice ch{P, 0, MAXS, 0};
     const int clusters = (U + P - 1) / P;
-    if (smem_layout(4, P, cmax, kmax).total > kMaxSmem) ch.stages = 3;
+    if (smem_layout(MAXS, P, cmax, kmax).total > kMaxSmem) ch.stages = kStagesMin;
     ch.smem = smem_layout(ch.stages, P, cmax, kmax).total;
     if (ch.smem > kMaxSmem) return ch;
     for (int c = MAXCS; c >= 1 && ch.cs == 0; --c)
@@ -2348,7 +2408,7 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   };
   // Units per SM (P / cs) set each SM's share of the rows: take the smaller,
   // two units per cluster on a tie.
-  const Choice c2 = U >= 2 ? choose(2) : Choice{2, 0, 4, 0};
+  const Choice c2 = U >= 2 ? choose(2) : Choice{2, 0, MAXS, 0};
   const Choice c1 = choose(1);
   Choice best = c2;
   if (c2.cs == 0 || (c1.cs > 0 && 1 * c2.cs < 2 * c1.cs)) best = c1;
@@ -2462,13 +2522,14 @@ cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd
   return cudaGetLastError();
 }
 
-// The grouped filter (wf_gqa_filter_kernel): bf16, d = 128, at most 256 stacked
+// The grouped filter (wf_gqa_filter_kernel): bf16, at most 256 stacked
 // query rows a key head of grouped heads, or of one head with a block of more
 // than 32 rows (up to 32 are the fused kernel's), candidate lists within the
 // Top-K's 8192.  (32 heads x 16K tokens with blocks of 64: a step took 171 us
 // with 20 launches for the filter and takes 80 us with this one.)
 // One unit per cluster; the largest cluster of up to 8 CTAs
 // whose grid fits the SMs in one wave with every cluster resident.
+constexpr int kGqaStages = 3 * 128 / D;
 GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int num_sms) {
   GqaPlan gp{};
   gp.ok = false;
@@ -2482,7 +2543,7 @@ GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int3
   for (int l = 1; l <= levels; ++l) cmax = cmax > 2 * keep[l] ? cmax : 2 * keep[l];
   if (cmax > kMaxCand || kmax > kMaxCand) return gp;
   const int nch = (G * q.seq + NQ - 1) / NQ;
-  constexpr int kStages = 3;
+  constexpr int kStages = kGqaStages;
   const size_t kMaxSmem = 227 * 1024;
   int cs = 0;
   size_t smem = 0;
@@ -2589,10 +2650,10 @@ cudaError_t launch_gqa_filter(const GqaPlan& gp, const void* Q, const wf_tensor&
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaFuncSetAttribute(wf_gqa_filter_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(wf_gqa_filter_kernel<kGqaStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)gp.smem);
   if (e != cudaSuccess) return e;
-  e = cudaLaunchKernelEx(&cfg, wf_gqa_filter_kernel<3>, p);
+  e = cudaLaunchKernelEx(&cfg, wf_gqa_filter_kernel<kGqaStages>, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -2625,7 +2686,7 @@ cudaError_t launch_literal_fused(const FusedPlan& fp, const FilterPlan& fl, cons
     r.jstride = fl.cmax;
     r.lrows = l == L ? top : arows;
     r.lrows_unit = l == L ? (int64_t)m * D : (int64_t)fl.cmax * D;
-    if ((e = launch_fused(fp, Q, qd, K, V, kv, Kg, Vg, g, nullptr, L, fl.keep, idx, level_sets, O, od ? *od : qd,
+    if ((e = WF_HD::launch_fused(fp, Q, qd, K, V, kv, Kg, Vg, g, nullptr, L, fl.keep, idx, level_sets, O, od ? *od : qd,
                           status, s, &r)) != cudaSuccess)
       return e;
     m = 2 * fl.keep[l];
@@ -2636,4 +2697,5 @@ cudaError_t launch_literal_fused(const FusedPlan& fp, const FilterPlan& fl, cons
   return cudaSuccess;
 }
 
+}  // namespace WF_HD
 }  // namespace wf

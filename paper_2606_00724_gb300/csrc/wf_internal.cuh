@@ -134,7 +134,7 @@ cudaError_t launch_tc_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd
                            const wf_tensor* g, float scale, int* status, void* ws, int* nsplit_out,
                            cudaStream_t s);
 
-// Fused step (bf16, head_dim 128, <= 32 query rows): one cluster of cs CTAs
+// Fused step (bf16, <= 32 query rows): one cluster of cs CTAs
 // per P units.
 struct FusedPlan {
   bool ok;
@@ -143,8 +143,6 @@ struct FusedPlan {
   bool trim;
   bool wide;  // one unit per cluster served by both compute warpgroups
 };
-// n_g: generation rows of the attention, or -1 for a plan of the filter alone.
-FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g, int num_sms);
 // Part of the chain in one launch (the literal-basis path runs one launch per
 // scale, with the transform of the candidates' blocks between launches):
 // scales lev_top down to lev_bot; the previous selection J_{lev_top+1} as its
@@ -162,26 +160,14 @@ struct FusedRange {
   const void* lrows;
   int64_t lrows_unit;
 };
-// range == nullptr: the whole step (every scale, mu^0, the attention).
-cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd, const void* K, const void* V,
-                         const wf_tensor& kv, const void* Kg, const void* Vg, const wf_tensor* g,
-                         const void* coeffs, int levels, const int32_t* keep, int32_t* idx, int32_t* level_sets,
-                         void* O, const wf_tensor& od, int* status, cudaStream_t s,
-                         const FusedRange* range = nullptr);
-
-// The literal-basis filter on the fused kernel (bf16, d 128, one query head
+// launch_literal_fused: the literal-basis filter on the fused kernel (bf16, one query head
 // per KV head, a fused plan fp for the same shapes): one launch per scale,
 // each after the transform of its candidates' gathered blocks
 // (launch_wavelet_approx, into the block after the filter plan's workspace);
 // the candidate lists pass between launches in the plan's two candidate
 // buffers.  With O not null the last launch also runs the attention (od its
 // descriptor; Kg/Vg/g the generation rows).
-cudaError_t launch_literal_fused(const FusedPlan& fp, const FilterPlan& fl, const void* Q, const wf_tensor& qd,
-                                 const void* top, const void* K, const void* V, const wf_tensor& kv, const void* Kg,
-                                 const void* Vg, const wf_tensor* g, int wavelet, int32_t* idx, int32_t* level_sets,
-                                 void* O, const wf_tensor* od, void* ws, int* status, cudaStream_t s);
-
-// The grouped-query filter on the fused kernel design (one cluster per
+// plan_gqa, launch_gqa_filter: the grouped-query filter on the fused kernel design (one cluster per
 // (batch, key head); the stacked query rows of the G query heads as MMA
 // columns): mu^0 and the level sets, for the per-stage attention after it.
 struct GqaPlan {
@@ -190,10 +176,63 @@ struct GqaPlan {
   size_t smem;
   bool trim;
 };
-GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int num_sms);
-cudaError_t launch_gqa_filter(const GqaPlan& gp, const void* Q, const wf_tensor& qd, const void* K,
-                              const wf_tensor& kv, const void* coeffs, int levels, const int32_t* keep, int32_t* idx,
-                              int32_t* level_sets, int* status, cudaStream_t s);
+// The entry points, once per head_dim (wf_fused.cu is compiled for each).
+// plan_fused: n_g generation rows of the attention, or -1 for a plan of the
+// filter alone.  launch_fused: range == nullptr is the whole step (every
+// scale, mu^0, the attention).
+#define WF_FUSED_ENTRY_POINTS                                                                                       \
+  FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g,           \
+                       int num_sms);                                                                                \
+  cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd, const void* K, const void* V,   \
+                           const wf_tensor& kv, const void* Kg, const void* Vg, const wf_tensor* g,                 \
+                           const void* coeffs, int levels, const int32_t* keep, int32_t* idx, int32_t* level_sets,  \
+                           void* O, const wf_tensor& od, int* status, cudaStream_t s, const FusedRange* range);     \
+  cudaError_t launch_literal_fused(const FusedPlan& fp, const FilterPlan& fl, const void* Q, const wf_tensor& qd,   \
+                                   const void* top, const void* K, const void* V, const wf_tensor& kv,              \
+                                   const void* Kg, const void* Vg, const wf_tensor* g, int wavelet, int32_t* idx,   \
+                                   int32_t* level_sets, void* O, const wf_tensor* od, void* ws, int* status,        \
+                                   cudaStream_t s);                                                                 \
+  GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int num_sms);          \
+  cudaError_t launch_gqa_filter(const GqaPlan& gp, const void* Q, const wf_tensor& qd, const void* K,               \
+                                const wf_tensor& kv, const void* coeffs, int levels, const int32_t* keep,           \
+                                int32_t* idx, int32_t* level_sets, int* status, cudaStream_t s);
+namespace hd64 {
+WF_FUSED_ENTRY_POINTS
+}
+namespace hd128 {
+WF_FUSED_ENTRY_POINTS
+}
+#undef WF_FUSED_ENTRY_POINTS
+
+inline FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g,
+                            int num_sms) {
+  return (kv.head_dim == 64 ? hd64::plan_fused : hd128::plan_fused)(q, kv, levels, keep, n_g, num_sms);
+}
+inline cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd, const void* K,
+                                const void* V, const wf_tensor& kv, const void* Kg, const void* Vg,
+                                const wf_tensor* g, const void* coeffs, int levels, const int32_t* keep, int32_t* idx,
+                                int32_t* level_sets, void* O, const wf_tensor& od, int* status, cudaStream_t s,
+                                const FusedRange* range) {
+  return (kv.head_dim == 64 ? hd64::launch_fused : hd128::launch_fused)(
+      fp, Q, qd, K, V, kv, Kg, Vg, g, coeffs, levels, keep, idx, level_sets, O, od, status, s, range);
+}
+inline cudaError_t launch_literal_fused(const FusedPlan& fp, const FilterPlan& fl, const void* Q, const wf_tensor& qd,
+                                        const void* top, const void* K, const void* V, const wf_tensor& kv,
+                                        const void* Kg, const void* Vg, const wf_tensor* g, int wavelet, int32_t* idx,
+                                        int32_t* level_sets, void* O, const wf_tensor* od, void* ws, int* status,
+                                        cudaStream_t s) {
+  return (kv.head_dim == 64 ? hd64::launch_literal_fused : hd128::launch_literal_fused)(
+      fp, fl, Q, qd, top, K, V, kv, Kg, Vg, g, wavelet, idx, level_sets, O, od, ws, status, s);
+}
+inline GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int num_sms) {
+  return (kv.head_dim == 64 ? hd64::plan_gqa : hd128::plan_gqa)(q, kv, levels, keep, num_sms);
+}
+inline cudaError_t launch_gqa_filter(const GqaPlan& gp, const void* Q, const wf_tensor& qd, const void* K,
+                                     const wf_tensor& kv, const void* coeffs, int levels, const int32_t* keep,
+                                     int32_t* idx, int32_t* level_sets, int* status, cudaStream_t s) {
+  return (kv.head_dim == 64 ? hd64::launch_gqa_filter : hd128::launch_gqa_filter)(
+      gp, Q, qd, K, kv, coeffs, levels, keep, idx, level_sets, status, s);
+}
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
