@@ -175,10 +175,10 @@ wf_status wf_level0_schedule(int64_t n, int levels, int64_t k, int32_t* keep);
  * Outputs: idx int32 [B*H][keep[0]] token positions, ascending per unit.
  * level_sets (optional, NULL to skip): int32
  * [B*H][keep[L] + .. + keep[1] + keep[0]] = J_L, .., J_1, mu^0 per unit.
- * For bf16 keys the whole filter is one launch of wf_step's
- * fused kernel without its attention (one query head per key head) or of its
- * grouped filter kernel, within those kernels' limits (see wf_step); other
- * shapes run three kernels a scale.
+ * The whole filter is one launch of wf_step's fused kernel without its
+ * attention (one query head per key head) or, for bf16, of its grouped filter
+ * kernel, within those kernels' limits (see wf_step); other shapes run three
+ * kernels a scale.
  * ws: device scratch of at least wf_filter_workspace_bytes() bytes,
  * 256-byte aligned.  Its first 4 bytes are a status word: for bf16 keys with
  * head_dim 128 the scores run on the tensor cores, and a kernel whose bounded
@@ -313,7 +313,10 @@ wf_status wf_noalloc_status(void* stream);
  * 33 to 64 rows with bf16 and at most 256 stacked rows a key
  * head run the grouped filter kernel (one cluster per (batch, key head), the
  * stacked rows as the MMA columns), then the attention of wf_sparse_attn.
- * Other shapes run the per-stage kernels.  The fused kernels' waits
+ * fp32 with one query head per key head runs as one fused kernel in fp32
+ * arithmetic throughout, one cluster per (batch, head).
+ * All three take candidate lists of at most 8192 at every scale.
+ * Other shapes run the per-stage kernels.  The bf16 fused kernels' waits
  * (on copies, tensor-core completion and the cluster's exchanges) are
  * bounded: if one gives up (it never should), the kernel returns early,
  * outputs are undefined, and a status word in the first 4 bytes of ws is set;

@@ -160,6 +160,10 @@ cudaError_t run_filter(const wf::FilterPlan& p, const void* Q, const wf_tensor& 
                               level_sets, nullptr, q, status, s, &r);
     }
   }
+  const wf::F32Plan f32 = wf::plan_f32(q, kv, levels, keep, sms);
+  if (f32.ok)
+    return wf::launch_f32(f32, Q, q, K, nullptr, kv, nullptr, nullptr, nullptr, coeffs, levels, keep, idx, level_sets,
+                          nullptr, q, s);
   const wf::GqaPlan gp = wf::plan_gqa(q, kv, levels, keep, sms);
   if (gp.ok) return wf::launch_gqa_filter(gp, Q, q, K, kv, coeffs, levels, keep, idx, level_sets, status, s);
   return wf::launch_filter(p, Q, q, coeffs, K, kv, idx, level_sets, scratch, status, s);
@@ -406,6 +410,10 @@ WF_API wf_status wf_step(const void* Q, const wf_tensor* q, const void* K, const
                          level_sets, O, *o, status, s, nullptr);
     return cuda_status(e);
   }
+  const wf::F32Plan f32 = wf::plan_f32(*q, *kv, levels, keep, sms);
+  if (f32.ok)
+    return cuda_status(wf::launch_f32(f32, Q, *q, K, V, *kv, Kg, Vg, n_g > 0 ? g : nullptr, coeffs, levels, keep, idx,
+                                      level_sets, O, *o, s));
   // Otherwise the filter (wf_filter's kernels), then the per-stage attention.
   const wf::FilterPlan fl = wf::plan_filter(*q, *kv, levels, keep);
   if ((e = run_filter(fl, Q, *q, coeffs, K, *kv, levels, keep, idx, level_sets, scratch, status, sms, s)) !=

@@ -234,6 +234,19 @@ inline cudaError_t launch_gqa_filter(const GqaPlan& gp, const void* Q, const wf_
       gp, Q, qd, K, kv, coeffs, levels, keep, idx, level_sets, status, s);
 }
 
+// The fp32 step (one query head per key head): one cluster of cs CTAs a unit.
+struct F32Plan {
+  bool ok, trim;
+  int U, cs, nbuf, srow, bufw;
+  size_t smem;
+};
+F32Plan plan_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int num_sms);
+// O == nullptr: the filter alone.
+cudaError_t launch_f32(const F32Plan& fp, const void* Q, const wf_tensor& qd, const void* K, const void* V,
+                       const wf_tensor& kv, const void* Kg, const void* Vg, const wf_tensor* g, const void* coeffs,
+                       int levels, const int32_t* keep, int32_t* idx, int32_t* level_sets, void* O,
+                       const wf_tensor& od, cudaStream_t s);
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // A kernel's dynamic shared-memory limit, raised once per device and kernel

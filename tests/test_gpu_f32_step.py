@@ -1,0 +1,57 @@
+"""The one-launch fp32 step and filter at the edges of its plan: one query
+row, blocks of 33 to 64 rows, ragged lists, clusters of 8 down to 1, one tile
+buffer or two, slices of several tiles, no generation rows, token trim,
+[B, rows, H, d] strides, and the kernels per scale past 8192 candidates.
+Indices and level sets bit-exact against the fp64 oracle on planted inputs,
+outputs within the fp32 bound (max-abs 1e-5)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import LibRun, assert_close_out, f64
+from paper_2606_00724_gb300 import synth, wf
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+
+def _bshd(t):
+    return t.transpose(1, 2).contiguous().transpose(1, 2)
+
+
+@pytest.mark.parametrize("B,H,d,q,n,L,k,ng,bshd", [
+    (1, 3, 64, 1, 2048, 2, 301, 0, False),      # one query row, token trim, no generation rows
+    (1, 1, 128, 32, 64, 3, 8, 5, True),         # fewer rows than CTAs in the cluster
+    (1, 5, 128, 17, 4104, 3, 512, 7, True),     # ragged n, [B, rows, H, d] strides
+    (2, 3, 64, 33, 4104, 3, 513, 32, False),    # the smallest block of the 64-row kernels
+    (1, 2, 128, 64, 8192, 4, 820, 64, False),   # the largest block
+    (2, 40, 64, 32, 2048, 2, 256, 32, False),   # one CTA a cluster: slices of several tiles
+    (3, 50, 128, 32, 2048, 2, 205, 3, False),   # the same with one tile buffer
+    (1, 1, 128, 32, 16384, 1, 4096, 1, False),  # 8192 candidates, the largest list
+    (1, 1, 64, 32, 16640, 1, 4096, 1, False),   # 8320: the kernels per scale
+])
+def test_step_f32(B, H, d, q, n, L, k, ng, bshd):
+    w = synth.Workload("f32", B, H, d, n, q, max(ng, 1), L, tuple(wf.wf_default_schedule(n, L, k)), "f32", "iid")
+    units = [u for u in (0, 1, 7, B * H // 2, B * H - 1) if u < B * H]
+    b = synth.make_batch(w, planted=True, device="cuda", cfg="f32", units=units)
+    if bshd:
+        b = synth.Batch(*(_bshd(t) for t in (b.Q, b.K, b.V, b.Kg, b.Vg)), b.targets)
+    Kg, Vg = (b.Kg, b.Vg) if ng else (None, None)
+    run = LibRun(b.Q, b.K, b.V, Kg, Vg, L, w.keep).dwt().step(refresh=False)
+    filt = LibRun(b.Q, b.K, b.V, Kg, Vg, L, w.keep, want_sets=False).dwt().filter()
+    torch.cuda.synchronize()
+    assert torch.equal(filt.idx, run.idx)
+    for u in units:
+        i, h = divmod(u, H)
+        Q, K, V = f64(b.Q[i, h]), f64(b.K[i, h]), f64(b.V[i, h])
+        kg, vg = (f64(Kg[i, h]), f64(Vg[i, h])) if ng else (None, None)
+        pyr = oracle.haar_pyramid_spec32(K.astype(np.float32), L, False)
+        mu0, sets = oracle.filter(Q, pyr, K, n, L, np.array(w.keep), want_sets=True)
+        got = run.level_sets(u)
+        for lev in range(L, -1, -1):
+            assert np.array_equal(got[lev], sets[lev]), f"unit {u} scale {lev}"
+        assert np.array_equal(run.idx[u].cpu().numpy(), mu0)
+        assert_close_out(f64(run.O[i, h]), oracle.sparse_attn(Q, K, V, mu0, kg, vg), torch.float32)
