@@ -7,7 +7,9 @@
 // analysis is a[j] = sum_k h[k] x[(2j + k) mod len]; b levels give one
 // approximation row per candidate.
 //
-// One CTA computes TO consecutive level-b rows for DS head-dim channels: it
+// Scales 1 to 5 stream the rows through registers (approx_stream_kernel).
+// Deeper ones go through shared memory (approx_kernel):
+// one CTA computes TO consecutive level-b rows for DS head-dim channels: it
 // gathers the TO 2^b input rows plus the (taps - 2)(2^b - 1) rows the filter
 // reaches past them (wrapping around the gathered sequence) into shared
 // memory with 16-byte cp.async copies, and runs the b levels of the cascade
@@ -244,6 +246,224 @@ __global__ void __launch_bounds__(NTH, 3) approx_kernel(const T* __restrict__ K,
   }
 }
 
+// ---------------------------------------------------------------------------
+// Scales 1 to 5: the cascade streamed through registers.
+// ---------------------------------------------------------------------------
+// A thread owns one 16-byte vector of channels and a run of consecutive
+// outputs.  It reads its input rows in order, one candidate block of 2^L rows
+// after the other (the sequence is made of whole blocks, so a block needs one
+// index), and pushes each row through all L levels at once.  Level l keeps of
+// its past inputs only the first half of the next output's sum,
+// fma(h[1], x1, h[0] x0), plus an unpaired input; every output is finished by
+// two more fused multiply-adds, in the order of the storage rule above, so
+// the results are the same bits.  A db2 output reaches 2 (2^L - 1) rows past
+// its own block: a run reads two blocks more than it has outputs (one at
+// L = 1), wrapping around the sequence.
+//
+// What bounds it: HBM.  Nothing goes through shared memory and no barrier
+// separates loading from computing: a thread loads its next 8 rows before it
+// works on the current 8, and the 16 warps an SM holds keep about 64 KB in
+// flight.  (Gathering 128 rows into shared memory, then transforming them
+// level by level between barriers, left DRAM at 44 % at scale 3.)  Measured:
+// the db2 step of 64 units x 32K tokens 233.1 -> 218.1 us; its three
+// transforms read 537 MB in about 84 us of that, 99 us before.  Scales 6 to 10
+// (a long halo, few outputs) keep the shared-memory kernel below.
+template <typename T, int TAPS, int L>
+struct Cascade {
+  static constexpr int VEC = Vec<T>::N;
+  static constexpr float c = 0.70710678118654752440f;  // fl32(1 / sqrt 2)
+  f32x2 h2[4];
+  Lanes<T> half[L + 1];  // an input whose pair is still to come
+  Lanes<T> acc[L + 1];   // h[0] x0 + h[1] x1 of the pair before
+  // Input E of the chunk (2^(L - LV + 1) inputs of level LV a block).  A db2
+  // output needs the pair after its own, so level 1 gives output j - 1 with
+  // pair j: the inputs of level 2 start at an odd index; level 2's shift of
+  // one more makes the later levels even again.
+  template <int LV, int E, typename F>
+  __device__ __forceinline__ void push(const Lanes<T>& x, F&& emit) {
+    constexpr int off = TAPS == 4 && LV == 2 ? 1 : 0;
+    if constexpr (((E + off) & 1) == 0) {
+      half[LV] = x;
+    } else {
+      Lanes<T> y;
+#pragma unroll
+      for (int i = 0; i < VEC / 2; ++i) {
+        if constexpr (TAPS == 2) {
+          // Scalar: the compiler merges a packed product with the next
+          // level's packed sum, which would skip the product's rounding.
+          const float2 a = up2(half[LV].v[i]), b = up2(x.v[i]);
+          y.v[i] = pk2(__fmul_rn(__fadd_rn(a.x, b.x), c), __fmul_rn(__fadd_rn(a.y, b.y), c));
+        } else {
+          y.v[i] = fma2(h2[3], x.v[i], fma2(h2[2], half[LV].v[i], acc[LV].v[i]));
+          acc[LV].v[i] = fma2(h2[1], x.v[i], mul2(h2[0], half[LV].v[i]));
+        }
+      }
+      if constexpr (LV == L) emit(y);
+      else push<LV + 1, (E + off - 1) / 2>(y, emit);
+    }
+  }
+  // Rows E .. E + N - 1 of a block, as loaded.
+  template <int E, int N, typename F>
+  __device__ __forceinline__ void rows(const uint4* w, F&& emit) {
+    if constexpr (N > 0) {
+      Lanes<T> x;
+      widen(*w, x);
+      push<1, E>(x, emit);
+      rows<E + 1, N - 1>(w + 1, emit);
+    }
+  }
+};
+
+constexpr int kStreamThreads = 128;
+constexpr int kStreamMaxLevel = 5;
+
+// CTAs an SM: 128 registers a thread hold the cascade's state up to scale 3;
+// eight db2 channels at scales 4 and 5 need more.
+template <typename T, int TAPS, int L>
+__host__ __device__ constexpr int stream_ctas() {
+  return Vec<T>::N == 8 && TAPS == 4 && L >= 4 ? 3 : 4;
+}
+
+template <typename T, int TAPS, int L, int D>
+__global__ void __launch_bounds__(kStreamThreads, (stream_ctas<T, TAPS, L>()))
+    approx_stream_kernel(const T* __restrict__ K, int64_t ksb, int64_t ksh, int64_t kss, int64_t n, FastDiv heads,
+                         const int32_t* __restrict__ cand, int64_t cand_stride, int m, int run, Taps taps,
+                         T* __restrict__ out, int64_t out_unit) {
+  constexpr int VEC = Vec<T>::N, LPR = D / VEC;    // lanes a row
+  constexpr int DLY = TAPS == 2 ? 0 : (L == 1 ? 1 : 2);  // blocks read before the first output
+  constexpr int RG = 8;                              // rows a load group
+  constexpr int BPG = L < 3 ? RG >> L : 1;           // blocks a group, or
+  constexpr int GPB = L > 3 ? (1 << L) / RG : 1;     // groups a block
+  constexpr int BR = L < 3 ? 1 << L : RG;            // rows of a block in a group
+  grid_dep_wait();  // the candidates (and the output's previous readers) come from the grids before
+  grid_dep_launch();
+  const int u = blockIdx.y;
+  const int t = (int)blockIdx.x * kStreamThreads + (int)threadIdx.x;
+  const int vt = t % LPR, j0 = t / LPR * run;
+  if (j0 >= m) return;
+  const int cnt = min(run, m - j0);  // outputs of this thread
+  const uint32_t bb = fastdiv((uint32_t)u, heads), hh = (uint32_t)u - bb * heads.d;
+  const T* src = K + (int64_t)bb * ksb + (int64_t)hh * ksh + vt * VEC;
+  T* dst = out + (int64_t)u * out_unit + (int64_t)j0 * D + vt * VEC;
+  const int32_t* cd = cand ? cand + (int64_t)u * cand_stride : nullptr;
+  const int blocks = cnt + DLY;
+
+  Cascade<T, TAPS, L> cas;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) cas.h2[k] = pk2(taps.h[k], taps.h[k]);
+#pragma unroll
+  for (int l = 0; l <= L; ++l)
+#pragma unroll
+    for (int i = 0; i < VEC / 2; ++i) cas.half[l].v[i] = cas.acc[l].v[i] = pk2(0.f, 0.f);
+
+  // The block indices of the next group to load, read a group ahead of their
+  // rows.  Block b of the run is position j0 + b of the sequence,
+  // modulo m.
+  int pos = j0;
+  int32_t ci[BPG];
+  auto fetch = [&]() {
+#pragma unroll
+    for (int b = 0; b < BPG; ++b) {
+      ci[b] = cd ? cd[pos] : pos;
+      if (++pos >= m) pos = 0;
+    }
+  };
+  // Load group g: BPG whole blocks, or part g % GPB of a block.  A block's
+  // row step is 0 for an index outside [0, n >> L): every token of the block is
+  // then clamped to the same one.
+  const T* row = src;
+  int64_t step = 0;
+  auto load = [&](int g, uint4 (&w)[RG]) {
+#pragma unroll
+    for (int b = 0; b < BPG; ++b) {
+      if (GPB == 1 || g % GPB == 0) {
+        const int64_t t0 = (int64_t)ci[b] << L;
+        const bool in = t0 >= 0 && t0 < n;
+        row = src + (in ? t0 : (t0 < 0 ? 0 : n - 1)) * kss;
+        step = in ? kss : 0;
+      }
+#pragma unroll
+      for (int i = 0; i < BR; ++i) {
+        w[b * BR + i] = __ldg(reinterpret_cast<const uint4*>(row));
+        row += step;
+      }
+    }
+    if (GPB == 1 || g % GPB == 0) fetch();
+  };
+  int blk = 0;
+  auto emit = [&](const Lanes<T>& y) {
+    const int j = blk - DLY;
+    if (j >= 0 && j < cnt) *reinterpret_cast<uint4*>(dst + (int64_t)j * D) = narrow(y);
+  };
+  const int groups = GPB > 1 ? blocks * GPB : (blocks + BPG - 1) / BPG;
+  uint4 w[2][RG];
+  fetch();
+  load(0, w[0]);
+#pragma unroll 1
+  for (int g = 0; g < groups; g += 2 * GPB) {
+    // Two blocks (GPB > 1) or two groups of blocks a turn, so that the buffers
+    // and the parts of a block have fixed places.
+#pragma unroll
+    for (int h = 0; h < 2 * GPB; ++h) {
+      if (g + h + 1 < groups) load(h + 1, w[(h + 1) & 1]);
+      if (g + h < groups) {
+        if constexpr (GPB == 1) {
+#pragma unroll
+          for (int b = 0; b < BPG; ++b) {
+            cas.template rows<0, BR>(w[h & 1] + b * BR, emit);
+            ++blk;
+          }
+        } else if (GPB == 2) {
+          if (h % 2 == 0) cas.template rows<0, RG>(w[h & 1], emit);
+          else cas.template rows<GPB == 2 ? RG : 0, RG>(w[h & 1], emit);
+          if (h % 2 == 1) ++blk;
+        } else {
+          if (h % 4 == 0) cas.template rows<0, RG>(w[h & 1], emit);
+          else if (h % 4 == 1) cas.template rows<GPB == 4 ? RG : 0, RG>(w[h & 1], emit);
+          else if (h % 4 == 2) cas.template rows<GPB == 4 ? 2 * RG : 0, RG>(w[h & 1], emit);
+          else cas.template rows<GPB == 4 ? 3 * RG : 0, RG>(w[h & 1], emit);
+          if (h % 4 == 3) ++blk;
+        }
+      }
+    }
+  }
+}
+
+// Outputs a thread: as many CTAs as the SMs hold at once, an equal number a
+// unit, so that the runs are long enough to hide the two extra blocks and no
+// partial second wave is left; at least 4.
+inline int stream_run(int64_t units, int m, int lpr, int ctas) {
+  int sms = sm_count();
+  if (sms <= 0) sms = 148;
+  const int64_t per_unit = (int64_t)sms * ctas / units;
+  const int64_t runs = (per_unit < 1 ? 1 : per_unit) * (kStreamThreads / lpr);
+  const int64_t run = (m + runs - 1) / runs;
+  return (int)(run < 4 ? 4 : run);
+}
+
+template <typename T, int TAPS, int L, int D>
+cudaError_t run_stream(const void* K, const wf_tensor& kv, const int32_t* cand, int64_t cand_stride, int m,
+                       const Taps& taps, void* out, int64_t out_unit, cudaStream_t s, bool pdl) {
+  constexpr int LPR = D / Vec<T>::N;
+  const int64_t units = (int64_t)kv.batch * kv.heads;
+  const int run = stream_run(units, m, LPR, stream_ctas<T, TAPS, L>());
+  const int64_t threads = (int64_t)((m + run - 1) / run) * LPR;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)((threads + kStreamThreads - 1) / kStreamThreads), (unsigned)units, 1);
+  cfg.blockDim = dim3(kStreamThreads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, approx_stream_kernel<T, TAPS, L, D>, static_cast<const T*>(K), kv.stride_b,
+                                     kv.stride_h, kv.stride_s, (int64_t)kv.seq, make_fastdiv((uint32_t)kv.heads), cand,
+                                     cand_stride, m, run, taps, static_cast<T*>(out), out_unit);
+  if (e != cudaSuccess) return e;
+  return cudaGetLastError();
+}
+
 // Shared memory of one CTA for DS channels: the raw rows, the first fp32
 // level (the raw buffer holds the later ones) and the row tokens.
 template <typename T, int TAPS>
@@ -291,13 +511,27 @@ cudaError_t run_ds(const void* K, const wf_tensor& kv, const int32_t* cand, int6
   return cudaGetLastError();
 }
 
-// Whole rows of 128 channels per CTA (each row's token resolved once, 256-byte
-// copies of bf16) while the shared memory allows, else 64 channels, else 16
-// (the deepest scales).  Measured at 32K (bf16, db2, three scales a step):
-// whole rows 265 us a step against 301 with 64 channels.
+// Scales above kStreamMaxLevel: whole rows of 128 channels per CTA (each row's
+// token resolved once, 256-byte copies of bf16) while the shared memory
+// allows, else 64 channels, else 16 (the deepest scales).
+template <typename T, int TAPS, int D>
+cudaError_t run_d(const void* K, const wf_tensor& kv, const int32_t* cand, int64_t cand_stride, int m, int level,
+                  const Taps& taps, void* out, int64_t out_unit, cudaStream_t s, bool pdl) {
+  switch (level) {
+    case 1: return run_stream<T, TAPS, 1, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s, pdl);
+    case 2: return run_stream<T, TAPS, 2, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s, pdl);
+    case 3: return run_stream<T, TAPS, 3, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s, pdl);
+    case 4: return run_stream<T, TAPS, 4, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s, pdl);
+    default: return run_stream<T, TAPS, 5, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s, pdl);
+  }
+}
+
 template <typename T, int TAPS>
 cudaError_t run(const void* K, const wf_tensor& kv, const int32_t* cand, int64_t cand_stride, int m, int level,
                 const Taps& taps, void* out, int64_t out_unit, cudaStream_t s, bool pdl) {
+  if (level <= kStreamMaxLevel && kv.batch * kv.heads <= 65535)
+    return kv.head_dim == 64 ? run_d<T, TAPS, 64>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl)
+                             : run_d<T, TAPS, 128>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl);
   if (kv.head_dim == 128 && approx_smem<T, TAPS>(level, 128) <= 200 * 1024)
     return run_ds<T, TAPS, 128>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl);
   if (approx_smem<T, TAPS>(level, 64) <= 200 * 1024)
