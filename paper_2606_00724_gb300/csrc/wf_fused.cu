@@ -127,6 +127,8 @@ struct UnitState {
   float red[NCW][32];
 };
 
+constexpr int MAXREG = 8;  // grouped filter: most TMEM regions of pass 2
+
 struct Misc {
   unsigned long long full[MAXS], empty[MAXS];
   unsigned long long mdone[MAXP], jready[MAXP], xbar[MAXP], kbar[MAXP];
@@ -134,7 +136,8 @@ struct Misc {
   unsigned long long pfull[MAXP][2], pempty[MAXP][2], cbar[MAXP], cready[MAXP];
   UnitState us[MAXP];
   unsigned long long qfull;     // the query blocks have landed (the producers' first copies)
-  unsigned long long rdone[2], rfree[2];  // grouped filter: a TMEM region's logits are ready / read
+  // Grouped filter: pass 1's TMEM buffers and pass 2's regions ready / read.
+  unsigned long long p1done[2], p1free[2], rdone[MAXREG], rfree[MAXREG];
   unsigned long long stallbar;  // completed by nothing (the test-only stalled first wait)
   unsigned long long drainbar;  // the MMA thread's final commit
   long long wait_limit;         // bound of the waits that can give up (cycles)
@@ -1440,24 +1443,44 @@ __global__ void __launch_bounds__(NT, 1) wf_fused_kernel(const __grid_constant__
 // ---------------------------------------------------------------------------
 //
 // One cluster of CS CTAs per (batch, key head) unit, both compute warpgroups
-// on the unit, the same producers and Top-K as the one-head kernel.  The
-// stacked query block (G q rows in chunks of 32) is the N side of the MMAs: a
-// tile's logits take 32 nch TMEM columns, so the CTA holds two tiles at a
-// time (warpgroup w reads region w, the tiles t = w, w + 2, ...), and every
-// scale runs two passes over its rows, the second re-streamed (from L2):
-//   1. per query column, a stabiliser (x sl2) and the sum of exponentials
-//      over the CTA's rows: each tile's exponentials are taken relative to the
-//      largest logit of the query chunk among the warp's rows of that tile
-//      (a column whose terms would all flush to zero takes its own maximum),
-//      and merged as they come, so nothing overflows; the warps' statistics
-//      merge into the CTA's (M, S),
-//      which the cluster exchanges into the normalisers c_i = M + log2 S;
-//   2. each row's ranking key log2 W_j = log2 sum_i 2^(l_ij sl2 - c_i) over
-//      all stacked rows (a running maximum over the chunks keeps tiny sums
-//      exact), all-gathered, then the Top-K (Eq. 9).
+// on the unit, the same producers and Top-K as the one-head kernel.  Every
+// scale runs two passes over the CTA's rows, each with the side of the
+// product on the TMEM lanes that its sums run along, so that both are serial
+// sums of a thread:
+//   1. query rows on the lanes (S = Q rows^T, M tiles of 128 stacked query
+//      rows, 128 candidates a tile): each thread holds one query row's
+//      stabiliser (x sl2, raised when a logit exceeds it by 2^64) and sum of
+//      exponentials over the tile's columns.  Two M tiles: warpgroup w takes M
+//      tile w of every tile; one: the warpgroups take alternate tiles, and a
+//      block of at most 64 rows stands 2 or 4 times in the M tile, so that
+//      every warp has real rows and takes that part of the columns.  The
+//      cluster exchanges the (M, S) into the normalisers c_i = M + log2 S.
+//   2. candidates on the lanes (S^T = rows Q^T, the stacked block's chunks of
+//      32 query rows as 32 nch columns): each thread sums its candidate's
+//      ranking key log2 W_j = log2 sum_i 2^(l_ij sl2 - c_i), all-gathered, then
+//      the Top-K (Eq. 9).  Warpgroup w reads every other TMEM region.  The last
+//      tiles of pass 1 (as many as the ring has stages) stay in shared memory
+//      and are multiplied again from there; only earlier ones are streamed
+//      again.
+// With two M tiles the passes use the same TMEM columns in turn; with one,
+// pass 2 has columns of its own (as many regions as fit), and its products
+// follow pass 1's at once.  (With the candidates on the lanes in both passes,
+// pass 1 needed a warp-wide maximum and a 31-shuffle transpose per 32 x 32
+// logits, about 7 instructions a logit against 2.5: 32 key heads x 32K tokens
+// with 224 stacked rows, 85.3 us a launch against 72.  Each tile's pass 2
+// product issued right behind its pass 1 product delayed the next tile's:
+// 64 stacked rows x 16K, 62 us a launch against 56.)
 // The selection is written as mu^0 (and the level sets); the attention runs
 // afterwards on the per-stage tensor-core kernels.
 constexpr int GQ_MAXCH = 8;  // chunks of 32 stacked query rows (G q <= 256)
+
+// How often the stacked block stands in its M tile (nch <= 2).
+__host__ __device__ constexpr int gqa_copies(int nch) { return nch <= 2 ? 4 / nch : 1; }
+// TMEM regions of pass 2 (an even number: warpgroup w reads regions w, w + 2,
+// ..) and the column of the first: beside pass 1's two buffers of 128 columns
+// (one M tile), or in their place (two).
+__host__ __device__ constexpr int gqa_regions(int nch) { return nch > 4 ? 2 : (256 / (32 * nch)) & ~1; }
+__host__ __device__ constexpr uint32_t gqa_region0(int nch) { return nch > 4 ? 0u : 256u; }
 
 struct GqaLayout {
   uint32_t q, sc, misc, wst, xst, cvec, buf, bufw, total;
@@ -1466,10 +1489,10 @@ __host__ __device__ inline GqaLayout gqa_layout(int stages, int nch, int cs, int
   GqaLayout l;
   const uint32_t nq = 32u * (uint32_t)nch;
   l.q = (uint32_t)stages * TILE_BYTES;
-  l.sc = l.q + (uint32_t)nch * Q_BYTES;                            // Top-K scratch
+  l.sc = l.q + (uint32_t)(nch * gqa_copies(nch)) * Q_BYTES;        // Top-K scratch
   l.misc = (l.sc + (uint32_t)sizeof(SelScratch) + 127u) / 128u * 128u;
-  l.wst = (l.misc + (uint32_t)sizeof(Misc) + 15u) / 16u * 16u;     // [8][nq] float2: each warp's column statistics
-  l.xst = l.wst + 8u * nq * 8u;                                    // [cs][nq] float2: every CTA's (M, S) per column
+  l.wst = (l.misc + (uint32_t)sizeof(Misc) + 15u) / 16u * 16u;     // [256] float2: each thread's statistics (one M tile)
+  l.xst = l.wst + 256u * 8u;                                       // [cs][nq] float2: every CTA's (M, S) per column
   l.cvec = l.xst + (uint32_t)cs * nq * 8u;                         // [nq] float: the normalisers c_i
   l.buf = (l.cvec + nq * 4u + 127u) / 128u * 128u;                 // two key / selection buffers
   l.bufw = (uint32_t)((max(cmax, kmax) + 3) / 4 * 4);
@@ -1494,8 +1517,9 @@ __device__ void gqa_producer_role(const Ctx& c, const FusedParams& p) {
   // rows >= G q zero-filled.
   const int64_t b = c.u0 / p.H, h = c.u0 % p.H;
   const int nq = p.G * p.q;
-  for (int ch = 0; ch < p.nch; ++ch) {
-    const uint32_t sq = smem_u32(c.smem + c.ly.q + ch * Q_BYTES);
+  for (int cc = 0; cc < p.nch * gqa_copies(p.nch); ++cc) {
+    const uint32_t sq = smem_u32(c.smem + c.ly.q + cc * Q_BYTES);
+    const int ch = cc % p.nch;
     for (int e = pt; e < NQ * (D / 8); e += NPT) {
       const int rr = e & 7, c16 = (e >> 3) & (D / 8 - 1), g8 = e / D;
       const int i = ch * NQ + g8 * 8 + rr;
@@ -1514,17 +1538,18 @@ __device__ void gqa_producer_role(const Ctx& c, const FusedParams& p) {
     const RowSrc src = scale_src(c, p, 0, lev, g0, mc);
     produce<S>(ms, p.status, smem_u32(c.smem), it, 0, ntl, src, pt);  // pass 1
     it += ntl;
-    // Pass 2: the same rows again, but for the last two tiles, which stay in
-    // TMEM from pass 1.
-    const int nre = max(ntl - 2, 0);
+    // Pass 2: the same rows again, but for the last tiles, which stay in the
+    // ring from pass 1.
+    const int nre = max(ntl - S, 0);
     produce<S>(ms, p.status, smem_u32(c.smem), it, 0, nre, src, pt);
     it += nre;
   }
   cp_async_wait_all();
 }
 
-// Both passes of every scale: tile t's logits for every query chunk into
-// TMEM region t % 2 once the warpgroup reading that region has released it.
+// Pass 1 of every scale: tile t's logits with the query rows on the lanes
+// into TMEM buffer t % 2 (128 columns an M tile); pass 2: with the candidates
+// on the lanes into region k % 2, the kept tiles first.
 template <int S>
 __device__ void gqa_mma_role(const Ctx& c, const FusedParams& p) {
   Misc& ms = *c.ms;
@@ -1532,53 +1557,98 @@ __device__ void gqa_mma_role(const Ctx& c, const FusedParams& p) {
   wait_or_abort(bar_addr(ms.qfull), 0u, ms, p.status);
   fence_proxy_async();
   const uint32_t sq = smem_u32(c.smem + c.ly.q);
-  const uint32_t rcols = 32u * (uint32_t)p.nch;
-  const uint32_t idesc = idesc_bf16(TM, 32 * p.nch, 0, 0);  // A = rows (K-major), B = the stacked queries (K-major)
-  uint32_t used[2] = {0u, 0u};
+  const int nmt = (p.nch + 3) / 4;                // M tiles of 128 query rows
+  const uint32_t rcols = 32u * (uint32_t)p.nch;   // columns of a pass 2 region
+  const uint32_t bcols = 128u * (uint32_t)nmt;    // columns of a pass 1 buffer
+  const int nreg = gqa_regions(p.nch);
+  const uint32_t tm2 = c.tmem + gqa_region0(p.nch);
+  const bool shared = nmt > 1;                    // the passes share their columns
+  const uint32_t idesc1 = idesc_bf16(TM, TM, 0, 0);          // A = query rows, B = candidate rows (both K-major)
+  const uint32_t idesc2 = idesc_bf16(TM, 32 * p.nch, 0, 0);  // A = candidate rows, B = the stacked queries
+  uint32_t used1 = 0, used2 = 0;  // pass 1 buffers and pass 2 regions filled so far: use i takes buffer i % 2, region i % nreg
+  // Buffer use % ring has been read since its use before.
+  auto wait_free = [&](const unsigned long long* bar, uint32_t use, uint32_t ring) {
+    if (use >= ring) wait_or_abort(bar_addr(bar[use % ring]), (use / ring - 1u) & 1u, ms, p.status);
+  };
+  // Pass 2's product of the tile in ring slot `slot` into the next region.
+  auto pass2 = [&](int slot) {
+    const int s = slot % S, r = (int)(used2 % (uint32_t)nreg);
+    wait_free(ms.rfree, used2, (uint32_t)nreg);
+    ++used2;
+    wait_or_abort(bar_addr(ms.full[s]), (uint32_t)(slot / S) & 1u, ms, p.status);
+    fence_proxy_async();
+    if (!aborted(ms)) {
+      tc_fence_after();
+      const uint32_t st = smem_u32(c.smem) + s * TILE_BYTES;
+      // One MMA per K step over every query chunk at once (N = 32 nch: the
+      // chunks' 8-row groups follow each other at the same stride).
+#pragma unroll
+      for (int h = 0; h < HALVES; ++h)
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          mma_bf16(tm2 + (uint32_t)r * rcols, smem_desc_sw128(st + h * HALF_BYTES + kk * 32, 16, 1024),
+                   smem_desc(sq + (4 * h + kk) * 256, 128, QGRP), idesc2, (h | kk) != 0);
+    }
+    mma_commit(bar_addr(ms.empty[s]));
+    mma_commit(bar_addr(ms.rdone[r]));
+  };
+  // Every read of the last `ring` uses is done.
+  auto wait_all_free = [&](const unsigned long long* bar, uint32_t used, uint32_t ring) {
+    for (uint32_t i = used < ring ? 0u : used - ring; i < used; ++i)
+      wait_or_abort(bar_addr(bar[i % ring]), (i / ring) & 1u, ms, p.status);
+  };
   int it = 0;
   for (int lev = c.lev_top; lev >= c.lev_end; --lev) {
     int g0, mc;
     scale_slice(m_total(p, lev), c.rank, c.cs, g0, mc);
-    const int ntl = tiles_of(mc);
-    // Pass 1: every tile; pass 2: all but the last two, whose logits are
-    // still in their regions (each issue into a region is released once by
-    // the warpgroup reading it, the kept tiles after their second reading).
-    const int nre = max(ntl - 2, 0);
+    const int ntl = tiles_of(mc), nkeep = min(ntl, S), nre = ntl - nkeep;
+    // Shared columns change hands between the passes: every read of the other
+    // pass is done first.
+    if (shared) wait_all_free(ms.rfree, used2, (uint32_t)nreg);
 #pragma unroll 1
-    for (int k = 0; k < ntl + nre; ++k) {
-      const int t = k < ntl ? k : k - ntl, r = t & 1, slot = it + k, s = slot % S;
-      if (used[r] > 0) wait_or_abort(bar_addr(ms.rfree[r]), (used[r] - 1u) & 1u, ms, p.status);
-      ++used[r];
+    for (int t = 0; t < ntl; ++t) {
+      const int r = (int)(used1 & 1u), slot = it + t, s = slot % S;
+      wait_free(ms.p1free, used1, 2u);
+      ++used1;
       wait_or_abort(bar_addr(ms.full[s]), (uint32_t)(slot / S) & 1u, ms, p.status);
       fence_proxy_async();
       if (!aborted(ms)) {
         tc_fence_after();
         const uint32_t st = smem_u32(c.smem) + s * TILE_BYTES;
-        // One MMA per K step over every query chunk at once (N = 32 nch: the
-        // chunks' 8-row groups follow each other at the same stride).
+        // Query rows past the stacked block (up to the M tile's 128) are
+        // whatever follows it in shared memory; nothing reads their rows.
+#pragma unroll 1
+        for (int m = 0; m < nmt; ++m)
 #pragma unroll
-        for (int h = 0; h < HALVES; ++h)
+          for (int h = 0; h < HALVES; ++h)
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            mma_bf16(c.tmem + (uint32_t)r * rcols, smem_desc_sw128(st + h * HALF_BYTES + kk * 32, 16, 1024),
-                     smem_desc(sq + (4 * h + kk) * 256, 128, QGRP), idesc, (h | kk) != 0);
+            for (int kk = 0; kk < 4; ++kk)
+              mma_bf16(c.tmem + (uint32_t)r * bcols + 128u * (uint32_t)m,
+                       smem_desc(sq + (uint32_t)m * 16u * QGRP + (4 * h + kk) * 256, 128, QGRP),
+                       smem_desc_sw128(st + h * HALF_BYTES + kk * 32, 16, 1024), idesc1, (h | kk) != 0);
       }
-      mma_commit(bar_addr(ms.empty[s]));
-      mma_commit(bar_addr(ms.rdone[r]));
+      if (t < nre) mma_commit(bar_addr(ms.empty[s]));
+      mma_commit(bar_addr(ms.p1done[r]));
     }
+    if (shared) wait_all_free(ms.p1free, used1, 2u);
+    // The kept tiles (slots it + nre ..), then the streamed ones (it + ntl ..).
+#pragma unroll 1
+    for (int k = 0; k < ntl; ++k) pass2(k < nkeep ? it + nre + k : it + ntl + k - nkeep);
     it += ntl + nre;
   }
   mma_commit(bar_addr(ms.drainbar));
   (void)mbar_wait_bounded(bar_addr(ms.drainbar), 0u, kDefaultWaitLimit);
 }
 
+template <int S>
 __device__ void gqa_compute_role(const Ctx& c, const FusedParams& p, const GqaLayout gl) {
   Misc& ms = *c.ms;
   constexpr int TN = 32 * unit_warps<true>();
   const int tid = ctid<true>(), lane = tid & 31, warp = tid >> 5, wg = tid >> 7, qd = warp & 3, row = tid & (TM - 1);
   const uint32_t lane_base = (uint32_t)(qd * 32) << 16;
   const int nch = p.nch, nqp = 32 * nch, nq = p.G * p.q;
-  const uint32_t treg = c.tmem + (uint32_t)wg * 32u * (uint32_t)nch;  // this warpgroup's TMEM region
+  const uint32_t nreg = (uint32_t)gqa_regions(nch);
+  uint32_t treg = 0;   // the TMEM region that pass 2 reads
   const uint32_t sc_a = smem_u32(c.smem + gl.sc);
   float2* wst = reinterpret_cast<float2*>(c.smem + gl.wst);
   float2* xst = reinterpret_cast<float2*>(c.smem + gl.xst);
@@ -1587,7 +1657,10 @@ __device__ void gqa_compute_role(const Ctx& c, const FusedParams& p, const GqaLa
   const float sl2 = p.scale_log2;
   const int u = c.u0;
   int64_t sets_off = 0;
-  uint32_t dpar = 0;  // parity of the next phase of this warpgroup's rdone barrier
+  uint32_t used = 0;   // tiles of the scales before: the uses of pass 1's buffers and of pass 2's regions
+  const bool two = nch > 4;  // two M tiles of query rows
+  const int copies = gqa_copies(nch);
+  const f32x2 s2 = pk2(sl2, sl2);
   // body(ra, ch) for every query chunk of the tile in the region.
   auto for_chunks = [&](auto&& body) {
 #pragma unroll 1
@@ -1609,66 +1682,74 @@ __device__ void gqa_compute_role(const Ctx& c, const FusedParams& p, const GqaLa
     int32_t* J = unit_J(c, p, 0, lev);
     const uint32_t keys_a = smem_u32(J);
 
-    // Pass 1: this warp's (stabiliser, sum) of each query column over its
-    // rows, in its own slots (lane l: column 32 ch + l of every chunk).
-    float2* wsw = wst + warp * nqp;
+    // Pass 1: this thread's query row over the tile's candidates, 32 columns at
+    // a time.
+    const int ncol = TM / (two ? 1 : copies);            // this thread's columns of a tile:
+    const int ccol = two ? 0 : row / nqp * ncol;           // from ccol on
+    float rmax = -INFINITY;  // the row's stabiliser (log2 units)
+    f32x2 rsum = pk2(0.f, 0.f);
 #pragma unroll 1
-    for (int ch = 0; ch < nch; ++ch) wsw[32 * ch + lane] = make_float2(-INFINITY, 0.f);
-    // This warpgroup's last tile stays in its region for pass 2.
-    const int tkeep = ntl - 1 - wg >= 0 ? wg + (ntl - 1 - wg) / 2 * 2 : -1;
-#pragma unroll 1
-    for (int t = wg; t < ntl; t += 2) {
-      wait_or_abort(bar_addr(ms.rdone[wg]), dpar, ms, p.status);
-      dpar ^= 1u;
+    for (int t = two ? 0 : (int)(((uint32_t)wg - used) & 1u); t < ntl; t += two ? 1 : 2) {
+      const uint32_t use = used + (uint32_t)t;
+      const int b = (int)(use & 1u);
+      wait_or_abort(bar_addr(ms.p1done[b]), (use >> 1) & 1u, ms, p.status);
       tc_fence_after();
-      const bool valid = t * TM + row < mc;
-      for_chunks([&](const uint32_t (&ra)[32], int ch) {
-        // Exponentials relative to the chunk's largest logit among the warp's
-        // rows (one warp-wide max), summed per column across the rows.
-        float e[32];
+      const uint32_t tc = c.tmem + lane_base + (two ? 256u * (uint32_t)b + 128u * (uint32_t)wg : 128u * (uint32_t)b);
+      const int nv = min(mc - t * TM, TM);  // candidates of the tile
+#pragma unroll 1
+      for (int c0 = ccol; c0 < min(nv, ccol + ncol); c0 += 32) {
+        uint32_t ra[32];
+        tmem_ld32_issue(tc + (uint32_t)c0, ra);
+        tmem_wait_ld();
+        if (nv - c0 < 32) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) ra[i] = i < nv - c0 ? ra[i] : __float_as_uint(-INFINITY);
+        }
         float vm = -INFINITY;
 #pragma unroll
         for (int i = 0; i < 32; i += 2) vm = fmax3(vm, __uint_as_float(ra[i]), __uint_as_float(ra[i + 1]));
-        float tm = warp_max_f32(valid ? vm : -INFINITY);
-        const float ntm = -tm * sl2;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) e[i] = valid ? ex2(fmaf(__uint_as_float(ra[i]), sl2, ntm)) : 0.f;
-        float ts = transpose_reduce32<false>(e, lane);  // lane l: column l's sum
-        // A column whose every term flushed to zero (logits more than ~126
-        // below the chunk's largest, in log2 units) is summed again against
-        // each column's own maximum (the warp decides together).
-        if (__any_sync(0xffffffffu, !(ts > 0.f) && tm > -INFINITY)) {
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const float v = valid ? __uint_as_float(ra[i]) : -INFINITY;
-            const float mi = warp_max_f32(v);  // column i's largest logit among the warp's rows
-            tm = lane == i ? mi : tm;
-            e[i] = valid ? ex2((v - mi) * sl2) : 0.f;
-          }
-          ts = transpose_reduce32<false>(e, lane);
+        const float xm = vm * sl2;
+        if (xm > rmax + kRaise) {  // also the first columns (rmax = -inf)
+          const float f = ex2(rmax - xm);
+          rsum = mul2(rsum, pk2(f, f));
+          rmax = xm;
         }
-        wsw[32 * ch + lane] = merge_ms(wsw[32 * ch + lane], make_float2(tm * sl2, ts));
-      });
+        const float nm = rmax > -INFINITY ? -rmax : 0.f;
+        const f32x2 nm2 = pk2(nm, nm);
+        f32x2 z[2] = {pk2(0.f, 0.f), pk2(0.f, 0.f)};
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          const float2 x = up2(fma2(pk2(__uint_as_float(ra[2 * k]), __uint_as_float(ra[2 * k + 1])), s2, nm2));
+          z[k & 1] = add2(z[k & 1], pk2(ex2(x.x), ex2(x.y)));
+        }
+        rsum = add2(rsum, add2(z[0], z[1]));
+      }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0 && t != tkeep) mbar_arrive(bar_addr(ms.rfree[wg]));
+      if (lane == 0) mbar_arrive(bar_addr(ms.p1free[b]));
     }
-    // The eight warps' statistics -> the CTA's (M, S) per column, sent to
-    // every cluster CTA.
-    csync<true>();
+    // The CTA's (M, S) per query row, sent to every cluster CTA.
     {
-      const uint32_t xbar = bar_addr(ms.xbar[0]);
-      const uint32_t nr = aborted(ms) ? 0u : c.cs;  // after a wait gave up, nothing goes to the cluster
+      const float2 rs2 = up2(rsum);
+      float2 st = make_float2(rmax, rs2.x + rs2.y);
+      if (!two) {
+        wst[tid] = st;
+        csync<true>();
+        // Query row `tid` from both warpgroups and every copy of the block.
+        if (tid < nqp) {
+          st = wst[tid];
 #pragma unroll 1
-      for (int col = tid; col < nqp; col += TN) {
-        float2 a = wst[col];
-#pragma unroll
-        for (int w8 = 1; w8 < 8; ++w8) a = merge_ms(a, wst[w8 * nqp + col]);
-        const uint32_t dst = smem_u32(&xst[c.rank * nqp + col]);
-#pragma unroll 1
-        for (uint32_t r = 0; r < nr; ++r)
-          st_async_v2(map_rank(dst, r), __float_as_uint(a.x), __float_as_uint(a.y), map_rank(xbar, r));
+          for (int e = 1; e < 2 * copies; ++e) st = merge_ms(st, wst[(e & 1) * TM + (e >> 1) * nqp + tid]);
+        }
       }
+      const int col = tid;  // (two M tiles: warpgroup w's row is query row 128 w + row)
+      const bool own = col < nqp;
+      const uint32_t xbar = bar_addr(ms.xbar[0]);
+      const uint32_t nr = aborted(ms) || !own ? 0u : c.cs;  // after a wait gave up, nothing goes to the cluster
+      const uint32_t dst = smem_u32(&xst[c.rank * nqp + (own ? col : 0)]);
+#pragma unroll 1
+      for (uint32_t r = 0; r < nr; ++r)
+        st_async_v2(map_rank(dst, r), __float_as_uint(st.x), __float_as_uint(st.y), map_rank(xbar, r));
     }
     wait_cluster_or_abort(bar_addr(ms.xbar[0]), ph, ms, p.status);
     if (tid == 0 && lev > c.lev_end && !aborted(ms))
@@ -1686,33 +1767,36 @@ __device__ void gqa_compute_role(const Ctx& c, const FusedParams& p, const GqaLa
     float kmin = INFINITY, kmax = -INFINITY;
     const uint32_t kbar = bar_addr(ms.kbar[0]);
     const uint32_t nr = aborted(ms) ? 0u : c.cs;
-    // The kept tile first (its logits are in the region), then the earlier
-    // tiles as the MMA thread re-issues them.
+    const int nkeep = min(ntl, S), nre = ntl - nkeep;
 #pragma unroll 1
-    for (int k = 0; tkeep >= 0 && k <= tkeep / 2; ++k) {
-      const int t = k == 0 ? tkeep : wg + 2 * (k - 1);
-      if (k > 0) {
-        wait_or_abort(bar_addr(ms.rdone[wg]), dpar, ms, p.status);
-        dpar ^= 1u;
-        tc_fence_after();
-      }
+    for (int k = (int)(((uint32_t)wg - used) & 1u); k < ntl; k += 2) {
+      const int t = k < nkeep ? nre + k : k - nkeep;
+      const uint32_t use = used + (uint32_t)k, reg = use % nreg;
+      wait_or_abort(bar_addr(ms.rdone[reg]), (use / nreg) & 1u, ms, p.status);
+      tc_fence_after();
+      treg = c.tmem + gqa_region0(nch) + reg * 32u * (uint32_t)nch;
       // Every exponent l sl2 - c_i is at most 0 (c_i is the log of a sum that
       // holds the row's own term), so the sum is taken unshifted; a row whose
       // sum is tiny (below 2^-96, where flushed terms could matter) is taken
       // again shifted by its largest exponent (the warp together).
       float rm = 0.f, rs = 0.f;
+      f32x2 z[2] = {pk2(0.f, 0.f), pk2(0.f, 0.f)};
       for_chunks([&](const uint32_t (&ra)[32], int ch) {
-        float z = 0.f;
 #pragma unroll
         for (int k4 = 0; k4 < 8; ++k4) {
           const uint4 cv = lds_v4(ncvec_a + 16u * (uint32_t)(8 * ch + k4));
-          z += ex2(fmaf(__uint_as_float(ra[4 * k4]), sl2, __uint_as_float(cv.x)));
-          z += ex2(fmaf(__uint_as_float(ra[4 * k4 + 1]), sl2, __uint_as_float(cv.y)));
-          z += ex2(fmaf(__uint_as_float(ra[4 * k4 + 2]), sl2, __uint_as_float(cv.z)));
-          z += ex2(fmaf(__uint_as_float(ra[4 * k4 + 3]), sl2, __uint_as_float(cv.w)));
+          const float2 x = up2(fma2(pk2(__uint_as_float(ra[4 * k4]), __uint_as_float(ra[4 * k4 + 1])), s2,
+                                    pk2(__uint_as_float(cv.x), __uint_as_float(cv.y))));
+          const float2 y = up2(fma2(pk2(__uint_as_float(ra[4 * k4 + 2]), __uint_as_float(ra[4 * k4 + 3])), s2,
+                                    pk2(__uint_as_float(cv.z), __uint_as_float(cv.w))));
+          z[0] = add2(z[0], pk2(ex2(x.x), ex2(x.y)));
+          z[1] = add2(z[1], pk2(ex2(y.x), ex2(y.y)));
         }
-        rs += z;
       });
+      {
+        const float2 zz = up2(add2(z[0], z[1]));
+        rs = zz.x + zz.y;
+      }
       if (__any_sync(0xffffffffu, rs < 0x1p-96f && t * TM + row < mc)) {
         float mxr = -INFINITY;
         for_chunks([&](const uint32_t (&ra)[32], int ch) {
@@ -1743,7 +1827,7 @@ __device__ void gqa_compute_role(const Ctx& c, const FusedParams& p, const GqaLa
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar_addr(ms.rfree[wg]));
+      if (lane == 0) mbar_arrive(bar_addr(ms.rfree[reg]));
       const int j = t * TM + row;
       if (j < mc) {
         const float key = rm + lg2(rs);
@@ -1776,6 +1860,7 @@ __device__ void gqa_compute_role(const Ctx& c, const FusedParams& p, const GqaLa
       lo = warp_min_f32(mm.x);
       hi = warp_max_f32(mm.y);
     }
+    used += (uint32_t)ntl;
     // Eq. 9: Top-K (the same result in every CTA of the cluster).
     select_topk<true>(keys_a, m, kb, smem_u32(unit_J(c, p, 0, lev + 1)), lev == p.L, sc_a, lo, hi);
     if (tid == 0) {
@@ -1838,6 +1923,10 @@ __global__ void __launch_bounds__(NT, 1) wf_gqa_filter_kernel(const __grid_const
     mbar_init(bar_addr(ms.xbar[0]), 1);
     mbar_init(bar_addr(ms.kbar[0]), 1);
     for (int r = 0; r < 2; ++r) {
+      mbar_init(bar_addr(ms.p1done[r]), 1);
+      mbar_init(bar_addr(ms.p1free[r]), p.nch > 4 ? 2 * NCW : NCW);
+    }
+    for (int r = 0; r < MAXREG; ++r) {
       mbar_init(bar_addr(ms.rdone[r]), 1);
       mbar_init(bar_addr(ms.rfree[r]), NCW);
     }
@@ -1873,7 +1962,7 @@ __global__ void __launch_bounds__(NT, 1) wf_gqa_filter_kernel(const __grid_const
     c.tmem = ms.tmem_base;
     cluster_sync();  // every CTA's barriers are armed before any remote arrival
     if (warp < MMA_WARP) {
-      gqa_compute_role(c, p, gl);
+      gqa_compute_role<S>(c, p, gl);
     } else {
       if ((tid & 31) == 0) gqa_mma_role<S>(c, p);
       __syncwarp();
@@ -2144,7 +2233,11 @@ cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd
 // with 20 launches for the filter and takes 80 us with this one.)
 // One unit per cluster; the largest cluster of up to 8 CTAs
 // whose grid fits the SMs in one wave with every cluster resident.
-constexpr int kGqaStages = 3 * 128 / D;
+constexpr int kGqaStages = 3 * 128 / D;  // least stages: beside 256 stacked query rows
+typedef void (*GqaKernel)(FusedParams);
+GqaKernel gqa_kernel(int stages) {
+  return stages == MAXS ? wf_gqa_filter_kernel<MAXS> : wf_gqa_filter_kernel<kGqaStages>;
+}
 GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int num_sms) {
   GqaPlan gp{};
   gp.ok = false;
@@ -2158,21 +2251,29 @@ GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int3
   for (int l = 1; l <= levels; ++l) cmax = cmax > 2 * keep[l] ? cmax : 2 * keep[l];
   if (cmax > kMaxCand || kmax > kMaxCand) return gp;
   const int nch = (G * q.seq + NQ - 1) / NQ;
-  constexpr int kStages = kGqaStages;
+  // As many stages as fit: tiles kept in the ring are not streamed again.
+  int stages = 0;
   const size_t kMaxSmem = 227 * 1024;
   int cs = 0;
   size_t smem = 0;
+  auto layout = [&](int c) {
+    stages = MAXS;
+    smem = gqa_layout(stages, nch, c, cmax, kmax).total;
+    if (smem <= kMaxSmem) return;
+    stages = kGqaStages;
+    smem = gqa_layout(stages, nch, c, cmax, kmax).total;
+  };
   for (int c = MAXCS; c >= 1 && cs == 0; --c) {
-    smem = gqa_layout(kStages, nch, c, cmax, kmax).total;
+    layout(c);
     if (smem > kMaxSmem || U * c > num_sms) continue;
     static std::mutex mu;
-    static std::map<std::tuple<int, int, size_t>, int> cache;
+    static std::map<std::tuple<int, int, int, size_t>, int> cache;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return gp;
     int n = 0;
     {
       std::lock_guard<std::mutex> lock(mu);
-      const auto key = std::make_tuple(dev, c, smem);
+      const auto key = std::make_tuple(dev, stages, c, smem);
       auto it = cache.find(key);
       if (it != cache.end()) {
         n = it->second;
@@ -2188,9 +2289,9 @@ GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int3
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaError_t e = cudaFuncSetAttribute(wf_gqa_filter_kernel<kStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kMaxSmem);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, wf_gqa_filter_kernel<kStages>, &cfg);
+        const GqaKernel k = gqa_kernel(stages);
+        cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(k), smem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
         if (e != cudaSuccess) {
           (void)cudaGetLastError();
           n = 0;
@@ -2202,14 +2303,13 @@ GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int3
   }
   if (cs == 0) {  // more units than one wave holds: single-CTA clusters in several waves
     cs = 1;
-    smem = gqa_layout(kStages, nch, 1, cmax, kmax).total;
+    layout(1);
     if (smem > kMaxSmem) return gp;
   }
-  int cols = 32;
-  while (cols < 2 * NQ * nch) cols *= 2;
+  const int cols = 512;  // both passes' columns
   gp.ok = true;
   gp.cs = cs;
-  gp.stages = kStages;
+  gp.stages = stages;
   gp.smem = smem;
   gp.tmem_cols = cols;
   gp.nch = nch;
@@ -2265,10 +2365,10 @@ cudaError_t launch_gqa_filter(const GqaPlan& gp, const void* Q, const wf_tensor&
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaFuncSetAttribute(wf_gqa_filter_kernel<kGqaStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)gp.smem);
+  const GqaKernel k = gqa_kernel(gp.stages);
+  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(k), gp.smem);
   if (e != cudaSuccess) return e;
-  e = cudaLaunchKernelEx(&cfg, wf_gqa_filter_kernel<kGqaStages>, p);
+  e = cudaLaunchKernelEx(&cfg, k, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

@@ -57,3 +57,24 @@ def test_filter_route(B, H, group, q, n, L, k, bshd):
         got = run.level_sets(u)
         for lev in range(L, -1, -1):
             assert np.array_equal(got[lev], sets[lev]), f"unit {u} scale {lev}"
+
+
+@pytest.mark.parametrize("B,H,group,q,n,L,k", [
+    (1, 20, 7, 32, 16384, 3, 2048),  # clusters of 6 or 7: three tiles a slice, every one kept in the ring
+    (3, 30, 4, 32, 16384, 3, 2048),  # one CTA a cluster: 16 tiles a scale, one M tile
+    (3, 30, 8, 32, 16384, 3, 2048),  # the same with two M tiles (three ring stages): 13 tiles streamed again
+    (5, 40, 1, 48, 4096, 2, 512),    # more units than SMs, a ragged chunk of query rows
+])
+def test_grouped_filter_streams_again(B, H, group, q, n, L, k):
+    # The grouped filter's second pass multiplies the tiles that are still in
+    # the ring and streams the others again.
+    w = synth.Workload("grouped_filter", B, H, 128, n, q, 1, L, tuple(wf.wf_default_schedule(n, L, k)), "bf16", "iid",
+                       group=group)
+    units = [0, B * H // 2, B * H - 1]
+    b = synth.make_batch(w, planted=True, device="cuda", cfg="grouped", units=units)
+    run = LibRun(b.Q, b.K, b.V, None, None, L, w.keep).dwt().filter()
+    torch.cuda.synchronize()
+    for u in units:
+        got = run.level_sets(u)
+        for lev in range(L, -1, -1):
+            assert np.array_equal(got[lev], b.targets[u][lev].cpu().numpy()), f"unit {u} scale {lev}"
