@@ -253,6 +253,8 @@ wf_status wf_filter_wavelet(const void* Q, const wf_tensor* q, const void* top, 
  * tensor-core kernel's bounded wait gives up (bf16 keys with head_dim 128 run
  * on the tensor cores): zero it once, read it with wf_workspace_status().
  * Out-of-range idx entries are clamped to [0, n) (never read out of bounds).
+ * bf16 with one query head per key head, q <= 32 and k <= 8192 runs as one
+ * launch of wf_step's fused kernel (its attention alone).
  * ------------------------------------------------------------------------- */
 size_t wf_attn_workspace_bytes(const wf_tensor* q, int k, int n_g);
 wf_status wf_sparse_attn(const void* Q, const wf_tensor* q, const void* K, const void* V, const wf_tensor* kv,

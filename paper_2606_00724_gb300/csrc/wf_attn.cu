@@ -242,7 +242,26 @@ cudaError_t launch_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd, c
                         const wf_tensor& kv, const int32_t* idx, const void* Kg, const void* Vg,
                         const wf_tensor* g, void* O, const wf_tensor& od, float scale, void* ws, int* status,
                         cudaStream_t s) {
-  // bf16 with head_dim 128: tensor cores.
+  // bf16, one query head per key head, at most 32 query rows: the attention of
+  // the fused step, one launch: the partials of a unit meet in the cluster's
+  // shared memory instead of going through memory to a second kernel.  32
+  // heads, 1042 keys, head_dim 128: 15.7 us against 9.1 + 6.2 and a gap between
+  // the two (filter then attention at 20K tokens 69.0 -> 65.5 us).
+  const int sms = sm_count();
+  if (p.dtype == WF_BF16 && p.G == 1 && sms > 0) {
+    const int32_t keep = p.k;
+    const FusedPlan fp = plan_fused(qd, kv, 0, &keep, p.ng, sms);
+    if (fp.ok) {
+      FusedRange r{};
+      r.lev_top = 0;
+      r.lev_bot = 1;
+      r.attn = 1;
+      r.sel = idx;
+      r.scale = scale;
+      return launch_fused(fp, Q, qd, K, V, kv, Kg, Vg, g, nullptr, 0, &keep, nullptr, nullptr, O, od, status, s, &r);
+    }
+  }
+  // Other bf16 with head_dim 128: tensor cores.
   if (tc_attn_supported(p, p.G * p.q)) {
     int nsplit = 0;
     cudaError_t e = launch_tc_attn(p, Q, qd, K, V, kv, idx, Kg, Vg, g, scale, status, ws, &nsplit, s);

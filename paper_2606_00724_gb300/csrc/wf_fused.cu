@@ -203,6 +203,9 @@ struct FusedParams {
   const int32_t* jin;
   int32_t* jout;
   int64_t jstride;  // entries per unit of jin and jout
+  // Attention alone (no scale; L = 0, trim): the caller's token list
+  // [units][keep[0]], any order, clamped to the prompt; else null.
+  const int32_t* sel;
   // Literal-basis rows: scale lev_top's candidate rows in candidate order
   // (row j of unit u at lrows + u lrows_unit + j D); null for the pyramid.
   const bf16* lrows;
@@ -471,7 +474,7 @@ __device__ void producer_role(const Ctx& c, const FusedParams& p) {
       it += ntl;
     }
   }
-  const int nsel = c.lev_top - c.lev_end + 1;
+  const int nsel = p.sel ? 1 : c.lev_top - c.lev_end + 1;  // selections made (or handed in)
   for (int pp = 0; pp < c.np && p.attn; ++pp) {
     wait_or_abort(bar_addr(ms.jready[pp]), (uint32_t)(nsel - 1) & 1u, ms, p.status);
     int a0, mc;
@@ -1219,6 +1222,14 @@ __device__ void compute_role(const Ctx& c, const FusedParams& p) {
 #pragma unroll 1
     for (int i = tid; i < p.keep[c.lev_top + 1]; i += TN) Jp[i] = src[2 * i] >> 1;
   }
+  if (p.sel) {
+    const int32_t* src = p.sel + (int64_t)u * p.keep[0];
+    int32_t* J = unit_J(c, p, pp, 0);
+#pragma unroll 1
+    for (int i = tid; i < p.keep[0]; i += TN) J[i] = min(max(src[i], 0), p.n - 1);
+    csync<WIDE>();
+    if (tid == 0) mbar_arrive(bar_addr(ms.jready[pp]));
+  }
   // The first pass through the Top-K's code fetches its instructions from
   // memory, where they queue behind the first scale's row streams (several us
   // at 32K).  In a two-unit cluster unit 1's warpgroup, which waits for its
@@ -1381,9 +1392,11 @@ __global__ void __launch_bounds__(NT, 1) wf_fused_kernel(const __grid_constant__
     if (tid == 0) {
       // Arm the first phase of every receive barrier (bytes this CTA expects).
       for (int pp = 0; pp < c.np; ++pp) {
-        mbar_arrive_expect_tx(bar_addr(ms.xbar[pp]), c.cs * NQ * 8u);
-        mbar_arrive_expect_tx(bar_addr(ms.kbar[pp]),
-                              4u * (uint32_t)m_total(p, c.lev_top) + c.cs * unit_warps<WIDE>() * 8u);
+        if (c.lev_top >= c.lev_end) {
+          mbar_arrive_expect_tx(bar_addr(ms.xbar[pp]), c.cs * NQ * 8u);
+          mbar_arrive_expect_tx(bar_addr(ms.kbar[pp]),
+                                4u * (uint32_t)m_total(p, c.lev_top) + c.cs * unit_warps<WIDE>() * 8u);
+        }
         const uint32_t rows = (uint32_t)(dlo((int)c.rank + 1, c.cs) - dlo((int)c.rank, c.cs));
         mbar_arrive_expect_tx(bar_addr(ms.cbar[pp]), c.cs * rows * NQ * 4u + c.cs * NQ * 8u);
       }
@@ -2058,8 +2071,9 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   if (kv.dtype != WF_BF16 || kv.head_dim != D || q.seq > NQ || levels > 10) return fp;
   const int U = kv.batch * kv.heads;
   const int n = kv.seq;
-  const bool trim = keep[0] < 2 * keep[1];
-  int cmax = n >> levels, kmax = 0;
+  const bool filter = levels > 0;  // else the attention alone, over a list of keep[0] tokens
+  const bool trim = !filter || keep[0] < 2 * keep[1];
+  int cmax = filter ? n >> levels : 0, kmax = 0;
   for (int l = 0; l <= levels; ++l) kmax = kmax > keep[l] ? kmax : keep[l];
   for (int l = 1; l <= levels; ++l) cmax = cmax > 2 * keep[l] ? cmax : 2 * keep[l];
   if (cmax > kMaxCand || kmax > kMaxCand) return fp;
@@ -2069,7 +2083,7 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   // TMEM tiles of the widest scale slice at cluster size cs.
   auto scale_tiles = [&](int cs) {
     auto slice_tiles = [&](int m) { return (2 * (((m + 1) / 2 + cs - 1) / cs) + TM - 1) / TM; };
-    int tmax = slice_tiles(n >> levels);
+    int tmax = filter ? slice_tiles(n >> levels) : 0;
     for (int l = levels; l >= 1; --l) {
       const int t = slice_tiles(2 * keep[l]);
       tmax = tmax > t ? tmax : t;
@@ -2087,7 +2101,7 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   // are long enough for the halved per-thread work to outweigh the wider
   // barriers (measured: 128K tokens 123.6 -> 116.8 us; 8K tokens, lists of at
   // most 1024, 49.5 -> 51.6 us).
-  const bool wide1 = cmax >= 2048;
+  const bool wide1 = cmax >= 2048 || (!filter && total >= 2048);
   // For P units per cluster (1, or 2 so that one unit's copies overlap the
   // other's exchanges and Top-K): the largest cluster (any size up to 8)
   // whose grid fits the SMs in one wave, all clusters resident at once, and
@@ -2126,7 +2140,7 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   const int stiles = scale_tiles(cs);
   int ecol = 0;
   const int ecols = ucols > 64 * stiles ? ucols : 64 * stiles;
-  if (P * ecols <= 512) {
+  if (filter && P * ecols <= 512) {
     ecol = 32 * stiles;
     ucols = ecols;
   }
@@ -2196,6 +2210,8 @@ cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd
     p.jin = range->jin;
     p.jout = range->jout;
     p.jstride = range->jstride;
+    p.sel = range->sel;
+    if (range->scale > 0.f) p.scale_log2 = kLog2e * range->scale;
     p.lrows = static_cast<const bf16*>(range->lrows);
     p.lrows_unit = range->lrows_unit;
   } else {

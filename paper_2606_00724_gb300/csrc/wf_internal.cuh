@@ -159,6 +159,10 @@ struct FusedRange {
   int64_t jstride;
   const void* lrows;
   int64_t lrows_unit;
+  // The attention alone (levels = 0, lev_top = 0, lev_bot = 1): the token lists
+  // [units][keep[0]] and the softmax scale (0: 1 / sqrt(d)).
+  const int32_t* sel;
+  float scale;
 };
 // launch_literal_fused: the literal-basis filter on the fused kernel (bf16, one query head
 // per KV head, a fused plan fp for the same shapes): one launch per scale,
@@ -178,7 +182,7 @@ struct GqaPlan {
 };
 // The entry points, once per head_dim (wf_fused.cu is compiled for each).
 // plan_fused: n_g generation rows of the attention, or -1 for a plan of the
-// filter alone.  launch_fused: range == nullptr is the whole step (every
+// filter alone; levels = 0 for a plan of the attention alone (keep[0] tokens).  launch_fused: range == nullptr is the whole step (every
 // scale, mu^0, the attention).
 #define WF_FUSED_ENTRY_POINTS                                                                                       \
   FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g,           \

@@ -1,0 +1,56 @@
+"""wf_sparse_attn on the fused kernel's attention (bf16, one query head a key
+head, at most 32 query rows) at its edges: fewer keys than CTAs in the
+cluster, ragged slices, two units a cluster, both warpgroups on a unit, lists
+of 8192 tokens (its largest) and beyond (the split kernels), unsorted,
+repeated and out-of-range tokens (clamped), an explicit scale, [B, rows, H, d]
+strides, both head dims.  Outputs against the fp64 oracle: O is rounded to
+bf16 once and, for head_dim 128, so is P (relative 2^-9 each, the weights'
+errors averaging below their bound): the bf16 bound of the other tests."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import assert_close_out, f64
+from paper_2606_00724_gb300 import wf
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+
+@pytest.mark.parametrize("B,H,d,q,n,k,ng,scale,bshd", [
+    (1, 1, 128, 1, 64, 1, 0, 0.0, False),
+    (1, 2, 64, 32, 256, 3, 2, 0.0, True),
+    (2, 3, 128, 17, 2048, 333, 5, 0.25, True),
+    (2, 32, 128, 32, 4096, 517, 32, 0.0, False),   # two units a cluster
+    (1, 32, 64, 31, 8192, 1000, 7, 0.2, True),
+    (1, 2, 128, 32, 16384, 8192, 3, 0.0, False),   # both warpgroups, the largest list
+    (1, 1, 128, 32, 16384, 8193, 0, 0.0, False),   # the split kernels
+    (3, 60, 128, 5, 1024, 200, 0, 0.0, False),     # more clusters than fit at once
+])
+def test_attention_route(B, H, d, q, n, k, ng, scale, bshd):
+    g = torch.Generator(device="cpu").manual_seed(k + d)
+
+    def rn(rows):
+        t = torch.randn(B, H, rows, d, generator=g).to(torch.bfloat16).cuda()
+        return t.transpose(1, 2).contiguous().transpose(1, 2) if bshd else t
+
+    Q, K, V, Kg, Vg = rn(q), rn(n), rn(n), rn(max(ng, 1)), rn(max(ng, 1))
+    idx = torch.randint(0, n, (B * H, k), generator=g, dtype=torch.int32)
+    if k > 2:
+        idx[0, 0], idx[-1, -1] = -5, n + 7
+    O = torch.empty_like(Q)
+    ws = torch.zeros(wf.wf_attn_workspace_bytes(Q, k, ng), dtype=torch.uint8, device="cuda")
+    wf.wf_sparse_attn(Q, K, V, idx.cuda(), k, Kg if ng else None, Vg if ng else None, O, ws, scale)
+    wf.wf_workspace_status(ws)
+    torch.cuda.synchronize()
+    for u in {0, B * H // 2, B * H - 1}:
+        i, h = divmod(u, H)
+        # an explicit scale is a factor of the queries
+        Qs = f64(Q[i, h]) * (scale * d ** 0.5 if scale else 1.0)
+        at = idx[u].numpy().clip(0, n - 1)
+        want = oracle.sparse_attn(Qs, f64(K[i, h]), f64(V[i, h]), at, f64(Kg[i, h]) if ng else None,
+                                  f64(Vg[i, h]) if ng else None)
+        assert_close_out(f64(O[i, h]), want, torch.bfloat16)
