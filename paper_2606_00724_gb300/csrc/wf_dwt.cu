@@ -11,9 +11,15 @@
 //
 // The update mode (wf_cache_update) runs the same cascade over only the blocks
 // that contain token positions [pos, pos + count): a thread takes its slice of
-// a new row from the update buffer, writes it into the cache (and the value
-// slice too), and takes every other row of the block from the cache, so the
-// coefficients it writes equal those of a full build of the updated keys.
+// a new row from the update buffer and writes it into the cache, and takes
+// every other row of the block from the cache, so the coefficients it writes
+// equal those of a full build of the updated keys.  The value rows are copied
+// by CTAs of their own.  An update moves a few MB over a few thousand threads,
+// so it is bound by its chain of memory latencies: every load of a chunk is
+// issued before the first store (the row's source is chosen as an address, not
+// by a branch around the load), the next chunk's loads before this one's
+// arithmetic, and CTAs are small, to use more SMs (32 rows of 64 units at 32K,
+// four scales: 9.3 -> 3.2 us a launch).
 #include "wf_internal.cuh"
 
 namespace wf {
@@ -30,16 +36,28 @@ struct Update {
   int64_t blk0;           // first block of the unit that holds a new row
 };
 
+constexpr int kBuildThreads = 256, kUpdateThreads = 64;
+
 template <typename T, int L, bool UPDATE>
-__global__ void __launch_bounds__(256) dwt_kernel(const T* K_in, T* K_out, int64_t sb, int64_t sh,
+__global__ void __launch_bounds__(UPDATE ? kUpdateThreads : kBuildThreads) dwt_kernel(const T* K_in, T* K_out, int64_t sb, int64_t sh,
                                                   int64_t ss, int H, int n, int D, T* __restrict__ coeffs,
                                                   int64_t rows_total, int64_t nblk, int64_t total_items,
-                                                  Update<T> up) {
+                                                  int64_t key_ctas, Update<T> up) {
   constexpr int VEC = Vec<T>::N;
   constexpr int LC = L < 3 ? L : 3;
   constexpr int CH = 1 << LC;
   constexpr int NP = L > LC ? L - LC : 1;
   const int lanes = D / VEC;
+  if (UPDATE && blockIdx.x >= key_ctas) {
+    // A 16-byte slice of a new value row.
+    const int64_t e = ((int64_t)blockIdx.x - key_ctas) * blockDim.x + threadIdx.x;
+    const int64_t r = e / lanes % up.count, u = e / lanes / up.count;
+    if (u >= total_items / (nblk * lanes)) return;
+    const int64_t bb = u / H, hh = u % H, x = e % lanes * VEC;
+    const uint4 w = __ldg(reinterpret_cast<const uint4*>(up.Vn + bb * up.nsb + hh * up.nsh + r * up.nss + x));
+    *reinterpret_cast<uint4*>(up.V + bb * sb + hh * sh + (up.pos + r) * ss + x) = w;
+    return;
+  }
   const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (item >= total_items) return;
   const int lane = (int)(item % lanes);
@@ -53,27 +71,38 @@ __global__ void __launch_bounds__(256) dwt_kernel(const T* K_in, T* K_out, int64
   const float c = 0.70710678118654752440f;  // fl32(1/sqrt 2)
 
   float pend[NP][VEC];
-#pragma unroll 1
-  for (int ch = 0; ch < (1 << (L - LC)); ++ch) {
-    float v[CH][VEC];
+  // Update mode: the chunk's rows as loaded, and which of them are new.
+  uint4 raw[CH];
+  auto is_new = [&](int64_t tok) { return tok >= up.pos && tok < up.pos + up.count; };
+  auto fetch = [&](int ch) {
 #pragma unroll
     for (int t = 0; t < CH; ++t) {
       const int64_t tok = tok0 + ch * CH + t;
-      if (UPDATE && tok >= up.pos && tok < up.pos + up.count) {
-        // A new row: read it from the update buffer, store it into the cache.
-        const int64_t r = tok - up.pos;
-        const int64_t no = bb * up.nsb + hh * up.nsh + r * up.nss + (int64_t)lane * VEC;
-        const int64_t co = bb * sb + hh * sh + tok * ss + (int64_t)lane * VEC;
-        ld_vec(up.Kn + no, v[t]);
-        st_vec(K_out + co, v[t]);
-        if (up.Vn) {
-          float vv[VEC];
-          ld_vec(up.Vn + no, vv);
-          st_vec(up.V + co, vv);
-        }
-      } else {
-        ld_vec(src + (int64_t)(ch * CH + t) * ss, v[t]);
+      const T* row = is_new(tok) ? up.Kn + bb * up.nsb + hh * up.nsh + (tok - up.pos) * up.nss + (int64_t)lane * VEC
+                                 : src + (int64_t)(ch * CH + t) * ss;
+      raw[t] = __ldg(reinterpret_cast<const uint4*>(row));
+    }
+  };
+  if (UPDATE) fetch(0);
+#pragma unroll 1
+  for (int ch = 0; ch < (1 << (L - LC)); ++ch) {
+    float v[CH][VEC];
+    if (UPDATE) {
+#pragma unroll
+      for (int t = 0; t < CH; ++t) widen_vec(src, raw[t], v[t]);
+      uint4 own[CH];
+#pragma unroll
+      for (int t = 0; t < CH; ++t) own[t] = raw[t];
+      if (ch + 1 < (1 << (L - LC))) fetch(ch + 1);
+#pragma unroll
+      for (int t = 0; t < CH; ++t) {
+        const int64_t tok = tok0 + ch * CH + t;
+        if (is_new(tok))
+          *reinterpret_cast<uint4*>(K_out + bb * sb + hh * sh + tok * ss + (int64_t)lane * VEC) = own[t];
       }
+    } else {
+#pragma unroll
+      for (int t = 0; t < CH; ++t) ld_vec(src + (int64_t)(ch * CH + t) * ss, v[t]);
     }
     const int64_t gc = (blk << (L - LC)) + ch;  // chunk index within the unit
 #pragma unroll
@@ -116,18 +145,19 @@ cudaError_t run(const void* K, void* K_out, const wf_tensor& kv, void* coeffs, c
   const int64_t rows_total = (int64_t)kv.seq - ((int64_t)kv.seq >> L);
   const int64_t nblk = up.count > 0 ? ((up.pos + up.count - 1) >> L) - (up.pos >> L) + 1 : ((int64_t)kv.seq >> L);
   const int64_t items = (int64_t)U * nblk * lanes;
-  const int threads = 256;
+  const int threads = up.count > 0 ? kUpdateThreads : kBuildThreads;
   const int64_t blocks = (items + threads - 1) / threads;
   if (up.count > 0) {
     Update<T> u2 = up;
     u2.blk0 = up.pos >> L;
-    dwt_kernel<T, L, true><<<(unsigned)blocks, threads, 0, s>>>(
+    const int64_t vblocks = up.Vn ? ((int64_t)U * up.count * lanes + threads - 1) / threads : 0;
+    dwt_kernel<T, L, true><<<(unsigned)(blocks + vblocks), threads, 0, s>>>(
         static_cast<const T*>(K), static_cast<T*>(K_out), kv.stride_b, kv.stride_h, kv.stride_s, kv.heads, kv.seq,
-        kv.head_dim, static_cast<T*>(coeffs), rows_total, nblk, items, u2);
+        kv.head_dim, static_cast<T*>(coeffs), rows_total, nblk, items, blocks, u2);
   } else {
     dwt_kernel<T, L, false><<<(unsigned)blocks, threads, 0, s>>>(
         static_cast<const T*>(K), nullptr, kv.stride_b, kv.stride_h, kv.stride_s, kv.heads, kv.seq, kv.head_dim,
-        static_cast<T*>(coeffs), rows_total, nblk, items, up);
+        static_cast<T*>(coeffs), rows_total, nblk, items, blocks, up);
   }
   return cudaGetLastError();
 }

@@ -19,15 +19,18 @@ template <> struct Vec<bf16> { static constexpr int N = 8; };
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-// Load one 16-byte vector of T and widen it to fp32 (exact).
-__device__ __forceinline__ void ld_vec(const float* p, float* o) {
-  float4 v = __ldg(reinterpret_cast<const float4*>(p));
-  o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+// One 16-byte vector as loaded, widened to fp32 (exact).
+__device__ __forceinline__ void widen_vec(const float*, const uint4& v, float* o) {
+  o[0] = __uint_as_float(v.x); o[1] = __uint_as_float(v.y); o[2] = __uint_as_float(v.z); o[3] = __uint_as_float(v.w);
 }
-__device__ __forceinline__ void ld_vec(const bf16* p, float* o) {
-  uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+__device__ __forceinline__ void widen_vec(const bf16*, const uint4& v, float* o) {
   o[0] = bf16_lo(v.x); o[1] = bf16_hi(v.x); o[2] = bf16_lo(v.y); o[3] = bf16_hi(v.y);
   o[4] = bf16_lo(v.z); o[5] = bf16_hi(v.z); o[6] = bf16_lo(v.w); o[7] = bf16_hi(v.w);
+}
+// Load one 16-byte vector of T and widen it.
+template <typename T>
+__device__ __forceinline__ void ld_vec(const T* p, float* o) {
+  widen_vec(p, __ldg(reinterpret_cast<const uint4*>(p)), o);
 }
 
 // Round fp32 to the storage type (bf16: round to nearest even) and store 16 bytes.

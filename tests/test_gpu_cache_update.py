@@ -87,3 +87,24 @@ def test_cache_update_then_step_matches_rebuild():
     torch.cuda.synchronize()
     assert torch.equal(idx_a, idx_b)
     assert torch.equal(O_a, O_b)
+
+
+@pytest.mark.parametrize("dtype,d,L,pos,count", [
+    (torch.bfloat16, 128, 4, 12340 % 4096, 33),  # blocks of two chunks, the value rows in CTAs of their own
+    (torch.float32, 64, 5, 0, 4096),             # every block
+    (torch.bfloat16, 64, 6, 4095, 1),            # the last token
+])
+def test_update_rows_and_values(dtype, d, L, pos, count):
+    B, H, n = 2, 3, 4096
+    g = torch.Generator(device="cuda").manual_seed(L)
+    rn = lambda rows: torch.randn(B, H, rows, d, generator=g, device="cuda").to(dtype)
+    K, V, Kn, Vn = rn(n), rn(n), rn(count), rn(count)
+    coeffs = torch.empty(wf.wf_coeffs_bytes(K, L), dtype=torch.uint8, device="cuda")
+    wf.wf_dwt_build(K, L, coeffs)
+    K2, V2 = K.clone(), V.clone()
+    K2[:, :, pos:pos + count], V2[:, :, pos:pos + count] = Kn, Vn
+    want = torch.empty_like(coeffs)
+    wf.wf_dwt_build(K2, L, want)
+    wf.wf_cache_update(Kn, Vn, K, V, pos, L, coeffs)
+    torch.cuda.synchronize()
+    assert torch.equal(K, K2) and torch.equal(V, V2) and torch.equal(coeffs, want)
