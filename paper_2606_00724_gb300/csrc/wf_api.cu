@@ -160,7 +160,7 @@ cudaError_t run_filter(const wf::FilterPlan& p, const void* Q, const wf_tensor& 
                               level_sets, nullptr, q, status, s, &r);
     }
   }
-  const wf::F32Plan f32 = wf::plan_f32(q, kv, levels, keep, sms);
+  const wf::F32Plan f32 = wf::plan_f32(q, kv, levels, keep, -1, sms);
   if (f32.ok)
     return wf::launch_f32(f32, Q, q, K, nullptr, kv, nullptr, nullptr, nullptr, coeffs, levels, keep, idx, level_sets,
                           nullptr, q, s);
@@ -410,7 +410,7 @@ WF_API wf_status wf_step(const void* Q, const wf_tensor* q, const void* K, const
                          level_sets, O, *o, status, s, nullptr);
     return cuda_status(e);
   }
-  const wf::F32Plan f32 = wf::plan_f32(*q, *kv, levels, keep, sms);
+  const wf::F32Plan f32 = wf::plan_f32(*q, *kv, levels, keep, n_g, sms);
   if (f32.ok)
     return cuda_status(wf::launch_f32(f32, Q, *q, K, V, *kv, Kg, Vg, n_g > 0 ? g : nullptr, coeffs, levels, keep, idx,
                                       level_sets, O, *o, s));

@@ -6,30 +6,31 @@
 // holds one contiguous slice of the unit's candidate list at every scale, and
 // finally of its sparse key list:
 //   rows    the slice's rows gathered into shared memory (16-byte cp.async),
-//           128 at a time;
-//   logits  2 rows x QM / 4 queries a thread in fp32 FMAs, queries read as
-//           warp-wide broadcasts, kept in shared memory as [query][row];
-//   stats   (max, sum of exp) per query over the slice, one warp a query,
-//           exchanged over the cluster;
-//   keys    log W_j of each row (log-sum-exp over the queries against the
-//           cluster's normalisers), written into every CTA's key array;
+//           all at once where they fit;
+//   logits  2 rows x QM / 4 queries a thread in packed fp32 FMAs, queries read
+//           as warp-wide broadcasts, kept in shared memory as [query][row];
+//   stats   (max, sum of exp) per query over the slice, four queries a warp at a
+//           time, exchanged over the cluster;
+//   keys    log W_j of each row (the sum over the queries against the cluster's
+//           normalisers), written into every CTA's key array;
 //   Top-K   the same selection in every CTA, giving the next scale's rows;
 //   attention over the slice with a running max per query, partial outputs
 //           combined from the cluster's shared memories.
-// Exact fp32 throughout: fused multiply-adds in channel order, expf and logf.
+// Exact fp32 throughout: fused multiply-adds, expf and logf.
 //
 // What bounds it: the chain of dependent phases of a scale (gather, FMAs,
 // two cluster exchanges, Top-K), so the cluster is as wide as the SMs and 8
 // CTAs allow, which shortens the gather and the FMAs.  A 2 x 8 register tile
-// needs 16 shared-memory wavefronts for 64 FMAs a lane: the FMA pipe and
-// shared memory are then about equally busy, where one row x 4 queries a
-// thread needed twice the wavefronts.  Measured against three kernels a scale
-// and two for the attention: 4 heads x 1K tokens (d 64) 63.5 -> 28.7 us a
-// step, 16 heads x 8K (d 128) 170.2 -> 94.0 us, the error against 64 bits
-// unchanged (4.4e-7 and 3.9e-6).
+// takes 16 shared-memory wavefronts for 64 FMAs a lane, which is the most that
+// the reads allow; the FMAs are packed pairs of channels, so that they do not
+// also fill the issue slots.  Measured against three kernels a scale
+// and two for the attention: 4 heads x 1K tokens (d 64) 64.9 -> 22.5 us a
+// step, 16 heads x 8K (d 128) 170.6 -> 75.8 us, the error against 64 bits
+// no larger (3.1e-7 and 2.3e-6; 5.6e-7 and 3.8e-6 before).
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -46,7 +47,6 @@ using namespace topk;
 
 constexpr int NTH = 2 * NCT;  // threads: both warpgroups of a WIDE Top-K
 constexpr int NW = NTH / 32;
-constexpr int TR = 128;       // rows of a tile
 constexpr int MAXCS = 8;
 
 struct F32Params {
@@ -66,7 +66,7 @@ struct F32Params {
   int32_t* level_sets;
   int64_t sets_stride;
   int q, n, ng, H, L, trim, attn;
-  int nbuf, srow, bufw;  // tile buffers, floats of a query's logit row, words of a key buffer
+  int trow, srow, bufw;  // rows of the row buffer, floats of a query's logit row, words of a key buffer
   int32_t keep[12];
   float scale;
 };
@@ -78,16 +78,16 @@ struct F32Layout {
 struct F32Stat {
   float2 xstat[MAXCS][64];  // (max, sum of exp) per query of every CTA's slice
   float2 kmm[MAXCS][NW];    // (min, max) of every warp's keys
-  float2 xch[TR];           // second half's (max, sum) per row
+  float xch[128];           // second half's sum per row
   float ms[64];             // the normalisers; the attention's running max
   float l[64];              // the attention's running row sums
   float alpha[64];          // this tile's factor of the partial output
 };
-__host__ __device__ inline F32Layout f32_layout(int D, int QM, int nbuf, int srow, int bufw) {
+__host__ __device__ inline F32Layout f32_layout(int D, int QM, int trow, int srow, int bufw) {
   F32Layout y;
   y.q = 0;
   y.tile = y.q + 4u * (uint32_t)(QM * D);
-  y.s = y.tile + 4u * (uint32_t)(nbuf * TR * (D + 4));
+  y.s = y.tile + 4u * (uint32_t)(trow * (D + 4));
   y.buf = y.s + 4u * (uint32_t)(QM * srow);
   y.sel = y.buf + 2u * 4u * (uint32_t)bufw;
   y.stat = y.sel + (uint32_t)((sizeof(SelScratch) + 15) / 16 * 16);
@@ -112,64 +112,111 @@ __device__ __forceinline__ float4 ld_cluster_v4(uint32_t a) {
   return v;
 }
 
-// Rows [t0, t0 + min(TR, mc - t0)) of a list into a tile (row stride D + 4
-// floats); row(j) is the address of the list's row j.
+// Rows [t0, t0 + cnt) of a list into a tile (row stride D + 4 floats); row(j)
+// is the address of the list's row j.
 template <int D, typename F>
-__device__ __forceinline__ void gather(float* tile, int t0, int mc, F&& row) {
+__device__ __forceinline__ void gather(float* tile, int t0, int cnt, F&& row) {
   constexpr int LPR = D / 4;  // lanes a row
-  const int c = threadIdx.x % LPR, cnt = min(TR, mc - t0);
+  const int c = threadIdx.x % LPR;
 #pragma unroll 4
   for (int r = threadIdx.x / LPR; r < cnt; r += NTH / LPR)
     cp_async16(smem_u32(tile + r * (D + 4) + 4 * c), row(t0 + r) + 4 * c);
 }
 
-// Logits (x scale) of a tile's rows against every query into S[query][t0 + row].
-// Warp w: rows 64 (w % 2) + lane and + 32, queries QG (w / 2) ..; rows past the
-// tile's cnt compute whatever the tile holds and are not stored.
-template <int D, int QM>
-__device__ __forceinline__ void score_tile(const float* Qs, const float* tile, float* S, int srow, int t0, int cnt,
-                                           float scale) {
-  constexpr int QG = QM / 4;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int r0 = 64 * (w & 1) + lane, q0 = QG * (w >> 1);
-  if (64 * (w & 1) >= cnt) return;
-  const float* p0 = tile + r0 * (D + 4);
-  const float* p1 = p0 + 32 * (D + 4);
-  float a0[QG], a1[QG];
+// Rows of a tile for a list of mc rows in tiles of at most cap: equal tiles,
+// a multiple of 4.
+__device__ __forceinline__ int tile_rows(int mc, int cap) {
+  const int nt = max((mc + cap - 1) / cap, 1);
+  return ((mc + nt - 1) / nt + 3) & ~3;
+}
+
+// Logits (x scale) of rows r0 + lane (+ 32 i, i < RPL) of a tile against QG
+// queries from q0 into S[query][t0 + row].  Rows past the tile's cnt compute
+// whatever the tile holds and are not stored.  Each accumulator is a packed
+// pair, the sums over the even and the odd channels.
+template <int D, int RPL, int QG>
+__device__ __forceinline__ void score_item(const float* Qs, const float* tile, float* S, int srow, int t0, int cnt,
+                                           int r0, int q0, float scale) {
+  const int r = r0 + (threadIdx.x & 31);
+  const ulonglong2* p[RPL];
 #pragma unroll
-  for (int i = 0; i < QG; ++i) a0[i] = a1[i] = 0.f;
+  for (int i = 0; i < RPL; ++i) p[i] = reinterpret_cast<const ulonglong2*>(tile + min(r + 32 * i, cnt - 1) * (D + 4));
+  f32x2 a[RPL][QG];
+#pragma unroll
+  for (int i = 0; i < RPL; ++i)
+#pragma unroll
+    for (int k = 0; k < QG; ++k) a[i][k] = pk2(0.f, 0.f);
 #pragma unroll 2
-  for (int c = 0; c < D; c += 4) {
-    const float4 x = *reinterpret_cast<const float4*>(p0 + c);
-    const float4 y = *reinterpret_cast<const float4*>(p1 + c);
+  for (int c = 0; c < D / 4; ++c) {
+    ulonglong2 x[RPL];
 #pragma unroll
-    for (int i = 0; i < QG; ++i) {
-      const float4 v = *reinterpret_cast<const float4*>(Qs + (q0 + i) * D + c);
-      a0[i] = fmaf(v.w, x.w, fmaf(v.z, x.z, fmaf(v.y, x.y, fmaf(v.x, x.x, a0[i]))));
-      a1[i] = fmaf(v.w, y.w, fmaf(v.z, y.z, fmaf(v.y, y.y, fmaf(v.x, y.x, a1[i]))));
+    for (int i = 0; i < RPL; ++i) x[i] = p[i][c];
+#pragma unroll
+    for (int k = 0; k < QG; ++k) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(Qs + (q0 + k) * D + 4 * c);
+#pragma unroll
+      for (int i = 0; i < RPL; ++i) a[i][k] = fma2(v.y, x[i].y, fma2(v.x, x[i].x, a[i][k]));
     }
   }
 #pragma unroll
-  for (int i = 0; i < QG; ++i) {
-    float* s = S + (q0 + i) * srow + t0;
-    if (r0 < cnt) s[r0] = a0[i] * scale;
-    if (r0 + 32 < cnt) s[r0 + 32] = a1[i] * scale;
+  for (int k = 0; k < QG; ++k) {
+#pragma unroll
+    for (int i = 0; i < RPL; ++i) {
+      const float2 z = up2(a[i][k]);
+      if (r + 32 * i < cnt) S[(q0 + k) * srow + t0 + r + 32 * i] = (z.x + z.y) * scale;
+    }
   }
 }
 
-__device__ __forceinline__ float warp_sum(float x) {
+// A tile's rows against every query: a tile of at most 32 rows splits its
+// queries over all the warps, a larger one goes 64 rows x QM / 4 queries a warp
+// at a time.
+template <int D, int QM>
+__device__ __forceinline__ void score_tile(const float* Qs, const float* tile, float* S, int srow, int t0, int cnt,
+                                           float scale) {
+  const int w = threadIdx.x >> 5;
+  if (cnt <= 32) {
+    if (cnt > 0) score_item<D, 1, QM / NW>(Qs, tile, S, srow, t0, cnt, 0, QM / NW * w, scale);
+    return;
+  }
+#pragma unroll 1
+  for (int it = w; it < 4 * ((cnt + 63) / 64); it += NW)
+    score_item<D, 2, QM / 4>(Qs, tile, S, srow, t0, cnt, 64 * (it >> 2), QM / 4 * (it & 3), scale);
+}
+
+// Four queries' rows of S (srow apart) over cnt rows, by one warp: their maxima
+// (at least m0) and the sums of exp(s - max); with P, the exponentials replace
+// the logits and zeros follow up to row pad.
+template <bool P>
+__device__ __forceinline__ void row_stats(float* s, int srow, int cnt, int pad, float (&mx)[4], float (&z)[4]) {
+  const int lane = threadIdx.x & 31;
+  for (int j = lane; j < cnt; j += 32)
 #pragma unroll
-  for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
+    for (int k = 0; k < 4; ++k) mx[k] = fmaxf(mx[k], s[k * srow + j]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    mx[k] = warp_max_f32(mx[k]);
+    z[k] = 0.f;
+  }
+  for (int j = lane; j < (P ? pad : cnt); j += 32)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float e = !P || j < cnt ? expf(s[k * srow + j] - mx[k]) : 0.f;
+      if (P) s[k * srow + j] = e;
+      z[k] += e;
+    }
+#pragma unroll
+  for (int o = 16; o; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) z[k] += __shfl_xor_sync(0xffffffffu, z[k], o);
 }
 
 template <int D, int QM>
 __global__ void __launch_bounds__(NTH, 1) wf_f32_kernel(const __grid_constant__ F32Params p) {
   extern __shared__ __align__(16) uint8_t smem[];
-  const F32Layout ly = f32_layout(D, QM, p.nbuf, p.srow, p.bufw);
+  const F32Layout ly = f32_layout(D, QM, p.trow, p.srow, p.bufw);
   float* Qs = reinterpret_cast<float*>(smem + ly.q);
   float* T0 = reinterpret_cast<float*>(smem + ly.tile);
-  float* T1 = T0 + (p.nbuf > 1 ? TR * (D + 4) : 0);  // the same buffer when there is one
   float* S = reinterpret_cast<float*>(smem + ly.s);
   F32Stat& st = *reinterpret_cast<F32Stat*>(smem + ly.stat);
   const uint32_t sc_a = smem_u32(smem + ly.sel);
@@ -190,23 +237,18 @@ __global__ void __launch_bounds__(NTH, 1) wf_f32_kernel(const __grid_constant__ 
     *reinterpret_cast<uint4*>(smem + ly.sel + 16 * e) = make_uint4(0, 0, 0, 0);
   cluster_sync();  // every CTA of the cluster runs before any remote store
 
-  // S = scale Q rows^T of a list of mc rows; with two buffers the next tile's
-  // copies run under the current tile's FMAs.
+  // S = scale Q rows^T of a list of mc rows.
   auto score_list = [&](int mc, auto&& row) {
-    gather<D>(T0, 0, mc, row);
-    cp_async_commit();
-    for (int t0 = 0, k = 0; t0 < mc; t0 += TR, k ^= 1) {
-      const bool more = t0 + TR < mc;
-      if (more && p.nbuf > 1) gather<D>(k ? T0 : T1, t0 + TR, mc, row);
-      cp_async_commit();
-      if (p.nbuf > 1) cp_async_wait<1>();
-      else cp_async_wait<0>();
+    const int tr = tile_rows(mc, p.trow);
+    for (int t0 = 0; t0 < mc; t0 += tr) {
+      const int cnt = min(tr, mc - t0);
+      gather<D>(T0, t0, cnt, row);
+      cp_async_wait_all();
       __syncthreads();
-      score_tile<D, QM>(Qs, (p.nbuf > 1 && k) ? T1 : T0, S, p.srow, t0, min(TR, mc - t0), p.scale);
+      score_tile<D, QM>(Qs, T0, S, p.srow, t0, cnt, p.scale);
       __syncthreads();
-      if (more && p.nbuf == 1) gather<D>(T0, t0 + TR, mc, row);
     }
-    cp_async_wait<0>();  // (an empty list's query block)
+    cp_async_wait_all();  // (an empty list's query block)
     __syncthreads();
   };
 
@@ -235,24 +277,27 @@ __global__ void __launch_bounds__(NTH, 1) wf_f32_kernel(const __grid_constant__ 
       });
     }
     // (max, sum of exp) of every query over the slice, to every CTA.
-    for (int i = warp; i < QM; i += NW) {
-      const float* s = S + i * p.srow;
-      float mx = -INFINITY;
-      for (int j = lane; j < mc; j += 32) mx = fmaxf(mx, s[j]);
-      mx = warp_max_f32(mx);
-      float z = 0.f;
-      for (int j = lane; j < mc; j += 32) z += expf(s[j] - mx);
-      z = warp_sum(z);
-      if (lane < cs) st_cluster_v2f32(map_rank(smem_u32(&st.xstat[rank][i]), (uint32_t)lane), mx, z);
+    for (int i = 4 * warp; i < QM; i += 4 * NW) {
+      float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY}, z[4];
+      row_stats<false>(S + i * p.srow, p.srow, mc, 0, mx, z);
+      if (lane < cs)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          st_cluster_v2f32(map_rank(smem_u32(&st.xstat[rank][i + k]), (uint32_t)lane), mx[k], z[k]);
     }
     cluster_sync();
     if (tid < QM) {
+      float2 x[MAXCS];
       float M = -INFINITY;
-      for (int r = 0; r < cs; ++r)
-        if (st.xstat[r][tid].y > 0.f) M = fmaxf(M, st.xstat[r][tid].x);
+#pragma unroll
+      for (int r = 0; r < MAXCS; ++r) {
+        x[r] = r < cs ? st.xstat[r][tid] : make_float2(-INFINITY, 0.f);
+        if (x[r].y > 0.f) M = fmaxf(M, x[r].x);
+      }
       float z = 0.f;
-      for (int r = 0; r < cs; ++r)
-        if (st.xstat[r][tid].y > 0.f) z = fmaf(st.xstat[r][tid].y, expf(st.xstat[r][tid].x - M), z);
+#pragma unroll
+      for (int r = 0; r < MAXCS; ++r)
+        if (x[r].y > 0.f) z = fmaf(x[r].y, expf(x[r].x - M), z);
       st.ms[tid] = M + logf(z);
     }
     __syncthreads();
@@ -260,23 +305,31 @@ __global__ void __launch_bounds__(NTH, 1) wf_f32_kernel(const __grid_constant__ 
     int32_t* J = buf(lev);  // receives this scale's keys, then its selection
     float kmin = INFINITY, kmax = -INFINITY;
     {
-      const int h = tid >> 7, rl = tid & (TR - 1);
+      // Every exponent s - ms is at most 0 (ms is the log of a sum that contains
+      // the row's own term), so the sum is taken unshifted; a row whose sum is
+      // tiny (below 1e-28, where flushed terms could matter) is taken again
+      // shifted by its largest exponent.
+      const int h = tid >> 7, rl = tid & 127;
       const int i0 = h * ((p.q + 1) / 2), i1 = h ? p.q : (p.q + 1) / 2;
-      for (int t0 = 0; t0 < mc; t0 += TR) {
+      for (int t0 = 0; t0 < mc; t0 += 128) {
         const int j = t0 + rl;
-        float mx = -INFINITY, z = 0.f;
+        float z = 0.f;
         if (j < mc) {
 #pragma unroll 8
-          for (int i = i0; i < i1; ++i) mx = fmaxf(mx, S[i * p.srow + j] - st.ms[i]);
-#pragma unroll 8
-          for (int i = i0; i < i1 && mx > -INFINITY; ++i) z += expf((S[i * p.srow + j] - st.ms[i]) - mx);
+          for (int i = i0; i < i1; ++i) z += expf(S[i * p.srow + j] - st.ms[i]);
         }
-        if (h) st.xch[rl] = make_float2(mx, z);
+        if (h) st.xch[rl] = z;
         __syncthreads();
         if (!h && j < mc) {
-          const float2 o = st.xch[rl];
-          const float M = fmaxf(mx, o.x);
-          const float key = M + logf((z > 0.f ? z * expf(mx - M) : 0.f) + (o.y > 0.f ? o.y * expf(o.x - M) : 0.f));
+          z += st.xch[rl];
+          float key = logf(z);
+          if (z < 1e-28f) {
+            float mx = -INFINITY;
+            for (int i = 0; i < p.q; ++i) mx = fmaxf(mx, S[i * p.srow + j] - st.ms[i]);
+            z = 0.f;
+            for (int i = 0; i < p.q && mx > -INFINITY; ++i) z += expf((S[i * p.srow + j] - st.ms[i]) - mx);
+            key = mx + logf(z);
+          }
           kmin = fminf(kmin, key);
           kmax = fmaxf(kmax, key);
           const uint32_t dst = smem_u32(J + g0 + j);
@@ -346,57 +399,44 @@ __global__ void __launch_bounds__(NTH, 1) wf_f32_kernel(const __grid_constant__ 
     for (int i = 0; i < QG; ++i)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
-    for (int t0 = 0; t0 < mc; t0 += TR) {
-      const int cnt = min(TR, mc - t0);
-      gather<D>(T0, t0, mc, krow);
-      cp_async_commit();
-      if (p.nbuf > 1) {
-        gather<D>(T1, t0, mc, vrow);
-        cp_async_commit();
-        cp_async_wait<1>();
-      } else {
-        cp_async_wait<0>();
-      }
+    // K and V tiles in the two halves of the row buffer; the next tile's K rows
+    // are copied under the softmax, its V rows under the next logits.
+    const int cap = min(p.trow / 8 * 4, p.srow - 4), tr = tile_rows(mc, cap);
+    float* T1 = T0 + cap * (D + 4);
+    gather<D>(T0, 0, min(tr, mc), krow);
+    cp_async_commit();
+    gather<D>(T1, 0, min(tr, mc), vrow);
+    cp_async_commit();
+    for (int t0 = 0; t0 < mc; t0 += tr) {
+      const int cnt = min(tr, mc - t0), pad = (cnt + 3) & ~3, nxt = min(tr, max(mc - t0 - tr, 0));
+      cp_async_wait<1>();  // K (V's copies are the newest group)
       __syncthreads();
       score_tile<D, QM>(Qs, T0, S, p.srow, 0, cnt, p.scale);
       __syncthreads();
-      if (p.nbuf == 1) {
-        gather<D>(T1, t0, mc, vrow);
-        cp_async_commit();
-      }
-      // P = exp(s - m) against the running max; keys past the tile get 0.
-      for (int i = warp; i < QM; i += NW) {
-        float* s = S + i * p.srow;
-        float mx = -INFINITY;
-        for (int j = lane; j < cnt; j += 32) mx = fmaxf(mx, s[j]);
-        const float mo = st.ms[i], mn = fmaxf(mo, warp_max_f32(mx));
-        float z = 0.f;
-        for (int j = lane; j < TR; j += 32) {
-          const float e = j < cnt ? expf(s[j] - mn) : 0.f;
-          s[j] = e;
-          z += e;
-        }
-        z = warp_sum(z);
+      gather<D>(T0, t0 + tr, nxt, krow);
+      cp_async_commit();
+      // P = exp(s - m) against the running max, zeros up to a multiple of 4 keys.
+      for (int i = 4 * warp; i < QM; i += 4 * NW) {
+        float mo[4], mx[4], z[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mx[k] = mo[k] = st.ms[i + k];
+        row_stats<true>(S + i * p.srow, p.srow, cnt, pad, mx, z);
         __syncwarp();
-        if (lane == 0) {
-          const float a = mo > -INFINITY ? expf(mo - mn) : 0.f;
-          st.alpha[i] = a;
-          st.ms[i] = mn;
-          st.l[i] = fmaf(st.l[i], a, z);
-        }
+        if (lane == 0)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float a = mo[k] > -INFINITY ? expf(mo[k] - mx[k]) : 0.f;
+            st.alpha[i + k] = a;
+            st.ms[i + k] = mx[k];
+            st.l[i + k] = fmaf(st.l[i + k], a, z[k]);
+          }
       }
-      // Rows past the tile are zero: P is 0 there, and the last tile's rows
-      // of the buffer may hold anything (infinities included).
-      for (int e = tid; e < (TR - cnt) * LPR; e += NTH)
-        if (p.nbuf > 1)
-          *reinterpret_cast<float4*>(T1 + (cnt + e / LPR) * (D + 4) + 4 * (e % LPR)) = make_float4(0.f, 0.f, 0.f, 0.f);
-      cp_async_wait<0>();
+      // The padding keys' V rows are zero: P is 0 there, and the buffer may
+      // hold anything (infinities included).
+      for (int e = tid; e < (pad - cnt) * LPR; e += NTH)
+        *reinterpret_cast<float4*>(T1 + (cnt + e / LPR) * (D + 4) + 4 * (e % LPR)) = make_float4(0.f, 0.f, 0.f, 0.f);
+      cp_async_wait<1>();  // V
       __syncthreads();
-      if (p.nbuf == 1) {
-        for (int e = tid; e < (TR - cnt) * LPR; e += NTH)
-          *reinterpret_cast<float4*>(T1 + (cnt + e / LPR) * (D + 4) + 4 * (e % LPR)) = make_float4(0.f, 0.f, 0.f, 0.f);
-        __syncthreads();
-      }
       if (t0 > 0) {
 #pragma unroll
         for (int i = 0; i < QG; ++i)
@@ -418,7 +458,10 @@ __global__ void __launch_bounds__(NTH, 1) wf_f32_kernel(const __grid_constant__ 
         }
       }
       __syncthreads();
+      gather<D>(T1, t0 + tr, nxt, vrow);
+      cp_async_commit();
     }
+    cp_async_wait_all();
     // The subsets' sums meet in the tile buffer: Op[query][channel].
     float* Op = T0;
     for (int k = NS - 1; k >= 0; --k) {
@@ -517,9 +560,9 @@ int resident_clusters(F32Kernel k, int cs, size_t smem) {
 
 // fp32, one query head per key head, candidate lists within the Top-K's 8192.
 // The largest cluster (up to 8) whose grid fits the SMs in one wave, all
-// clusters resident, and whose slice's logits fit shared memory; else the
-// smallest whose logits fit.
-F32Plan plan_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int num_sms) {
+// clusters resident, and whose slice's logits and at least 64 rows fit shared
+// memory; else the smallest whose logits fit.
+F32Plan plan_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g, int num_sms) {
   F32Plan fp{};
   if (kv.dtype != WF_F32 || q.heads != kv.heads || q.seq > kMaxQ || levels > 10) return fp;
   const int D = kv.head_dim, QM = q.seq <= 32 ? 32 : 64;
@@ -533,14 +576,16 @@ F32Plan plan_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int3
   const size_t kMaxSmem = 227 * 1024;
   const F32Kernel k = f32_kernel(D, q.seq);
   auto fit = [&](int cs) {
-    int rows = 2 * (((cmax + 1) / 2 + cs - 1) / cs);  // the widest slice
-    rows = rows > TR ? rows : TR;
-    fp.srow = (rows + 3) / 4 * 4 + 4;
-    for (fp.nbuf = 2; fp.nbuf >= 1; --fp.nbuf) {
-      fp.smem = f32_layout(D, QM, fp.nbuf, fp.srow, fp.bufw).total;
-      if (fp.smem <= kMaxSmem) return true;
-    }
-    return false;
+    // The widest slices of candidates and of keys; the row buffer takes all of
+    // the first, and the second's K and V, as far as there is room.
+    const int rows = 2 * (((cmax + 1) / 2 + cs - 1) / cs), keys = n_g < 0 ? 0 : (keep[0] + n_g + cs - 1) / cs;
+    const int want = std::max({rows, 2 * ((keys + 3) / 4 * 4), 64});
+    fp.srow = (std::max(rows, std::min(keys, 128)) + 3) / 4 * 4 + 4;
+    const size_t rest = f32_layout(D, QM, 0, fp.srow, fp.bufw).total, row = 4 * (size_t)(D + 4);
+    if (rest + 64 * row > kMaxSmem) return false;
+    fp.trow = std::min(want, (int)((kMaxSmem - rest) / row)) / 8 * 8;
+    fp.smem = f32_layout(D, QM, fp.trow, fp.srow, fp.bufw).total;
+    return true;
   };
   for (int cs = MAXCS; cs >= 1 && fp.cs == 0; --cs)
     if (U * cs <= num_sms && fit(cs) && U <= resident_clusters(k, cs, fp.smem)) fp.cs = cs;
@@ -576,7 +621,7 @@ cudaError_t launch_f32(const F32Plan& fp, const void* Q, const wf_tensor& qd, co
   p.q = qd.seq; p.n = kv.seq; p.ng = g ? g->seq : 0; p.H = kv.heads; p.L = levels;
   p.trim = fp.trim;
   p.attn = O != nullptr;
-  p.nbuf = fp.nbuf; p.srow = fp.srow; p.bufw = fp.bufw;
+  p.trow = fp.trow; p.srow = fp.srow; p.bufw = fp.bufw;
   for (int l = 0; l <= levels; ++l) p.keep[l] = keep[l];
   p.scale = 1.0f / sqrtf((float)kv.head_dim);
   const F32Kernel k = f32_kernel(kv.head_dim, qd.seq);

@@ -241,13 +241,14 @@ inline cudaError_t launch_gqa_filter(const GqaPlan& gp, const void* Q, const wf_
       gp, Q, qd, K, kv, coeffs, levels, keep, idx, level_sets, status, s);
 }
 
-// The fp32 step (one query head per key head): one cluster of cs CTAs a unit.
+// The fp32 step (one query head per key head): one cluster of cs CTAs a unit
+// (n_g as for plan_fused).
 struct F32Plan {
   bool ok, trim;
-  int U, cs, nbuf, srow, bufw;
+  int U, cs, trow, srow, bufw;
   size_t smem;
 };
-F32Plan plan_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int num_sms);
+F32Plan plan_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g, int num_sms);
 // O == nullptr: the filter alone.
 cudaError_t launch_f32(const F32Plan& fp, const void* Q, const wf_tensor& qd, const void* K, const void* V,
                        const wf_tensor& kv, const void* Kg, const void* Vg, const wf_tensor* g, const void* coeffs,
