@@ -388,16 +388,17 @@ __device__ __forceinline__ RowSrc attn_src(const Ctx& c, const FusedParams& p, i
 constexpr int LPR = D / 8;                       // lanes (16-byte chunks) a row
 constexpr int RSTEP = NPT / LPR;
 constexpr int RROWS = (TM + RSTEP - 1) / RSTEP;  // most rows of one thread
+static_assert(RSTEP * LPR <= TM && LPR <= RROWS, "a lane's first resolved row needs no clamp");
 static_assert(RSTEP % 2 == 0 && RROWS <= 2 * LPR, "4 swizzle terms and two resolved rows a lane cover a thread's rows");
 template <int KIND>
 __device__ __forceinline__ void load_share(uint32_t st, int t, const RowSrc& src, int pt) {
-  const int c = pt & (LPR - 1), r0 = pt / LPR, grp = pt & (32 - LPR);
+  const int c = pt & (LPR - 1), r0 = (int)((unsigned)pt / LPR), grp = pt & (32 - LPR);
   const uint32_t dbase = st + ((c >> 3) << 14) + (uint32_t)r0 * 128u;
   uint32_t xr[4];
 #pragma unroll
   for (int m = 0; m < 4; ++m) xr[m] = (uint32_t)((c ^ (r0 + RSTEP * m)) & 7) << 4;
-  // Rows j = c and j = LPR + c of these lanes (clamped into the tile).
-  const int ra = t * TM + min(r0 + RSTEP * min(c, RROWS - 1), TM - 1);
+  // Rows j = c and j = LPR + c of these lanes (the second clamped into the tile).
+  const int ra = t * TM + r0 + RSTEP * c;
   const int rb = t * TM + min(r0 + RSTEP * min(LPR + c, RROWS - 1), TM - 1);
   if (KIND <= 1) {
     const char* cb = reinterpret_cast<const char*>(src.base) + c * 16;

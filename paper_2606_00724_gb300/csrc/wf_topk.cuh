@@ -186,12 +186,14 @@ __device__ __forceinline__ uint3 warp_boundary(uint32_t hist_a, uint32_t need, i
 // every warp then finds the bucket holding the boundary from the counts: keys
 // above it are taken, keys below it dropped.  A boundary bucket of at most
 // as many keys as the unit has threads is resolved exactly: its keys go to a
-// list, and each is ranked on (key, -position) against the whole list, by its
-// owner (one warpgroup) or by the list entry's thread, which marks a winner in
-// its owner's position mask (both warpgroups: measured 116.9 -> 110.6 us at
-// 128K, while one warpgroup ran slower that way).  A larger bucket is
-// bucketed again over its own range.  If only equal keys remain, the lowest
-// positions are taken.
+// list and are ranked on (key, -position) against the whole list.  Up to 32
+// keys (the common case: a few), every warp does that by itself with an entry
+// a lane and the owners take their winners from the lanes, with no further
+// barrier; more are ranked by their owners (one warpgroup) or by the list
+// entries' threads, which mark winners in the owners' position masks (both
+// warpgroups: measured 116.9 -> 110.6 us at 128K, while one warpgroup ran
+// slower that way).  A larger bucket is bucketed again over its own range.
+// If only equal keys remain, the lowest positions are taken.
 template <typename MT, bool WIDE>
 __device__ __noinline__ void select_keys(uint32_t keys_a, int m, int kk, uint32_t jprev_a, int top, uint32_t sc_a,
                                          float lo, float hi, int R) {
@@ -211,6 +213,27 @@ __device__ __noinline__ void select_keys(uint32_t keys_a, int m, int kk, uint32_
     const uint4 v = lds_v4(keys_a + 4u * min((uint32_t)(j0 + 4 * g), m4 - 4u));
     return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
   };
+  // body(g, keys of group g) for every group of the run, up to four groups'
+  // loads in flight (shared-memory accesses keep their order, so a load issued
+  // between another group's updates would be waited for by itself).
+  auto for_groups = [&](auto&& body) {
+    if (G < 4) {
+#pragma unroll 1
+      for (int gg = 0; gg < G; ++gg) {
+        const int g = (gg + rotg) & (G - 1);
+        body(g, group(g));
+      }
+      return;
+    }
+#pragma unroll 1
+    for (int g4 = 0; g4 < G; g4 += 4) {
+      float4 v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = group((g4 + k + rotg) & (G - 1));
+#pragma unroll
+      for (int k = 0; k < 4; ++k) body((g4 + k + rotg) & (G - 1), v[k]);
+    }
+  };
   const uint32_t hist_a = SC_ADDR(sc_a, hist);
   const uint32_t own_a = hist_a + 4u * (uint32_t)(BPT * tid);  // the buckets this thread clears
   uint32_t need = (uint32_t)kk;
@@ -219,10 +242,7 @@ __device__ __noinline__ void select_keys(uint32_t keys_a, int m, int kk, uint32_
   for (int iter = 0; iter < 6; ++iter) {
     if (!(hi > lo)) break;  // every undecided key is equal (or none is left)
     const float scale = (float)NB / (hi - lo);
-#pragma unroll 4
-    for (int gg = 0; gg < G; ++gg) {
-      const int g = (gg + rotg) & (G - 1);
-      const float4 v = group(g);
+    for_groups([&](int g, const float4& v) {
       const uint32_t a4 = (uint32_t)(act >> (4 * g));
       const int b0 = bucket_of(v.x, lo, scale), b1 = bucket_of(v.y, lo, scale);
       const int b2 = bucket_of(v.z, lo, scale), b3 = bucket_of(v.w, lo, scale);
@@ -230,16 +250,13 @@ __device__ __noinline__ void select_keys(uint32_t keys_a, int m, int kk, uint32_
       reds_add_if(a4 & 2u, hist_a + 4u * b1, 1u);
       reds_add_if(a4 & 4u, hist_a + 4u * b2, 1u);
       reds_add_if(a4 & 8u, hist_a + 4u * b3, 1u);
-    }
+    });
     csync<WIDE>();
     const uint3 bd = warp_boundary(hist_a, need, lane);
     const int sb = (int)bd.x;
     need = bd.y;
     const uint32_t cnt = bd.z;
-#pragma unroll 4
-    for (int gg = 0; gg < G; ++gg) {
-      const int g = (gg + rotg) & (G - 1);
-      const float4 v = group(g);
+    for_groups([&](int g, const float4& v) {
       const int bk[4] = {bucket_of(v.x, lo, scale), bucket_of(v.y, lo, scale), bucket_of(v.z, lo, scale),
                          bucket_of(v.w, lo, scale)};
 #pragma unroll
@@ -248,7 +265,7 @@ __device__ __noinline__ void select_keys(uint32_t keys_a, int m, int kk, uint32_
         took |= bk[e] > sb ? bit : (MT)0;
         act &= bk[e] != sb ? ~bit : ~(MT)0;
       }
-    }
+    });
     if (cnt == need) {
       took |= act;
       act = 0;
@@ -256,28 +273,41 @@ __device__ __noinline__ void select_keys(uint32_t keys_a, int m, int kk, uint32_
       break;
     }
     if (cnt <= (uint32_t)TN) {
-      // Append the boundary keys (one atomic per warp), then every owner
-      // ranks its own keys against the list.
-      const int nb = popc_m(act);
-      int incl = nb;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      uint32_t wbase = 0;
-      if (lane == 31 && incl > 0) wbase = atoms_add(SC_ADDR(sc_a, bcnt), (uint32_t)incl);
-      wbase = __shfl_sync(0xffffffffu, wbase, 31);
-      uint32_t slot = wbase + (uint32_t)(incl - nb);
+      // Append the boundary keys, one atomic each: there are few, and their
+      // order in the list does not matter.
 #pragma unroll 1
-      for (MT a = act; a; a &= a - 1, ++slot) {
+      for (MT a = act; a; a &= a - 1) {
         const int i = ffs_m(a) - 1;
+        const uint32_t key = lds_u32(keys_a + 4u * (uint32_t)(j0 + i));
+        const uint32_t slot = atoms_add(SC_ADDR(sc_a, bcnt), 1u);
         // slot < TN always (the list holds cnt <= TN keys); the predicate
         // keeps the store in the list should a wait have given up.
-        sts_v2_if(slot < (uint32_t)TN, SC_ADDR(sc_a, blist) + 8u * slot, lds_u32(keys_a + 4u * (uint32_t)(j0 + i)),
-                  (uint32_t)(j0 + i));
+        sts_v2_if(slot < (uint32_t)TN, SC_ADDR(sc_a, blist) + 8u * slot, key, (uint32_t)(j0 + i));
       }
       csync<WIDE>();
+      if (cnt <= 32u) {
+        // Every warp ranks the whole list by itself, entry l on lane l, on
+        // (key, -position); the owners then take their winners from the lanes.
+        const uint2 me = lds_v2(SC_ADDR(sc_a, blist) + 8u * min((uint32_t)lane, cnt - 1));
+        const float kx = __uint_as_float(me.x);
+        const int jx = (int)me.y;
+        uint32_t rank = 0;
+#pragma unroll 4
+        for (int v = 0; v < (int)cnt; ++v) {
+          const float ko = __shfl_sync(0xffffffffu, kx, v);
+          const int jo = __shfl_sync(0xffffffffu, jx, v);
+          rank += (ko > kx) || (ko == kx && jo < jx);
+        }
+        const bool win = (uint32_t)lane < cnt && rank < need;
+#pragma unroll 1
+        for (uint32_t w = __ballot_sync(0xffffffffu, win); w; w &= w - 1) {
+          const int off = __shfl_sync(0xffffffffu, jx, __ffs(w) - 1) - j0;
+          took |= (uint32_t)off < (uint32_t)R ? (MT)1 << off : (MT)0;
+        }
+        act = 0;
+        resolved = true;
+        break;
+      }
       if (!WIDE) {
         // Every owner ranks its own boundary keys on (key, -position)
         // against the list (measured faster with one warpgroup).
@@ -369,31 +399,39 @@ __device__ __noinline__ void select_keys(uint32_t keys_a, int m, int kk, uint32_
   // of the keys, the histogram and the boundary list before the key array is
   // overwritten and the scratch cleared.
   int r = cta_excl_scan<WIDE>(popc_m(take), SC_ADDR(sc_a, wsum) + 64u);
+  // (Four groups a turn, so that their entries of the previous selection load
+  // together; a run shorter than that has entries of its last group repeated.)
 #pragma unroll 1
-  for (int g = 0; g < G; ++g) {
-    const uint32_t t4 = (uint32_t)(take >> (4 * g)) & 15u;
-    if (!t4) continue;
-    const int j = j0 + 4 * g;
-    int c[4] = {j, j + 1, j + 2, j + 3};
-    if (!top) {
-      const uint2 pj = lds_v2(jprev_a + 4u * (uint32_t)(j >> 1));
-      c[0] = 2 * (int)pj.x;
-      c[1] = 2 * (int)pj.x + 1;
-      c[2] = 2 * (int)pj.y;
-      c[3] = 2 * (int)pj.y + 1;
+  for (int g4 = 0; g4 < G; g4 += 4) {
+    uint2 pj[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int j = j0 + 4 * min(g4 + k, G - 1);
+      // Entries past the previous selection (positions past m) are not used;
+      // the clamp keeps the load in the array.
+      pj[k] = top ? make_uint2(0u, 0u) : lds_v2(jprev_a + 4u * min((uint32_t)(j >> 1), (m4 >> 1) - 2u));
     }
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      // r < kk <= m always; the bound keeps the store in the array should a
-      // wait have given up.
-      sts_u32_if(((t4 >> e) & 1u) && (uint32_t)r < (uint32_t)m, keys_a + 4u * (uint32_t)r, (uint32_t)c[e]);
-      r += (t4 >> e) & 1u;
+    for (int k = 0; k < 4; ++k) {
+      const int j = j0 + 4 * (g4 + k);
+      const uint32_t t4 = g4 + k < G ? (uint32_t)(take >> (4 * (g4 + k))) & 15u : 0u;
+      const int c[4] = {top ? j : 2 * (int)pj[k].x, top ? j + 1 : 2 * (int)pj[k].x + 1, top ? j + 2 : 2 * (int)pj[k].y,
+                        top ? j + 3 : 2 * (int)pj[k].y + 1};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        // r < kk <= m always; the bound keeps the store in the array should a
+        // wait have given up.
+        sts_u32_if(((t4 >> e) & 1u) && (uint32_t)r < (uint32_t)m, keys_a + 4u * (uint32_t)r, (uint32_t)c[e]);
+        r += (t4 >> e) & 1u;
+      }
     }
   }
+  csync<WIDE>();
+  // The scratch is cleared after the selection's last barrier: nothing uses it
+  // again before another barrier of these threads.
 #pragma unroll
   for (int i = 0; i < BPT / 4; ++i) sts_v4(own_a + 16u * i, make_uint4(0, 0, 0, 0));
   if (tid == 0) sts_u32(SC_ADDR(sc_a, bcnt), 0u);
-  csync<WIDE>();
 }
 
 // Top-K dispatch: R = the smallest power of two (at least 4) with R TN >= m
