@@ -10,9 +10,13 @@
 #include <math.h>
 
 #include "wf_internal.cuh"
+#include "wf_sm100.cuh"
 
 namespace wf {
 namespace {
+
+using sm100::grid_dep_launch;
+using sm100::grid_dep_wait;
 
 constexpr int CH = kAttnChunk;
 constexpr int QMAX = kMaxQ;
@@ -148,6 +152,8 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const float* __restri
                                                            int qstride, T* __restrict__ O, int64_t osb, int64_t osh,
                                                            int64_t oss) {
   constexpr int CPL = D / 32;
+  grid_dep_wait();
+  grid_dep_launch();
   const int u = blockIdx.x;
   const int i = blockIdx.y * 8 + (threadIdx.x >> 5);  // query row of this warp
   if (i >= q) return;
@@ -188,13 +194,8 @@ cudaError_t combine(const AttnPlan& p, int nsplit, void* O, const wf_tensor& od,
   float* Opart = reinterpret_cast<float*>(static_cast<char*>(ws) + p.off_o);
   float2* ML = reinterpret_cast<float2*>(static_cast<char*>(ws) + p.off_ml);
   const dim3 grid((unsigned)p.U, (unsigned)((p.q + 7) / 8));
-  if (p.d == 128)
-    attn_combine_kernel<T, 128><<<grid, 256, 0, s>>>(Opart, ML, nsplit, p.q, p.H, p.qstride, static_cast<T*>(O),
-                                                     od.stride_b, od.stride_h, od.stride_s);
-  else
-    attn_combine_kernel<T, 64><<<grid, 256, 0, s>>>(Opart, ML, nsplit, p.q, p.H, p.qstride, static_cast<T*>(O),
-                                                    od.stride_b, od.stride_h, od.stride_s);
-  return cudaGetLastError();
+  return Launch(grid, 256, 0, s)(p.d == 128 ? attn_combine_kernel<T, 128> : attn_combine_kernel<T, 64>, Opart, ML, nsplit,
+                                 p.q, p.H, p.qstride, static_cast<T*>(O), od.stride_b, od.stride_h, od.stride_s);
 }
 
 template <typename T, int D, int QM>

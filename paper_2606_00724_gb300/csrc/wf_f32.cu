@@ -226,6 +226,8 @@ __global__ void __launch_bounds__(NTH, 1) wf_f32_kernel(const __grid_constant__ 
   const int64_t bb = u / p.H, hh = u % p.H;
   auto buf = [&](int lev) { return reinterpret_cast<int32_t*>(smem + ly.buf) + ((p.L - lev) & 1) * p.bufw; };
 
+  grid_dep_wait();
+  grid_dep_launch();
   // The query block (rows past q zero) with the first tile's copies; the
   // Top-K scratch starts zeroed.
   for (int e = tid; e < QM * (D / 4); e += NTH) {
@@ -519,19 +521,6 @@ F32Kernel f32_kernel(int d, int q) {
   return q <= 32 ? wf_f32_kernel<128, 32> : wf_f32_kernel<128, 64>;
 }
 
-void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, int clusters, int cs, size_t smem) {
-  cfg = cudaLaunchConfig_t{};
-  cfg.gridDim = dim3((unsigned)(clusters * cs), 1, 1);
-  cfg.blockDim = dim3(NTH, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = (unsigned)cs;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-}
-
 // Clusters of cs CTAs that can be resident at once; cached per configuration.
 int resident_clusters(F32Kernel k, int cs, size_t smem) {
   static std::mutex mu;
@@ -542,12 +531,10 @@ int resident_clusters(F32Kernel k, int cs, size_t smem) {
   std::lock_guard<std::mutex> lock(mu);
   auto it = cache.find(key);
   if (it != cache.end()) return it->second;
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr;
-  cluster_config(cfg, attr, 1, cs, smem);
+  Launch one(dim3((unsigned)cs), NTH, smem, nullptr, cs);
   int n = 0;
   cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(k), smem);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k, &one.cfg);
   if (e != cudaSuccess) {
     (void)cudaGetLastError();
     n = 0;
@@ -627,13 +614,7 @@ cudaError_t launch_f32(const F32Plan& fp, const void* Q, const wf_tensor& qd, co
   const F32Kernel k = f32_kernel(kv.head_dim, qd.seq);
   cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(k), fp.smem);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr;
-  cluster_config(cfg, attr, fp.U, fp.cs, fp.smem);
-  cfg.stream = s;
-  e = cudaLaunchKernelEx(&cfg, k, p);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return Launch(dim3((unsigned)(fp.U * fp.cs)), NTH, fp.smem, s, fp.cs)(k, p);
 }
 
 }  // namespace wf

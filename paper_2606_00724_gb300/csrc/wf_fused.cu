@@ -30,9 +30,9 @@
 //
 // A launch may also run part of the chain (a range of scales, the previous
 // selection handed in, the last one handed out, the attention optional): the
-// literal-basis path runs one launch per scale, each a programmatic dependent
-// of the kernel before it (every thread waits for that grid before its first
-// global access).
+// literal-basis path runs one launch per scale.  Launches are programmatic
+// dependents of the kernel before them (every thread waits for that grid
+// before its first global access).
 //
 // Every wait is bounded (~1 s): on timeout the CTA records a status word,
 // stops issuing MMAs and skips the remaining waits, so every thread reaches
@@ -1954,6 +1954,7 @@ __global__ void __launch_bounds__(NT, 1) wf_gqa_filter_kernel(const __grid_const
   __syncthreads();
   if (warp > MMA_WARP) {
     cluster_arrive_relaxed();
+    grid_dep_wait();
     gqa_producer_role<S>(c, p);
     cluster_wait();
   } else {
@@ -1970,6 +1971,8 @@ __global__ void __launch_bounds__(NT, 1) wf_gqa_filter_kernel(const __grid_const
     // The Top-K scratch starts zeroed (histogram, list counter, masks).
     for (int e = tid; e < (int)((sizeof(SelScratch) + 15) / 16); e += NS)
       *reinterpret_cast<uint4*>(smem + gl.sc + 16 * e) = make_uint4(0, 0, 0, 0);
+    grid_dep_wait();
+    grid_dep_launch();
     tc_fence_before();
     named_sync(kSetupSyncId, NS);
     tc_fence_after();
@@ -2222,25 +2225,10 @@ cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd
     p.attn = 1;
   }
 
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(fp.clusters * fp.cs), 1, 1);
-  cfg.blockDim = dim3(NT, 1, 1);
-  cfg.dynamicSmemBytes = fp.smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = fp.cs;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = range && range->pdl ? 2 : 1;
-  cudaError_t e = ensure_smem_limit(fp.stages, fp.wide, cfg.dynamicSmemBytes);
+  cudaError_t e = ensure_smem_limit(fp.stages, fp.wide, fp.smem);
   if (e != cudaSuccess) return e;
-  e = cudaLaunchKernelEx(&cfg, fused_kernel(fp.stages, fp.wide), p);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return Launch(dim3((unsigned)(fp.clusters * fp.cs)), NT, fp.smem, s, fp.cs,
+                range && range->plain)(fused_kernel(fp.stages, fp.wide), p);
 }
 
 // The grouped filter (wf_gqa_filter_kernel): bf16, at most 256 stacked
@@ -2370,24 +2358,10 @@ cudaError_t launch_gqa_filter(const GqaPlan& gp, const void* Q, const wf_tensor&
   p.final_sel = 1;
   p.G = gp.G;
   p.nch = gp.nch;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(gp.U * gp.cs), 1, 1);
-  cfg.blockDim = dim3(NT, 1, 1);
-  cfg.dynamicSmemBytes = gp.smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = gp.cs;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   const GqaKernel k = gqa_kernel(gp.stages);
   cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(k), gp.smem);
   if (e != cudaSuccess) return e;
-  e = cudaLaunchKernelEx(&cfg, k, p);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return Launch(dim3((unsigned)(gp.U * gp.cs)), NT, gp.smem, s, gp.cs)(k, p);
 }
 
 cudaError_t launch_literal_fused(const FusedPlan& fp, const FilterPlan& fl, const void* Q, const wf_tensor& qd,
@@ -2404,11 +2378,11 @@ cudaError_t launch_literal_fused(const FusedPlan& fp, const FilterPlan& fl, cons
   for (int l = L; l >= 1; --l) {
     // Scale l's rows: the whole prompt's scale-L rows at the top, else the
     // transform of the candidates' gathered blocks, in candidate order.
-    if (l < L && (e = launch_wavelet_approx(K, kv, cur, fl.cmax, m, l, wavelet, arows, (int64_t)fl.cmax * D, s,
-                                            true)) != cudaSuccess)
+    if (l < L && (e = launch_wavelet_approx(K, kv, cur, fl.cmax, m, l, wavelet, arows, (int64_t)fl.cmax * D,
+                                            s)) != cudaSuccess)
       return e;
     FusedRange r{};
-    r.pdl = l < L;  // every launch after the first follows one of this pipeline's own
+    r.plain = l == L;  // every launch after the first follows one of this pipeline's own
     r.lev_top = l;
     r.lev_bot = (l == 1 && fl.trim) ? 0 : l;
     r.final_sel = l == 1;

@@ -100,10 +100,8 @@ cudaError_t launch_tc_skim(const FilterPlan& p, const void* Q, const wf_tensor& 
 // WF_WAVELET_*) of the keys of blocks [2^level c, 2^level (c + 1)) for the m
 // candidates c of every unit (cand: [units][cand_stride], NULL = all blocks),
 // into out[unit * out_unit + j * head_dim + channel] in the key dtype.
-// pdl: launch as a programmatic dependent of the previous kernel on the stream.
 cudaError_t launch_wavelet_approx(const void* K, const wf_tensor& kv, const int32_t* cand, int64_t cand_stride, int m,
-                                  int level, int wavelet, void* out, int64_t out_unit, cudaStream_t s,
-                                  bool pdl = false);
+                                  int level, int wavelet, void* out, int64_t out_unit, cudaStream_t s);
 int wavelet_taps(int wavelet);       // 0 for an unknown basis
 int wavelet_max_level(int wavelet);  // deepest scale the approximation kernel supports
 // Filtering with a generic basis (Eq. 11 taken literally): the filter plan's
@@ -153,10 +151,9 @@ struct FusedPlan {
 // jout unless final_sel (then mu^0 goes to idx); the attention if attn.
 // Scale lev_top's rows come from lrows ([units][m][d], unit stride lrows_unit
 // elements) when not null, else from the pyramid (only when lev_top = L).
-// pdl: launch as a programmatic dependent of the previous kernel on the
-// stream (its set-up overlaps that kernel's tail).
+// plain: not as a programmatic dependent of the kernel before (see Launch).
 struct FusedRange {
-  int lev_top, lev_bot, final_sel, attn, pdl;
+  int lev_top, lev_bot, final_sel, attn, plain;
   const int32_t* jin;
   int32_t* jout;
   int64_t jstride;
@@ -263,6 +260,42 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 cudaError_t raise_smem_limit(const void* kernel, size_t smem);
 // The current device's SM count, looked up once per device (0 on an error).
 int sm_count();
+
+// A launch as a programmatic dependent of the kernel before it on the stream
+// (of clusters of `cluster` CTAs if that is not 0).  The kernel's CTAs are
+// placed as that kernel's leave, so its launch and set-up hide in the other's
+// tail; every kernel launched this way executes grid_dep_wait before its first
+// access to global memory, so it still starts after everything before it on
+// the stream, and grid_dep_launch to let the next one in.  Back-to-back steps:
+// 32 heads x 8K tokens 54.8 -> 53.3 us, 128K 93.4 -> 91.2; a filter and its
+// attention at 20K 65.5 -> 59.7.  The pyramid build stays an ordinary kernel
+// (`plain`): its 16,000 short CTAs slowed down with the two instructions, 391
+// against 425 us for a build and a step.
+struct Launch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[2];
+  Launch(dim3 grid, int threads, size_t smem, cudaStream_t s, int cluster = 0, bool plain = false) {
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = plain ? 0 : 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster ? 2 : 1;
+  }
+  Launch(const Launch&) = delete;
+  Launch& operator=(const Launch&) = delete;
+  template <typename... P, typename... A>
+  cudaError_t operator()(void (*kernel)(P...), const A&... args) {
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    return e != cudaSuccess ? e : cudaGetLastError();
+  }
+};
 
 // Bounds of the tensor-core kernels' waits.  The default, about one second of
 // SM clock cycles, can be lowered (and a stalled first wait requested) only

@@ -436,6 +436,8 @@ __global__ void __launch_bounds__(NTH, 2) tc_attn_kernel(const __grid_constant__
     mbar_init(smem_u32(&bar[2]), 1);
     fence_mbar_init();
   }
+  grid_dep_wait();
+  grid_dep_launch();
   for (int e = tid; e < 256; e += NTA) {
     cm[e] = -INFINITY;
     cl[e] = 0.f;
@@ -729,6 +731,8 @@ __global__ void __launch_bounds__(NTH, 1) tc_attn_rows_kernel(const __grid_const
     mbar_init(smem_u32(&bar[2]), 1);
     fence_mbar_init();
   }
+  grid_dep_wait();
+  grid_dep_launch();
   for (int e = tid; e < nmt * 128 * (D / 8); e += NTH) {
     const int rr = e & 7, ch = (e >> 3) & (D / 8 - 1), g = e >> 7;
     const int i = g * 8 + rr;
@@ -974,7 +978,6 @@ cudaError_t launch_tc_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd
     while (a.tps < tiles && units * ((tiles + a.tps - 1) / a.tps) > (int64_t)occ * sms) ++a.tps;
     a.nsplit = (tiles + a.tps - 1) / a.tps;
   };
-  const dim3 block(NTH);
   cudaError_t e;
   if (a.q > 32) {
     // Query rows on the TMEM lanes: one or two M tiles of 128 rows; S and O
@@ -985,7 +988,7 @@ cudaError_t launch_tc_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd
     const size_t smem = tc_attn_rows_smem(nmt);
     split(1);
     if ((e = raise_smem_limit(reinterpret_cast<const void*>(tc_attn_rows_kernel), smem)) != cudaSuccess) return e;
-    tc_attn_rows_kernel<<<dim3((unsigned)a.nsplit, (unsigned)units, 1), block, smem, s>>>(a);
+    e = Launch(dim3((unsigned)a.nsplit, (unsigned)units), NTH, smem, s)(tc_attn_rows_kernel, a);
   } else {
     // Keys on the TMEM lanes, one chunk of 32 query columns: S^T and O^T take
     // 64 TMEM columns; shared memory and registers hold two CTAs an SM.
@@ -994,10 +997,10 @@ cudaError_t launch_tc_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd
     const size_t smem = tc_attn_smem(a.nq);
     split(2);
     if ((e = raise_smem_limit(reinterpret_cast<const void*>(tc_attn_kernel), smem)) != cudaSuccess) return e;
-    tc_attn_kernel<<<dim3((unsigned)a.nsplit, (unsigned)units, 1), block, smem, s>>>(a);
+    e = Launch(dim3((unsigned)a.nsplit, (unsigned)units), NTH, smem, s)(tc_attn_kernel, a);
   }
   *nsplit_out = a.nsplit;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace wf

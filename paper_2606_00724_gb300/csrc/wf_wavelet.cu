@@ -443,25 +443,15 @@ inline int stream_run(int64_t units, int m, int lpr, int ctas) {
 
 template <typename T, int TAPS, int L, int D>
 cudaError_t run_stream(const void* K, const wf_tensor& kv, const int32_t* cand, int64_t cand_stride, int m,
-                       const Taps& taps, void* out, int64_t out_unit, cudaStream_t s, bool pdl) {
+                       const Taps& taps, void* out, int64_t out_unit, cudaStream_t s) {
   constexpr int LPR = D / Vec<T>::N;
   const int64_t units = (int64_t)kv.batch * kv.heads;
   const int run = stream_run(units, m, LPR, stream_ctas<T, TAPS, L>());
   const int64_t threads = (int64_t)((m + run - 1) / run) * LPR;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)((threads + kStreamThreads - 1) / kStreamThreads), (unsigned)units, 1);
-  cfg.blockDim = dim3(kStreamThreads, 1, 1);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, approx_stream_kernel<T, TAPS, L, D>, static_cast<const T*>(K), kv.stride_b,
-                                     kv.stride_h, kv.stride_s, (int64_t)kv.seq, make_fastdiv((uint32_t)kv.heads), cand,
-                                     cand_stride, m, run, taps, static_cast<T*>(out), out_unit);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return Launch(dim3((unsigned)((threads + kStreamThreads - 1) / kStreamThreads), (unsigned)units), kStreamThreads, 0,
+                s)(approx_stream_kernel<T, TAPS, L, D>, static_cast<const T*>(K), kv.stride_b, kv.stride_h, kv.stride_s,
+                   (int64_t)kv.seq, make_fastdiv((uint32_t)kv.heads), cand, cand_stride, m, run, taps,
+                   static_cast<T*>(out), out_unit);
 }
 
 // Shared memory of one CTA for DS channels: the raw rows, the first fp32
@@ -475,7 +465,7 @@ size_t approx_smem(int level, int ds) {
 
 template <typename T, int TAPS, int DS>
 cudaError_t run_ds(const void* K, const wf_tensor& kv, const int32_t* cand, int64_t cand_stride, int m, int level,
-                   const Taps& taps, void* out, int64_t out_unit, cudaStream_t s, bool pdl) {
+                   const Taps& taps, void* out, int64_t out_unit, cudaStream_t s) {
   const int to = outputs_per_cta(level);
   const size_t smem = approx_smem<T, TAPS>(level, DS);
   // The shared-memory limit, raised per device to the largest size requested
@@ -494,21 +484,10 @@ cudaError_t run_ds(const void* K, const wf_tensor& kv, const int32_t* cand, int6
       cur = smem;
     }
   }
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(kv.head_dim / DS), (unsigned)((m + to - 1) / to), (unsigned)(kv.batch * kv.heads));
-  cfg.blockDim = dim3(NTH, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  e = cudaLaunchKernelEx(&cfg, approx_kernel<T, TAPS, DS>, static_cast<const T*>(K), kv.stride_b, kv.stride_h,
-                         kv.stride_s, (int64_t)kv.seq, make_fastdiv((uint32_t)kv.heads), cand, cand_stride, m, level,
-                         taps, static_cast<T*>(out), out_unit, (int64_t)kv.head_dim);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return Launch(dim3((unsigned)(kv.head_dim / DS), (unsigned)((m + to - 1) / to), (unsigned)(kv.batch * kv.heads)), NTH,
+                smem, s)(approx_kernel<T, TAPS, DS>, static_cast<const T*>(K), kv.stride_b, kv.stride_h, kv.stride_s,
+                         (int64_t)kv.seq, make_fastdiv((uint32_t)kv.heads), cand, cand_stride, m, level, taps,
+                         static_cast<T*>(out), out_unit, (int64_t)kv.head_dim);
 }
 
 // Scales above kStreamMaxLevel: whole rows of 128 channels per CTA (each row's
@@ -516,27 +495,27 @@ cudaError_t run_ds(const void* K, const wf_tensor& kv, const int32_t* cand, int6
 // allows, else 64 channels, else 16 (the deepest scales).
 template <typename T, int TAPS, int D>
 cudaError_t run_d(const void* K, const wf_tensor& kv, const int32_t* cand, int64_t cand_stride, int m, int level,
-                  const Taps& taps, void* out, int64_t out_unit, cudaStream_t s, bool pdl) {
+                  const Taps& taps, void* out, int64_t out_unit, cudaStream_t s) {
   switch (level) {
-    case 1: return run_stream<T, TAPS, 1, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s, pdl);
-    case 2: return run_stream<T, TAPS, 2, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s, pdl);
-    case 3: return run_stream<T, TAPS, 3, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s, pdl);
-    case 4: return run_stream<T, TAPS, 4, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s, pdl);
-    default: return run_stream<T, TAPS, 5, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s, pdl);
+    case 1: return run_stream<T, TAPS, 1, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s);
+    case 2: return run_stream<T, TAPS, 2, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s);
+    case 3: return run_stream<T, TAPS, 3, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s);
+    case 4: return run_stream<T, TAPS, 4, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s);
+    default: return run_stream<T, TAPS, 5, D>(K, kv, cand, cand_stride, m, taps, out, out_unit, s);
   }
 }
 
 template <typename T, int TAPS>
 cudaError_t run(const void* K, const wf_tensor& kv, const int32_t* cand, int64_t cand_stride, int m, int level,
-                const Taps& taps, void* out, int64_t out_unit, cudaStream_t s, bool pdl) {
+                const Taps& taps, void* out, int64_t out_unit, cudaStream_t s) {
   if (level <= kStreamMaxLevel && kv.batch * kv.heads <= 65535)
-    return kv.head_dim == 64 ? run_d<T, TAPS, 64>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl)
-                             : run_d<T, TAPS, 128>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl);
+    return kv.head_dim == 64 ? run_d<T, TAPS, 64>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s)
+                             : run_d<T, TAPS, 128>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s);
   if (kv.head_dim == 128 && approx_smem<T, TAPS>(level, 128) <= 200 * 1024)
-    return run_ds<T, TAPS, 128>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl);
+    return run_ds<T, TAPS, 128>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s);
   if (approx_smem<T, TAPS>(level, 64) <= 200 * 1024)
-    return run_ds<T, TAPS, 64>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl);
-  return run_ds<T, TAPS, 16>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl);
+    return run_ds<T, TAPS, 64>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s);
+  return run_ds<T, TAPS, 16>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s);
 }
 
 }  // namespace
@@ -546,18 +525,18 @@ int wavelet_taps(int wavelet) { return wavelet == WF_WAVELET_HAAR ? 2 : (wavelet
 int wavelet_max_level(int wavelet) { return wavelet == WF_WAVELET_DB2 ? 8 : 10; }
 
 cudaError_t launch_wavelet_approx(const void* K, const wf_tensor& kv, const int32_t* cand, int64_t cand_stride, int m,
-                                  int level, int wavelet, void* out, int64_t out_unit, cudaStream_t s, bool pdl) {
+                                  int level, int wavelet, void* out, int64_t out_unit, cudaStream_t s) {
   Taps taps{};
   if (wavelet == WF_WAVELET_DB2) {
     // Daubechies' two-vanishing-moment scaling filter, from its closed form.
     const double r = sqrt(3.0), q = 4.0 * sqrt(2.0);
     const double h[4] = {(1.0 + r) / q, (3.0 + r) / q, (3.0 - r) / q, (1.0 - r) / q};
     for (int k = 0; k < 4; ++k) taps.h[k] = (float)h[k];
-    return kv.dtype == WF_BF16 ? run<bf16, 4>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl)
-                               : run<float, 4>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl);
+    return kv.dtype == WF_BF16 ? run<bf16, 4>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s)
+                               : run<float, 4>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s);
   }
-  return kv.dtype == WF_BF16 ? run<bf16, 2>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl)
-                             : run<float, 2>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s, pdl);
+  return kv.dtype == WF_BF16 ? run<bf16, 2>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s)
+                             : run<float, 2>(K, kv, cand, cand_stride, m, level, taps, out, out_unit, s);
 }
 
 }  // namespace wf
