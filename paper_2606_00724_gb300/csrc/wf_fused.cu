@@ -1095,6 +1095,10 @@ __device__ __noinline__ void attn_online(Misc& ms, int* status, float sl2, uint8
   csync<WIDE>();
 }
 
+// Rows of a query group in the combine buffer for a slice of `rows`: one of
+// padding, against bank conflicts, where the buffer has the room.
+__device__ __forceinline__ int comb_rows(int rows, int cs) { return rows + ((rows + 1) * cs <= D + MAXCS ? 1 : 0); }
+
 // Attention combine of unit pp: this CTA's partial O^T rows go to the CTA
 // owning their head-dim slice (with the CTA's (m, l) per query), and this
 // CTA combines the cluster's partials of its own slice and writes those
@@ -1125,10 +1129,16 @@ __device__ __noinline__ void attn_combine(Misc& ms, const FusedParams& p, uint32
     while (owner + 1 < (int)cs && dlo(owner + 1, cs) <= tid) ++owner;
     const int orows = dlo(owner + 1, cs) - dlo(owner, cs);
     const int dl = tid - dlo(owner, cs);
-    const uint32_t dst = map_rank(comb_a + 4u * (uint32_t)(((int)rank * orows + dl) * NQ), (uint32_t)owner);
+    // Four queries a store, at [source][query / 4][row] (comb_rows a group): the
+    // lanes of a warp hold consecutive rows, so each store of theirs
+    // covers consecutive addresses, and the owner's reads (a lane a query) hit
+    // distinct banks.
+    const uint32_t step = 16u * (uint32_t)comb_rows(orows, (int)cs);
+    const uint32_t dst = map_rank(comb_a + 8u * rank * step + 16u * (uint32_t)dl, (uint32_t)owner);
     const uint32_t rb = map_rank(cbar, (uint32_t)owner);
 #pragma unroll
-    for (int i = 0; i < 32; i += 4) st_async_v4(dst + 4u * i, orow[i], orow[i + 1], orow[i + 2], orow[i + 3], rb);
+    for (int i = 0; i < 32; i += 4)
+      st_async_v4(dst + (uint32_t)(i / 4) * step, orow[i], orow[i + 1], orow[i + 2], orow[i + 3], rb);
   }
   if (tid < 32 && send) {
     const uint32_t dst = smem_u32(&us.cstat[rank][tid]);
@@ -1161,11 +1171,14 @@ __device__ __noinline__ void attn_combine(Misc& ms, const FusedParams& p, uint32
   const float inv = 1.f / den;
   bf16* ob = p.O + (int64_t)(u / p.H) * p.osb + (int64_t)(u % p.H) * p.osh;
   const int d0 = dlo((int)rank, cs), rows = dlo((int)rank + 1, cs) - d0;
+  const int crows = comb_rows(rows, (int)cs);
   auto out = [&](int dl) {
     float n = 0.f;
 #pragma unroll
     for (int r = 0; r < MAXCS; ++r)
-      if (r < (int)cs) n = fmaf(lds_f32(comb_a + 4u * (uint32_t)((r * rows + dl) * NQ + qi)), f[r], n);
+      if (r < (int)cs)
+        n = fmaf(lds_f32(comb_a + 16u * (uint32_t)((r * 8 + (qi >> 2)) * crows + dl) + 4u * (uint32_t)(qi & 3)),
+                 f[r], n);
     return n * inv;
   };
   // A slice of a multiple of 8 rows (clusters of a power of two): warp w
