@@ -8,6 +8,11 @@ kernels; if libwf.so is missing this module raises on import of the library
 
 Tensors are [B, H, rows, d] views whose last axis is contiguous (BHSD or
 BSHD strides both work); idx / level_sets are int32.
+
+A short call is bound by the time spent here, so the marshalling avoids what
+costs most: addresses and descriptors go to ctypes as they are (the argtypes
+convert them), shapes and strides are read once a tensor, and the current
+stream's handle is asked for without building a stream object.
 """
 from __future__ import annotations
 
@@ -93,40 +98,53 @@ def _check(status: int, what: str):
 
 def desc(t: torch.Tensor) -> wf_tensor:
     """wf_tensor for a [B, H, rows, d] tensor with a contiguous last axis."""
-    if t.dim() != 4:
+    shape = t.shape
+    if len(shape) != 4:
         raise ValueError("expected a [B, H, rows, d] tensor")
-    if t.dtype not in _DTYPES:
+    code = _DTYPES.get(t.dtype)
+    if code is None:
         raise ValueError(f"unsupported dtype {t.dtype}")
-    if t.shape[3] > 1 and t.stride(3) != 1:
+    sb, sh, ss, sd = t.stride()
+    B, H, S, D = shape
+    if D > 1 and sd != 1:
         raise ValueError("head_dim axis must be contiguous")
-    B, H, S, D = t.shape
-    return wf_tensor(B, H, S, D, t.stride(0), t.stride(1), t.stride(2), _DTYPES[t.dtype])
+    return wf_tensor(B, H, S, D, sb, sh, ss, code)
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+def _same_layout(a, b) -> bool:
+    return a.shape == b.shape and a.stride() == b.stride()
 
 
 def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
+
+
+_KEEP_TYPES: dict = {}
 
 
 def _keep_arr(keep):
-    arr = (ctypes.c_int32 * len(keep))(*[int(x) for x in keep])
-    return arr
+    n = len(keep)
+    t = _KEEP_TYPES.get(n)
+    if t is None:
+        t = _KEEP_TYPES[n] = ctypes.c_int32 * n
+    return t(*map(int, keep))
 
 
 def wf_coeffs_bytes(K: torch.Tensor, levels: int) -> int:
     d = desc(K)
-    return int(lib().wf_coeffs_bytes(ctypes.byref(d), levels))
+    return int(lib().wf_coeffs_bytes(d, levels))
 
 
 def wf_dwt_build(K: torch.Tensor, levels: int, coeffs: torch.Tensor, stream=None):
     d = desc(K)
-    _check(lib().wf_dwt_build(_ptr(K), None, ctypes.byref(d), levels, _ptr(coeffs),
-                              coeffs.numel() * coeffs.element_size(), _stream(stream)), "wf_dwt_build")
+    _check(lib().wf_dwt_build(_ptr(K), None, d, levels, _ptr(coeffs),
+                              coeffs.nbytes, _stream(stream)), "wf_dwt_build")
 
 
 def wf_cache_update(Knew: torch.Tensor, Vnew, K: torch.Tensor, V, pos: int, levels: int, coeffs: torch.Tensor,
@@ -134,9 +152,9 @@ def wf_cache_update(Knew: torch.Tensor, Vnew, K: torch.Tensor, V, pos: int, leve
     """Write Knew (and Vnew) into the caches at [pos, pos + count) and refresh
     the touched pyramid blocks (see the C header)."""
     dn, dk = desc(Knew), desc(K)
-    _check(lib().wf_cache_update(_ptr(Knew), _ptr(Vnew) if Vnew is not None else None, ctypes.byref(dn), _ptr(K),
-                                 _ptr(V) if V is not None else None, ctypes.byref(dk), pos, levels, _ptr(coeffs),
-                                 coeffs.numel() * coeffs.element_size(), _stream(stream)), "wf_cache_update")
+    _check(lib().wf_cache_update(_ptr(Knew), _ptr(Vnew) if Vnew is not None else None, dn, _ptr(K),
+                                 _ptr(V) if V is not None else None, dk, pos, levels, _ptr(coeffs),
+                                 coeffs.nbytes, _stream(stream)), "wf_cache_update")
 
 
 def wf_default_schedule(n: int, levels: int, k: int) -> list[int]:
@@ -160,14 +178,14 @@ def wf_schedule_from_proportions(n: int, levels: int, m) -> list[int]:
 
 def wf_filter_workspace_bytes(Q: torch.Tensor, K: torch.Tensor, levels: int, keep) -> int:
     dq, dk = desc(Q), desc(K)
-    return int(lib().wf_filter_workspace_bytes(ctypes.byref(dq), ctypes.byref(dk), levels, _keep_arr(keep)))
+    return int(lib().wf_filter_workspace_bytes(dq, dk, levels, _keep_arr(keep)))
 
 
 def wf_filter(Q: torch.Tensor, coeffs: torch.Tensor, K: torch.Tensor, levels: int, keep, idx: torch.Tensor,
               ws: torch.Tensor, level_sets: torch.Tensor | None = None, stream=None):
     dq, dk = desc(Q), desc(K)
-    _check(lib().wf_filter(_ptr(Q), ctypes.byref(dq), _ptr(coeffs), _ptr(K), ctypes.byref(dk), levels,
-                           _keep_arr(keep), _ptr(idx), _ptr(level_sets), _ptr(ws), ws.numel() * ws.element_size(),
+    _check(lib().wf_filter(_ptr(Q), dq, _ptr(coeffs), _ptr(K), dk, levels,
+                           _keep_arr(keep), _ptr(idx), _ptr(level_sets), _ptr(ws), ws.nbytes,
                            _stream(stream)), "wf_filter")
 
 
@@ -181,39 +199,39 @@ def wf_wavelet_approx(K: torch.Tensor, level: int, wavelet: int, out: torch.Tens
     dk = desc(K)
     if m is None:
         m = cand.shape[1] if cand is not None else K.shape[2] >> level
-    _check(lib().wf_wavelet_approx(_ptr(K), ctypes.byref(dk), _ptr(cand), int(m), level, wavelet, _ptr(out),
-                                   out.numel() * out.element_size(), _stream(stream)), "wf_wavelet_approx")
+    _check(lib().wf_wavelet_approx(_ptr(K), dk, _ptr(cand), int(m), level, wavelet, _ptr(out),
+                                   out.nbytes, _stream(stream)), "wf_wavelet_approx")
 
 
 def wf_filter_wavelet_workspace_bytes(Q: torch.Tensor, K: torch.Tensor, levels: int, keep, wavelet: int) -> int:
     dq, dk = desc(Q), desc(K)
-    return int(lib().wf_filter_wavelet_workspace_bytes(ctypes.byref(dq), ctypes.byref(dk), levels, _keep_arr(keep),
+    return int(lib().wf_filter_wavelet_workspace_bytes(dq, dk, levels, _keep_arr(keep),
                                                        wavelet))
 
 
 def wf_filter_wavelet(Q: torch.Tensor, top: torch.Tensor, K: torch.Tensor, levels: int, keep, wavelet: int,
                       idx: torch.Tensor, ws: torch.Tensor, level_sets: torch.Tensor | None = None, stream=None):
     dq, dk = desc(Q), desc(K)
-    _check(lib().wf_filter_wavelet(_ptr(Q), ctypes.byref(dq), _ptr(top), _ptr(K), ctypes.byref(dk), levels,
+    _check(lib().wf_filter_wavelet(_ptr(Q), dq, _ptr(top), _ptr(K), dk, levels,
                                    _keep_arr(keep), wavelet, _ptr(idx), _ptr(level_sets), _ptr(ws),
-                                   ws.numel() * ws.element_size(), _stream(stream)), "wf_filter_wavelet")
+                                   ws.nbytes, _stream(stream)), "wf_filter_wavelet")
 
 
 def wf_attn_workspace_bytes(Q: torch.Tensor, k: int, n_g: int) -> int:
     dq = desc(Q)
-    return int(lib().wf_attn_workspace_bytes(ctypes.byref(dq), k, n_g))
+    return int(lib().wf_attn_workspace_bytes(dq, k, n_g))
 
 
 def wf_sparse_attn(Q, K, V, idx, k: int, Kg, Vg, O, ws, scale: float = 0.0, stream=None):
     dq, dk, do = desc(Q), desc(K), desc(O)
     dg = desc(Kg) if Kg is not None else None
-    if Vg is not None and Kg is not None and (Vg.stride() != Kg.stride() or Vg.shape != Kg.shape):
+    if Vg is not None and Kg is not None and not _same_layout(Vg, Kg):
         raise ValueError("Kg and Vg must share shape and strides")
-    if V.stride() != K.stride() or V.shape != K.shape:
+    if not _same_layout(V, K):
         raise ValueError("K and V must share shape and strides")
-    _check(lib().wf_sparse_attn(_ptr(Q), ctypes.byref(dq), _ptr(K), _ptr(V), ctypes.byref(dk), _ptr(idx), k,
-                                _ptr(Kg), _ptr(Vg), ctypes.byref(dg) if dg is not None else None, _ptr(O),
-                                ctypes.byref(do), float(scale), _ptr(ws), ws.numel() * ws.element_size(),
+    _check(lib().wf_sparse_attn(_ptr(Q), dq, _ptr(K), _ptr(V), dk, _ptr(idx), k,
+                                _ptr(Kg), _ptr(Vg), dg, _ptr(O),
+                                do, float(scale), _ptr(ws), ws.nbytes,
                                 _stream(stream)), "wf_sparse_attn")
 
 
@@ -224,13 +242,13 @@ def wf_sparse_attn_noalloc(Q, K, V, idx, k: int, Kg, Vg, O, scale: float = 0.0, 
     context."""
     dq, dk, do = desc(Q), desc(K), desc(O)
     dg = desc(Kg) if Kg is not None else None
-    if Vg is not None and Kg is not None and (Vg.stride() != Kg.stride() or Vg.shape != Kg.shape):
+    if Vg is not None and Kg is not None and not _same_layout(Vg, Kg):
         raise ValueError("Kg and Vg must share shape and strides")
-    if V.stride() != K.stride() or V.shape != K.shape:
+    if not _same_layout(V, K):
         raise ValueError("K and V must share shape and strides")
-    _check(lib().wf_sparse_attn_noalloc(_ptr(Q), ctypes.byref(dq), _ptr(K), _ptr(V), ctypes.byref(dk), _ptr(idx),
-                                        k, _ptr(Kg), _ptr(Vg), ctypes.byref(dg) if dg is not None else None,
-                                        _ptr(O), ctypes.byref(do), float(scale), _stream(stream)),
+    _check(lib().wf_sparse_attn_noalloc(_ptr(Q), dq, _ptr(K), _ptr(V), dk, _ptr(idx),
+                                        k, _ptr(Kg), _ptr(Vg), dg,
+                                        _ptr(O), do, float(scale), _stream(stream)),
            "wf_sparse_attn_noalloc")
 
 
@@ -242,26 +260,26 @@ def wf_noalloc_status(stream=None):
 
 def wf_step_workspace_bytes(Q: torch.Tensor, K: torch.Tensor, levels: int, keep, n_g: int) -> int:
     dq, dk = desc(Q), desc(K)
-    return int(lib().wf_step_workspace_bytes(ctypes.byref(dq), ctypes.byref(dk), levels, _keep_arr(keep), n_g))
+    return int(lib().wf_step_workspace_bytes(dq, dk, levels, _keep_arr(keep), n_g))
 
 
 def wf_step(Q, K, V, Kg, Vg, coeffs, refresh: bool, levels: int, keep, idx, O, ws, stream=None,
             level_sets=None):
     dq, dk, do = desc(Q), desc(K), desc(O)
     dg = desc(Kg) if Kg is not None else None
-    if V.stride() != K.stride() or V.shape != K.shape:
+    if not _same_layout(V, K):
         raise ValueError("K and V must share shape and strides")
-    _check(lib().wf_step(_ptr(Q), ctypes.byref(dq), _ptr(K), _ptr(V), ctypes.byref(dk), _ptr(Kg), _ptr(Vg),
-                         ctypes.byref(dg) if dg is not None else None, _ptr(coeffs),
-                         coeffs.numel() * coeffs.element_size(), int(bool(refresh)), levels, _keep_arr(keep),
-                         _ptr(idx), _ptr(level_sets), _ptr(O), ctypes.byref(do), _ptr(ws),
-                         ws.numel() * ws.element_size(), _stream(stream)), "wf_step")
+    _check(lib().wf_step(_ptr(Q), dq, _ptr(K), _ptr(V), dk, _ptr(Kg), _ptr(Vg),
+                         dg, _ptr(coeffs),
+                         coeffs.nbytes, int(bool(refresh)), levels, _keep_arr(keep),
+                         _ptr(idx), _ptr(level_sets), _ptr(O), do, _ptr(ws),
+                         ws.nbytes, _stream(stream)), "wf_step")
 
 
 def wf_step_wavelet_workspace_bytes(Q: torch.Tensor, K: torch.Tensor, levels: int, keep, wavelet: int,
                                     n_g: int) -> int:
     dq, dk = desc(Q), desc(K)
-    return int(lib().wf_step_wavelet_workspace_bytes(ctypes.byref(dq), ctypes.byref(dk), levels, _keep_arr(keep),
+    return int(lib().wf_step_wavelet_workspace_bytes(dq, dk, levels, _keep_arr(keep),
                                                      wavelet, n_g))
 
 
@@ -269,12 +287,12 @@ def wf_step_wavelet(Q, top, K, V, Kg, Vg, levels: int, keep, wavelet: int, idx, 
                     level_sets=None):
     dq, dk, do = desc(Q), desc(K), desc(O)
     dg = desc(Kg) if Kg is not None else None
-    if V.stride() != K.stride() or V.shape != K.shape:
+    if not _same_layout(V, K):
         raise ValueError("K and V must share shape and strides")
-    _check(lib().wf_step_wavelet(_ptr(Q), ctypes.byref(dq), _ptr(top), _ptr(K), _ptr(V), ctypes.byref(dk),
-                                 _ptr(Kg), _ptr(Vg), ctypes.byref(dg) if dg is not None else None, levels,
-                                 _keep_arr(keep), wavelet, _ptr(idx), _ptr(level_sets), _ptr(O), ctypes.byref(do),
-                                 _ptr(ws), ws.numel() * ws.element_size(), _stream(stream)), "wf_step_wavelet")
+    _check(lib().wf_step_wavelet(_ptr(Q), dq, _ptr(top), _ptr(K), _ptr(V), dk,
+                                 _ptr(Kg), _ptr(Vg), dg, levels,
+                                 _keep_arr(keep), wavelet, _ptr(idx), _ptr(level_sets), _ptr(O), do,
+                                 _ptr(ws), ws.nbytes, _stream(stream)), "wf_step_wavelet")
 
 
 def wf_workspace_status(ws: torch.Tensor, stream=None):
