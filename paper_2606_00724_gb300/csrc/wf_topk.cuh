@@ -170,6 +170,53 @@ __device__ __forceinline__ uint3 warp_boundary(uint32_t hist_a, uint32_t need, i
                     __shfl_sync(0xffffffffu, ct, l2));
 }
 
+// The boundary bucket of the histogram: the bucket holding the need-th largest
+// undecided key (buckets ranked high to low), how many of its keys are still
+// needed, and how many it holds.  Thread t sums the BPT buckets
+// [NB - BPT (t + 1), NB - BPT t) (reading them in a lane-rotated order, free of
+// bank conflicts); a scan over the threads finds the one whose buckets reach
+// `need`, which searches them and publishes the result.  For two warpgroups:
+// with each warp searching the whole histogram by itself as below, its reads
+// were 1100 cycles of a Top-K of 5300 (128K step 90.2 -> 88.1 us).  One
+// warpgroup keeps that: two more barriers a Top-K cost two-unit clusters more
+// than they saved (64 units x 32K 68.6 -> 68.9 us).
+template <bool WIDE>
+__device__ __forceinline__ uint3 unit_boundary(uint32_t hist_a, uint32_t need, uint32_t sc_a) {
+  constexpr int TN = 32 * unit_warps<WIDE>(), BPT = NB / TN, NV = BPT / 4;
+  static_assert(NV == 4 || NV == 2, "the rotation below");
+  const int tid = ctid<WIDE>(), lane = tid & 31;
+  const uint32_t own = hist_a + 4u * (uint32_t)(NB - BPT * (tid + 1));
+  uint32_t tot = 0;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const uint4 v = lds_v4(own + 16u * (uint32_t)((i + (lane >> (NV == 4 ? 1 : 2))) & (NV - 1)));
+    tot += (v.x + v.y) + (v.z + v.w);
+  }
+  const uint32_t excl = (uint32_t)cta_excl_scan<WIDE>((int)tot, SC_ADDR(sc_a, wsum));
+  if (excl < need && need <= excl + tot) {  // one thread
+    uint32_t cum = excl, b = 0, nd = 0, ct = 0;
+    bool found = false;
+#pragma unroll
+    for (int g = NV - 1; g >= 0; --g) {
+      const uint4 v = lds_v4(own + 16u * (uint32_t)g);
+      const uint32_t c[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int e = 3; e >= 0; --e) {
+        const bool hit = !found && cum + c[e] >= need;
+        b = hit ? (uint32_t)(NB - BPT * (tid + 1) + 4 * g + e) : b;
+        nd = hit ? need - cum : nd;
+        ct = hit ? c[e] : ct;
+        found |= hit;
+        cum += c[e];
+      }
+    }
+    sts_v4(SC_ADDR(sc_a, wsum) + 32u, make_uint4(b, nd, ct, 0u));
+  }
+  csync<WIDE>();
+  const uint4 r = lds_v4(SC_ADDR(sc_a, wsum) + 32u);
+  return make_uint3(r.x, r.y, r.z);
+}
+
 // Top-K of the m keys at keys_a (largest first, lower position wins ties):
 // the kk chosen candidate indices, in ascending position order, overwrite the
 // key array.  A candidate's index is its position at the top scale, else
@@ -183,8 +230,8 @@ __device__ __forceinline__ uint3 warp_boundary(uint32_t hist_a, uint32_t need, i
 // order so that the 8 lanes of a quarter warp hit distinct banks).  Each
 // round spreads the undecided keys over NB buckets linear in [lo, hi] (fp32
 // arithmetic is monotone, so a key in a higher bucket is strictly larger);
-// every warp then finds the bucket holding the boundary from the counts: keys
-// above it are taken, keys below it dropped.  A boundary bucket of at most
+// the bucket holding the boundary is found from the counts: keys above it are
+// taken, keys below it dropped.  A boundary bucket of at most
 // as many keys as the unit has threads is resolved exactly: its keys go to a
 // list and are ranked on (key, -position) against the whole list.  Up to 32
 // keys (the common case: a few), every warp does that by itself with an entry
@@ -252,7 +299,7 @@ __device__ __noinline__ void select_keys(uint32_t keys_a, int m, int kk, uint32_
       reds_add_if(a4 & 8u, hist_a + 4u * b3, 1u);
     });
     csync<WIDE>();
-    const uint3 bd = warp_boundary(hist_a, need, lane);
+    const uint3 bd = WIDE ? unit_boundary<WIDE>(hist_a, need, sc_a) : warp_boundary(hist_a, need, lane);
     const int sb = (int)bd.x;
     need = bd.y;
     const uint32_t cnt = bd.z;
@@ -302,7 +349,7 @@ __device__ __noinline__ void select_keys(uint32_t keys_a, int m, int kk, uint32_
 #pragma unroll 1
         for (uint32_t w = __ballot_sync(0xffffffffu, win); w; w &= w - 1) {
           const int off = __shfl_sync(0xffffffffu, jx, __ffs(w) - 1) - j0;
-          took |= (uint32_t)off < (uint32_t)R ? (MT)1 << off : (MT)0;
+          took |= (uint32_t)off < (uint32_t)R ? act & ((MT)1 << off) : (MT)0;
         }
         act = 0;
         resolved = true;
