@@ -1535,11 +1535,12 @@ __device__ __forceinline__ float2 merge_ms(float2 a, float2 b) {
   return make_float2(M, a.y * ex2(a.x - M) + b.y * ex2(b.x - M));
 }
 
-template <int S>
-__device__ void gqa_producer_role(const Ctx& c, const FusedParams& p) {
-  Misc& ms = *c.ms;
-  const int pt = threadIdx.x - P0;
-  // The stacked query block first: row i = g q + r is row r of query head
+// The stacked query block, by the compute warps (idle until the first tile is
+// multiplied) while the producers start on the rows: up to 56 KB of copies took
+// the producers several us ahead of their first row.
+__device__ void gqa_load_queries(const Ctx& c, const FusedParams& p) {
+  const int tid = threadIdx.x;
+  // Row i = g q + r is row r of query head
   // h G + g; chunk ch holds rows 32 ch .. 32 ch + 31 (K-major core matrices),
   // rows >= G q zero-filled.
   const int64_t b = c.u0 / p.H, h = c.u0 % p.H;
@@ -1547,7 +1548,7 @@ __device__ void gqa_producer_role(const Ctx& c, const FusedParams& p) {
   for (int cc = 0; cc < p.nch * gqa_copies(p.nch); ++cc) {
     const uint32_t sq = smem_u32(c.smem + c.ly.q + cc * Q_BYTES);
     const int ch = cc % p.nch;
-    for (int e = pt; e < NQ * (D / 8); e += NPT) {
+    for (int e = tid; e < NQ * (D / 8); e += 64 * NCW) {
       const int rr = e & 7, c16 = (e >> 3) & (D / 8 - 1), g8 = e / D;
       const int i = ch * NQ + g8 * 8 + rr;
       const int ic = min(i, nq - 1), hd = ic / p.q, r = ic - hd * p.q;
@@ -1555,7 +1556,13 @@ __device__ void gqa_producer_role(const Ctx& c, const FusedParams& p) {
       cp_async16_zfill(sq + (uint32_t)(g8 * QGRP + c16 * 128 + rr * 16), src, i < nq);
     }
   }
-  cp_async_arrive_noinc(bar_addr(ms.qfull));
+  cp_async_arrive_noinc(bar_addr(c.ms->qfull));
+}
+
+template <int S>
+__device__ void gqa_producer_role(const Ctx& c, const FusedParams& p) {
+  Misc& ms = *c.ms;
+  const int pt = threadIdx.x - P0;
   int it = 0;
   for (int lev = c.lev_top; lev >= c.lev_end; --lev) {
     if (lev != c.lev_top) wait_or_abort(bar_addr(ms.jready[0]), (uint32_t)(c.lev_top - lev - 1) & 1u, ms, p.status);
@@ -1957,7 +1964,7 @@ __global__ void __launch_bounds__(NT, 1) wf_gqa_filter_kernel(const __grid_const
       mbar_init(bar_addr(ms.rdone[r]), 1);
       mbar_init(bar_addr(ms.rfree[r]), NCW);
     }
-    mbar_init(bar_addr(ms.qfull), NPT);
+    mbar_init(bar_addr(ms.qfull), 64 * NCW);
     mbar_init(bar_addr(ms.stallbar), 1);
     mbar_init(bar_addr(ms.drainbar), 1);
     ms.wait_limit = p.wait_limit;
@@ -1986,6 +1993,7 @@ __global__ void __launch_bounds__(NT, 1) wf_gqa_filter_kernel(const __grid_const
       *reinterpret_cast<uint4*>(smem + gl.sc + 16 * e) = make_uint4(0, 0, 0, 0);
     grid_dep_wait();
     grid_dep_launch();
+    if (warp < MMA_WARP) gqa_load_queries(c, p);
     tc_fence_before();
     named_sync(kSetupSyncId, NS);
     tc_fence_after();
@@ -1993,6 +2001,7 @@ __global__ void __launch_bounds__(NT, 1) wf_gqa_filter_kernel(const __grid_const
     cluster_sync();  // every CTA's barriers are armed before any remote arrival
     if (warp < MMA_WARP) {
       gqa_compute_role<S>(c, p, gl);
+      cp_async_wait_all();  // (query copies still in flight only after a wait gave up)
     } else {
       if ((tid & 31) == 0) gqa_mma_role<S>(c, p);
       __syncwarp();
