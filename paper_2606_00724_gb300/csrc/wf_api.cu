@@ -139,24 +139,24 @@ wf_status check_attn_args(const wf_tensor* q, const wf_tensor* kv, int k, const 
   return WF_OK;
 }
 
-// The skim and scan of one layer: wf_step's fused kernel without its attention
+// The skim and scan of one layer: the fused kernel without its attention
 // where it applies (one launch; one query head per key head), else the grouped
 // filter kernel, else three kernels a scale.  wf_filter's scratch beyond the
 // status word is used by the last only.  The line lies where the kernels'
 // limits do, because one launch is faster over the whole range: 32 heads x
 // 20K tokens, filter then attention, 152 us with 13 launches for the filter
-// and 69 us with one.
+// and two for the attention, 60 us with one each.
 cudaError_t run_filter(const wf::FilterPlan& p, const void* Q, const wf_tensor& q, const void* coeffs, const void* K,
                        const wf_tensor& kv, int levels, const int32_t* keep, int32_t* idx, int32_t* level_sets,
                        void* scratch, int* status, int sms, cudaStream_t s) {
   if (q.heads == kv.heads) {
-    const wf::FusedPlan fp = wf::plan_fused(q, kv, levels, keep, -1, sms);
+    const wf::FusedPlan fp = wf::plan_stage(q, kv, levels, keep, -1, sms);
     if (fp.ok) {
       wf::FusedRange r{};
       r.lev_top = levels;
       r.lev_bot = fp.trim ? 0 : 1;
       r.final_sel = 1;
-      return wf::launch_fused(fp, Q, q, K, nullptr, kv, nullptr, nullptr, nullptr, coeffs, levels, keep, idx,
+      return wf::launch_stage(fp, Q, q, K, nullptr, kv, nullptr, nullptr, nullptr, coeffs, levels, keep, idx,
                               level_sets, nullptr, q, status, s, &r);
     }
   }

@@ -246,12 +246,14 @@ cudaError_t launch_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd, c
   // bf16, one query head per key head, at most 32 query rows: the attention of
   // the fused step, one launch: the partials of a unit meet in the cluster's
   // shared memory instead of going through memory to a second kernel.  32
-  // heads, 1042 keys, head_dim 128: 15.7 us against 9.1 + 6.2 and a gap between
-  // the two (filter then attention at 20K tokens 69.0 -> 65.5 us).
+  // heads, 1042 keys, head_dim 128: 16.4 us against 9.1 + 6.2 and a gap between
+  // the two, and the code is the filter's, fetched already (filter then
+  // attention at 20K tokens 60.3 us, 65.2 with the split kernels), with P in
+  // two bf16 terms where those round it to one (wf_fused_stages.cu).
   const int sms = sm_count();
   if (p.dtype == WF_BF16 && p.G == 1 && sms > 0) {
     const int32_t keep = p.k;
-    const FusedPlan fp = plan_fused(qd, kv, 0, &keep, p.ng, sms);
+    const FusedPlan fp = plan_stage(qd, kv, 0, &keep, p.ng, sms);
     if (fp.ok) {
       FusedRange r{};
       r.lev_top = 0;
@@ -259,7 +261,7 @@ cudaError_t launch_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd, c
       r.attn = 1;
       r.sel = idx;
       r.scale = scale;
-      return launch_fused(fp, Q, qd, K, V, kv, Kg, Vg, g, nullptr, 0, &keep, nullptr, nullptr, O, od, status, s, &r);
+      return launch_stage(fp, Q, qd, K, V, kv, Kg, Vg, g, nullptr, 0, &keep, nullptr, nullptr, O, od, status, s, &r);
     }
   }
   // Other bf16 with head_dim 128: tensor cores.

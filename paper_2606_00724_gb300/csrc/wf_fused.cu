@@ -49,11 +49,18 @@
 #include "wf_topk.cuh"
 
 // The file is compiled once per head_dim (wf_fused_d64.cu defines 64 and
-// includes it); the entry points live in a namespace of that head_dim.
+// includes it), and for head_dim 128 once more for the filter and the attention
+// as calls of their own (wf_fused_stages.cu defines WF_STAGE_CALLS and includes
+// it); the entry points live in a namespace of each.
 #ifndef WF_HEAD_DIM
 #define WF_HEAD_DIM 128
 #endif
-#if WF_HEAD_DIM == 128
+#ifndef WF_STAGE_CALLS
+#define WF_STAGE_CALLS 0
+#endif
+#if WF_STAGE_CALLS
+#define WF_HD stage128
+#elif WF_HEAD_DIM == 128
 #define WF_HD hd128
 #else
 #define WF_HD hd64
@@ -88,8 +95,10 @@ constexpr int Q_BYTES = NQ * D * 2;
 // The attention's P = 2^(s - m) is the bf16 operand of the PV product.  For
 // head_dim 128 P is rounded to bf16.  For head_dim 64 P keeps its 24 bits, as
 // three bf16 terms (each the rounding of what the terms before it leave) that
-// multiply V one after the other into the same fp32 accumulator.
+// multiply V one after the other into the same fp32 accumulator.  An attention
+// of its own at head_dim 128 keeps 16 bits, as two terms (wf_fused_stages.cu).
 constexpr int PTERMS = D == 64 ? 3 : 1;
+constexpr bool kLowTerm = WF_STAGE_CALLS != 0;  // a launch of the attention alone has a second term
 constexpr int PT_BYTES = NQ * TM * 2;      // one term of one P tile
 constexpr int P_BYTES = PTERMS * PT_BYTES;
 constexpr int MAXCS_PAD_BYTES = 8 * NQ * 4;  // the ragged head-dim slices of a cluster of up to 8 CTAs
@@ -154,9 +163,9 @@ __device__ __forceinline__ UnitState& wslots(Misc& ms, int pp, int w) {
 // Shared-memory layout (byte offsets; the stage ring starts at 0, 1024-byte
 // aligned for the 128-byte swizzle).
 struct SmemLayout {
-  uint32_t q, p, misc, buf, bufw, total;
+  uint32_t q, p, misc, buf, bufw, lo, total;
 };
-__host__ __device__ inline SmemLayout smem_layout(int stages, int P, int cmax, int kmax) {
+__host__ __device__ inline SmemLayout smem_layout(int stages, int P, int cmax, int kmax, bool alone) {
   SmemLayout l;
   l.q = (uint32_t)stages * TILE_BYTES;
   l.p = l.q + (uint32_t)P * Q_BYTES;
@@ -165,7 +174,8 @@ __host__ __device__ inline SmemLayout smem_layout(int stages, int P, int cmax, i
   // then its selection J_b, the other still holds J_{b+1}.
   l.buf = (l.misc + (uint32_t)sizeof(Misc) + 127u) / 128u * 128u;
   l.bufw = (uint32_t)((max(cmax, kmax) + 3) / 4 * 4);
-  l.total = l.buf + (uint32_t)P * 2u * 4u * l.bufw;
+  l.lo = l.buf + (uint32_t)P * 2u * 4u * l.bufw;  // the second terms' double buffer
+  l.total = l.lo + (kLowTerm && alone ? (uint32_t)P * 2u * PT_BYTES : 0u);
   return l;
 }
 
@@ -544,6 +554,13 @@ __device__ __forceinline__ void mma_pv_tile(const Ctx& c, const FusedParams& p, 
         mma_bf16(ocol, smem_desc_sw128(st + kq * 2048, HALF_BYTES, 1024),
                  smem_desc(pa + pb * P_BYTES + e * PT_BYTES + kq * 1024, 512, 128), kIdescPV,
                  (t > 0 || kq > 0 || e > 0) ? 1u : 0u);
+    if (kLowTerm && p.sel) {
+      const uint32_t lo = smem_u32(c.smem + c.ly.lo) + (2u * pp + pb) * PT_BYTES;
+#pragma unroll
+      for (int kq = 0; kq < TM / 16; ++kq)
+        mma_bf16(ocol, smem_desc_sw128(st + kq * 2048, HALF_BYTES, 1024), smem_desc(lo + kq * 1024, 512, 128),
+                 kIdescPV, 1u);
+    }
   }
   mma_commit(bar_addr(ms.empty[s]));
   mma_commit(bar_addr(ms.pempty[pp][pb]));
@@ -929,10 +946,11 @@ __device__ __forceinline__ bool csync_or(bool v) {
 // stabiliser flush to zero, as they do below the largest term.  Rows past the
 // slice get P = 0.  The final m -> us.mloc, the row sums of P -> us.lacc.
 // WIDE: warpgroup w forms the P tiles t = w, w + 2, ... (always P buffer w).
+// LOW: P has a second term, in the unit's buffers lo.
 constexpr float kRaise = 64.f;
-template <bool WIDE>
-__device__ __noinline__ void attn_online(Misc& ms, int* status, float sl2, uint8_t* pbase, int pp, uint32_t tb,
-                                         int ntl, int mc, uint32_t& tpar, uint32_t ocol) {
+template <bool WIDE, bool LOW>
+__device__ __noinline__ void attn_online(Misc& ms, int* status, float sl2, uint8_t* pbase, uint8_t* lo, int pp,
+                                         uint32_t tb, int ntl, int mc, uint32_t& tpar, uint32_t ocol) {
   const int tid = ctid<WIDE>(), lane = tid & 31, warp = tid >> 5, row = tid & (TM - 1);
   const int wg = unit_wg<WIDE>();
   constexpr int NW = unit_warps<WIDE>();
@@ -1023,8 +1041,9 @@ __device__ __noinline__ void attn_online(Misc& ms, int* status, float sl2, uint8
       }
       // P^T, MN-major core matrices: key group r / 8, query chunk ch.  Rows
       // past the slice: P = 0.
-      uint8_t* dst = pbase + pb * P_BYTES + (row >> 3) * 512 + (row & 7) * 16;
-      if (PTERMS == 1) {
+      const int at = (row >> 3) * 512 + (row & 7) * 16;
+      uint8_t* dst = pbase + pb * P_BYTES + at;
+      if (PTERMS == 1 && !LOW) {
         uint32_t w[16];
         if (valid) {
 #pragma unroll
@@ -1054,7 +1073,8 @@ __device__ __noinline__ void attn_online(Misc& ms, int* status, float sl2, uint8
           ra[2 * k + 1] = __float_as_uint(e1);
         }
 #pragma unroll
-        for (int e = 0; e < PTERMS; ++e)
+        for (int e = 0; e < (LOW ? 2 : PTERMS); ++e) {
+          uint8_t* de = LOW && e == 1 ? lo + pb * PT_BYTES + at : dst + e * PT_BYTES;
 #pragma unroll
           for (int ch = 0; ch < 4; ++ch) {
             uint32_t w[4];
@@ -1067,8 +1087,9 @@ __device__ __noinline__ void attn_online(Misc& ms, int* status, float sl2, uint8
               ra[i + 1] = __float_as_uint(__uint_as_float(ra[i + 1]) - __high2float(h2));
               w[k] = *reinterpret_cast<const uint32_t*>(&h2);
             }
-            *reinterpret_cast<uint4*>(dst + e * PT_BYTES + ch * 128) = make_uint4(w[0], w[1], w[2], w[3]);
+            *reinterpret_cast<uint4*>(de + ch * 128) = make_uint4(w[0], w[1], w[2], w[3]);
           }
+        }
       }
       fence_proxy_async();
       tc_fence_before();
@@ -1341,7 +1362,8 @@ __device__ void compute_role(const Ctx& c, const FusedParams& p) {
   int a0, mc;
   attn_slice(p.keep[0] + p.ng, c.rank, c.cs, a0, mc);
   const int ntl = tiles_of(mc);
-  attn_online<WIDE>(ms, p.status, sl2, ubuf, pp, tb, ntl, mc, tpar, tb + p.ucols - 32);
+  attn_online<WIDE, kLowTerm>(ms, p.status, sl2, ubuf, c.smem + c.ly.lo + 2 * pp * PT_BYTES, pp, tb, ntl, mc, tpar,
+                              tb + p.ucols - 32);
   if (ntl > 0) wait_mdone();  // every PV product of the unit is done
   if (unit_wg<WIDE>() != 0) return;  // one warpgroup combines
   attn_combine(ms, p, c.rank, c.cs, u, ubuf, us, pp, tb + p.ucols - 32);
@@ -1352,7 +1374,7 @@ __global__ void __launch_bounds__(NT, 1) wf_fused_kernel(const __grid_constant__
   extern __shared__ __align__(1024) uint8_t smem[];
   Ctx c;
   c.smem = smem;
-  c.ly = smem_layout(S, p.P, p.cmax, p.kmax);
+  c.ly = smem_layout(S, p.P, p.cmax, p.kmax, p.sel != nullptr);
   c.ms = reinterpret_cast<Misc*>(smem + c.ly.misc);
   Misc& ms = *c.ms;
   c.rank = cluster_rank();
@@ -1462,6 +1484,7 @@ __global__ void __launch_bounds__(NT, 1) wf_fused_kernel(const __grid_constant__
   }
 }
 
+#if !WF_STAGE_CALLS
 
 // ---------------------------------------------------------------------------
 // Grouped query heads (reading 21): the filter of one key head for the
@@ -2022,6 +2045,7 @@ __global__ void __launch_bounds__(NT, 1) wf_gqa_filter_kernel(const __grid_const
     tmem_dealloc(c.tmem, p.tmem_cols);
   }
 }
+#endif  // !WF_STAGE_CALLS
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -2139,8 +2163,8 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   auto choose = [&](int P) {
     Choice ch{P, 0, MAXS, 0};
     const int clusters = (U + P - 1) / P;
-    if (smem_layout(MAXS, P, cmax, kmax).total > kMaxSmem) ch.stages = kStagesMin;
-    ch.smem = smem_layout(ch.stages, P, cmax, kmax).total;
+    if (smem_layout(MAXS, P, cmax, kmax, !filter).total > kMaxSmem) ch.stages = kStagesMin;
+    ch.smem = smem_layout(ch.stages, P, cmax, kmax, !filter).total;
     if (ch.smem > kMaxSmem) return ch;
     for (int c = MAXCS; c >= 1 && ch.cs == 0; --c)
       if (clusters * c <= num_sms && P * unit_cols(c) <= 512 &&
@@ -2253,6 +2277,7 @@ cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd
                 range && range->plain)(fused_kernel(fp.stages, fp.wide), p);
 }
 
+#if !WF_STAGE_CALLS
 // The grouped filter (wf_gqa_filter_kernel): bf16, at most 256 stacked
 // query rows a key head of grouped heads, or of one head with a block of more
 // than 32 rows (up to 32 are the fused kernel's), candidate lists within the
@@ -2424,6 +2449,7 @@ cudaError_t launch_literal_fused(const FusedPlan& fp, const FilterPlan& fl, cons
   }
   return cudaSuccess;
 }
+#endif  // !WF_STAGE_CALLS
 
 }  // namespace WF_HD
 }  // namespace wf

@@ -184,13 +184,15 @@ struct GqaPlan {
 // plan_fused: n_g generation rows of the attention, or -1 for a plan of the
 // filter alone; levels = 0 for a plan of the attention alone (keep[0] tokens).  launch_fused: range == nullptr is the whole step (every
 // scale, mu^0, the attention).
-#define WF_FUSED_ENTRY_POINTS                                                                                       \
+#define WF_CHAIN_ENTRY_POINTS                                                                                       \
   FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g,           \
                        int num_sms);                                                                                \
   cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd, const void* K, const void* V,   \
                            const wf_tensor& kv, const void* Kg, const void* Vg, const wf_tensor* g,                 \
                            const void* coeffs, int levels, const int32_t* keep, int32_t* idx, int32_t* level_sets,  \
-                           void* O, const wf_tensor& od, int* status, cudaStream_t s, const FusedRange* range);     \
+                           void* O, const wf_tensor& od, int* status, cudaStream_t s, const FusedRange* range);
+#define WF_FUSED_ENTRY_POINTS                                                                                       \
+  WF_CHAIN_ENTRY_POINTS                                                                                             \
   cudaError_t launch_literal_fused(const FusedPlan& fp, const FilterPlan& fl, const void* Q, const wf_tensor& qd,   \
                                    const void* top, const void* K, const void* V, const wf_tensor& kv,              \
                                    const void* Kg, const void* Vg, const wf_tensor* g, int wavelet, int32_t* idx,   \
@@ -206,7 +208,11 @@ WF_FUSED_ENTRY_POINTS
 namespace hd128 {
 WF_FUSED_ENTRY_POINTS
 }
+namespace stage128 {  // the filter and the attention as calls of their own
+WF_CHAIN_ENTRY_POINTS
+}
 #undef WF_FUSED_ENTRY_POINTS
+#undef WF_CHAIN_ENTRY_POINTS
 
 inline FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g,
                             int num_sms) {
@@ -218,6 +224,19 @@ inline cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_ten
                                 int32_t* level_sets, void* O, const wf_tensor& od, int* status, cudaStream_t s,
                                 const FusedRange* range) {
   return (kv.head_dim == 64 ? hd64::launch_fused : hd128::launch_fused)(
+      fp, Q, qd, K, V, kv, Kg, Vg, g, coeffs, levels, keep, idx, level_sets, O, od, status, s, range);
+}
+// The same for a call of the filter alone or of the attention alone.
+inline FusedPlan plan_stage(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g,
+                            int num_sms) {
+  return (kv.head_dim == 64 ? hd64::plan_fused : stage128::plan_fused)(q, kv, levels, keep, n_g, num_sms);
+}
+inline cudaError_t launch_stage(const FusedPlan& fp, const void* Q, const wf_tensor& qd, const void* K, const void* V,
+                                const wf_tensor& kv, const void* Kg, const void* Vg, const wf_tensor* g,
+                                const void* coeffs, int levels, const int32_t* keep, int32_t* idx,
+                                int32_t* level_sets, void* O, const wf_tensor& od, int* status, cudaStream_t s,
+                                const FusedRange* range) {
+  return (kv.head_dim == 64 ? hd64::launch_fused : stage128::launch_fused)(
       fp, Q, qd, K, V, kv, Kg, Vg, g, coeffs, levels, keep, idx, level_sets, O, od, status, s, range);
 }
 inline cudaError_t launch_literal_fused(const FusedPlan& fp, const FilterPlan& fl, const void* Q, const wf_tensor& qd,
