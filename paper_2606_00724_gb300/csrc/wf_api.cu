@@ -145,7 +145,7 @@ wf_status check_attn_args(const wf_tensor* q, const wf_tensor* kv, int k, const 
 // status word is used by the last only.  The line lies where the kernels'
 // limits do, because one launch is faster over the whole range: 32 heads x
 // 20K tokens, filter then attention, 152 us with 13 launches for the filter
-// and two for the attention, 60 us with one each.
+// and two for the attention, 57 us with one each.
 cudaError_t run_filter(const wf::FilterPlan& p, const void* Q, const wf_tensor& q, const void* coeffs, const void* K,
                        const wf_tensor& kv, int levels, const int32_t* keep, int32_t* idx, int32_t* level_sets,
                        void* scratch, int* status, int sms, cudaStream_t s) {
@@ -331,7 +331,7 @@ WF_API wf_status wf_filter_wavelet(const void* Q, const wf_tensor* q, const void
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int sms = 0;
   if (!device_sms(&sms)) return WF_ERR_CUDA;
-  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, -1, sms);
+  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, -1, sms, true);
   if (fp.ok && q->heads == kv->heads)
     return cuda_status(wf::launch_literal_fused(fp, p, Q, *q, top, K, nullptr, *kv, nullptr, nullptr, nullptr,
                                                 wavelet, idx, level_sets, nullptr, nullptr, ws,
@@ -404,7 +404,7 @@ WF_API wf_status wf_step(const void* Q, const wf_tensor* q, const void* K, const
   cudaError_t e = cudaSuccess;
   if (refresh_coeffs && (e = wf::launch_dwt(K, *kv, levels, coeffs, s)) != cudaSuccess) return WF_ERR_CUDA;
   // The fused kernel takes one query head per KV head.
-  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, n_g, sms);
+  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, n_g, sms, false);
   if (fp.ok && q->heads == kv->heads) {
     e = wf::launch_fused(fp, Q, *q, K, V, *kv, Kg, Vg, n_g > 0 ? g : nullptr, coeffs, levels, keep, idx,
                          level_sets, O, *o, status, s, nullptr);
@@ -457,7 +457,7 @@ WF_API wf_status wf_step_wavelet(const void* Q, const wf_tensor* q, const void* 
   int* status = static_cast<int*>(ws);
   void* scratch = static_cast<char*>(ws) + kStatusBytes;
   const wf::FilterPlan fl = wf::plan_filter(*q, *kv, levels, keep);
-  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, n_g, sms);
+  const wf::FusedPlan fp = wf::plan_fused(*q, *kv, levels, keep, n_g, sms, true);
   if (fp.ok && q->heads == kv->heads)
     return cuda_status(wf::launch_literal_fused(fp, fl, Q, *q, top, K, V, *kv, Kg, Vg, n_g > 0 ? g : nullptr, wavelet,
                                                 idx, level_sets, O, o, scratch, status, s));

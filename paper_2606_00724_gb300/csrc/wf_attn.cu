@@ -245,10 +245,9 @@ cudaError_t launch_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd, c
                         cudaStream_t s) {
   // bf16, one query head per key head, at most 32 query rows: the attention of
   // the fused step, one launch: the partials of a unit meet in the cluster's
-  // shared memory instead of going through memory to a second kernel.  32
-  // heads, 1042 keys, head_dim 128: 16.4 us against 9.1 + 6.2 and a gap between
-  // the two, and the code is the filter's, fetched already (filter then
-  // attention at 20K tokens 60.3 us, 65.2 with the split kernels), with P in
+  // shared memory instead of going through memory to a second kernel, and the
+  // code is the filter's, fetched already (filter then attention, 32 heads, 1042
+  // keys out of 20K tokens: 57.2 us, 62 with the split kernels), with P in
   // two bf16 terms where those round it to one (wf_fused_stages.cu).
   const int sms = sm_count();
   if (p.dtype == WF_BF16 && p.G == 1 && sms > 0) {

@@ -2115,7 +2115,8 @@ int max_active_clusters(int stages, bool wide, int cs, size_t smem) {
 
 }  // namespace
 
-FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g, int num_sms) {
+FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g, int num_sms,
+                     bool split) {
   FusedPlan fp{};
   fp.ok = false;
   if (kv.dtype != WF_BF16 || kv.head_dim != D || q.seq > NQ || levels > 10) return fp;
@@ -2147,11 +2148,14 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
     return 32 * tmax;
   };
   const size_t kMaxSmem = 227 * 1024;
-  // A one-unit plan runs both warpgroups on its unit when the candidate lists
-  // are long enough for the halved per-thread work to outweigh the wider
-  // barriers (measured: 128K tokens 123.6 -> 116.8 us; 8K tokens, lists of at
-  // most 1024, 49.5 -> 51.6 us).
-  const bool wide1 = cmax >= 2048 || (!filter && total >= 2048);
+  // A one-unit plan runs both warpgroups on its unit unless the candidate lists
+  // are too short for the halved per-thread work to outweigh the wider barriers
+  // (32 heads, head_dim 128, a step: lists of 512 22.0 -> 22.5 us; of 1024 38.5
+  // -> 38.4, and 47 -> 35 where outlying keys leave more in the Top-K's boundary
+  // bucket than one warpgroup lists at once; of 1638 46.7 -> 45.2).  Filter and
+  // attention calls take the same instance at any size: alternating two costs
+  // 5 us of code fetches.
+  const bool wide1 = split || D == 64 || cmax >= 1024;
   // For P units per cluster (1, or 2 so that one unit's copies overlap the
   // other's exchanges and Top-K): the largest cluster (any size up to 8)
   // whose grid fits the SMs in one wave, all clusters resident at once, and
@@ -2174,12 +2178,20 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
       if (P * unit_cols(c) <= 512) ch.cs = c;
     return ch;
   };
-  // Units per SM (P / cs) set each SM's share of the rows: take the smaller,
-  // two units per cluster on a tie.
+  // Units per SM (P / cs) set each SM's share of the rows: take the smaller.
+  // On a tie two units per cluster, so that one's copies run under the other's
+  // reductions over the whole chain of a step (64 units x 32K 71.6 -> 68.9 us,
+  // 128 units 106 -> 92), but one, on both warpgroups, where the chain is split
+  // over launches and there is little to overlap (64 units: filter and
+  // attention at 16K 82.3 -> 68.5 us, the db2 step at 32K 217.9 -> 189.0), and
+  // where the lists are short (at most 128 KB of rows: 64 units x 2K 26.3 ->
+  // 23.6 us, x 8K of head_dim 64 46.1 -> 43.3; 96 units x 8K, 256 KB, 60.4
+  // against 63.2).
+  const bool one_unit = split || cmax * D <= 1 << 16;
   const Choice c2 = U >= 2 ? choose(2) : Choice{2, 0, MAXS, 0};
   const Choice c1 = choose(1);
   Choice best = c2;
-  if (c2.cs == 0 || (c1.cs > 0 && 1 * c2.cs < 2 * c1.cs)) best = c1;
+  if (c2.cs == 0 || (c1.cs > 0 && c2.cs < 2 * c1.cs + (one_unit ? 1 : 0))) best = c1;
   if (best.cs == 0) return fp;
   const int P = best.P, cs = best.cs, stages = best.stages;
   const size_t smem = best.smem;

@@ -3,7 +3,7 @@
 // keeps two bf16 terms of P and the step's kernel loses registers and
 // instruction cache to them (64 units x 32K: 68.5 -> 70 us); one instance for
 // both calls, because a filter and its attention that alternate two kernels
-// fetch their instructions anew each time (20K tokens 60.4 -> 65 us).
+// fetch their instructions anew each time (20K tokens 57 -> 62 us).
 //
 // Why two terms: the fused attention takes P about the first tile's maximum,
 // where the split kernels that served this call before took each tile's own,

@@ -182,11 +182,12 @@ struct GqaPlan {
 };
 // The entry points, once per head_dim (wf_fused.cu is compiled for each).
 // plan_fused: n_g generation rows of the attention, or -1 for a plan of the
-// filter alone; levels = 0 for a plan of the attention alone (keep[0] tokens).  launch_fused: range == nullptr is the whole step (every
-// scale, mu^0, the attention).
+// filter alone; levels = 0 for a plan of the attention alone (keep[0] tokens);
+// split: the chain goes over several launches (or calls).  launch_fused: range
+// == nullptr is the whole step (every scale, mu^0, the attention).
 #define WF_CHAIN_ENTRY_POINTS                                                                                       \
   FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g,           \
-                       int num_sms);                                                                                \
+                       int num_sms, bool split);                                                                    \
   cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd, const void* K, const void* V,   \
                            const wf_tensor& kv, const void* Kg, const void* Vg, const wf_tensor* g,                 \
                            const void* coeffs, int levels, const int32_t* keep, int32_t* idx, int32_t* level_sets,  \
@@ -215,8 +216,8 @@ WF_CHAIN_ENTRY_POINTS
 #undef WF_CHAIN_ENTRY_POINTS
 
 inline FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g,
-                            int num_sms) {
-  return (kv.head_dim == 64 ? hd64::plan_fused : hd128::plan_fused)(q, kv, levels, keep, n_g, num_sms);
+                            int num_sms, bool split) {
+  return (kv.head_dim == 64 ? hd64::plan_fused : hd128::plan_fused)(q, kv, levels, keep, n_g, num_sms, split);
 }
 inline cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd, const void* K,
                                 const void* V, const wf_tensor& kv, const void* Kg, const void* Vg,
@@ -229,7 +230,7 @@ inline cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_ten
 // The same for a call of the filter alone or of the attention alone.
 inline FusedPlan plan_stage(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g,
                             int num_sms) {
-  return (kv.head_dim == 64 ? hd64::plan_fused : stage128::plan_fused)(q, kv, levels, keep, n_g, num_sms);
+  return (kv.head_dim == 64 ? hd64::plan_fused : stage128::plan_fused)(q, kv, levels, keep, n_g, num_sms, true);
 }
 inline cudaError_t launch_stage(const FusedPlan& fp, const void* Q, const wf_tensor& qd, const void* K, const void* V,
                                 const wf_tensor& kv, const void* Kg, const void* Vg, const wf_tensor* g,
