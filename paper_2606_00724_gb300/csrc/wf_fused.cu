@@ -98,7 +98,11 @@ constexpr int Q_BYTES = NQ * D * 2;
 // multiply V one after the other into the same fp32 accumulator.  An attention
 // of its own at head_dim 128 keeps 16 bits, as two terms (wf_fused_stages.cu).
 constexpr int PTERMS = D == 64 ? 3 : 1;
-constexpr bool kLowTerm = WF_STAGE_CALLS != 0;  // a launch of the attention alone has a second term
+constexpr bool kLowTerm = WF_STAGE_CALLS != 0;
+// Whether a launch may be the attention alone.  Its code is left out of the
+// other instance, whose first pass fetches all of it from memory (64 units x
+// 32K with L2 flushed 79.3 -> 78.2 us).
+constexpr bool kAlone = D == 64 || WF_STAGE_CALLS != 0;
 constexpr int PT_BYTES = NQ * TM * 2;      // one term of one P tile
 constexpr int P_BYTES = PTERMS * PT_BYTES;
 constexpr int MAXCS_PAD_BYTES = 8 * NQ * 4;  // the ragged head-dim slices of a cluster of up to 8 CTAs
@@ -485,7 +489,7 @@ __device__ void producer_role(const Ctx& c, const FusedParams& p) {
       it += ntl;
     }
   }
-  const int nsel = p.sel ? 1 : c.lev_top - c.lev_end + 1;  // selections made (or handed in)
+  const int nsel = kAlone && p.sel ? 1 : c.lev_top - c.lev_end + 1;  // selections made (or handed in)
   for (int pp = 0; pp < c.np && p.attn; ++pp) {
     wait_or_abort(bar_addr(ms.jready[pp]), (uint32_t)(nsel - 1) & 1u, ms, p.status);
     int a0, mc;
@@ -1257,7 +1261,7 @@ __device__ void compute_role(const Ctx& c, const FusedParams& p) {
 #pragma unroll 1
     for (int i = tid; i < p.keep[c.lev_top + 1]; i += TN) Jp[i] = src[2 * i] >> 1;
   }
-  if (p.sel) {
+  if (kAlone && p.sel) {
     const int32_t* src = p.sel + (int64_t)u * p.keep[0];
     int32_t* J = unit_J(c, p, pp, 0);
 #pragma unroll 1
@@ -1428,7 +1432,7 @@ __global__ void __launch_bounds__(NT, 1) wf_fused_kernel(const __grid_constant__
     if (tid == 0) {
       // Arm the first phase of every receive barrier (bytes this CTA expects).
       for (int pp = 0; pp < c.np; ++pp) {
-        if (c.lev_top >= c.lev_end) {
+        if (!kAlone || c.lev_top >= c.lev_end) {
           mbar_arrive_expect_tx(bar_addr(ms.xbar[pp]), c.cs * NQ * 8u);
           mbar_arrive_expect_tx(bar_addr(ms.kbar[pp]),
                                 4u * (uint32_t)m_total(p, c.lev_top) + c.cs * unit_warps<WIDE>() * 8u);
@@ -2294,7 +2298,7 @@ cudaError_t launch_fused(const FusedPlan& fp, const void* Q, const wf_tensor& qd
 // query rows a key head of grouped heads, or of one head with a block of more
 // than 32 rows (up to 32 are the fused kernel's), candidate lists within the
 // Top-K's 8192.  (32 heads x 16K tokens with blocks of 64: a step took 171 us
-// with 20 launches for the filter and takes 80 us with this one.)
+// with 20 launches for the filter and takes 73 us with this one.)
 // One unit per cluster; the largest cluster of up to 8 CTAs
 // whose grid fits the SMs in one wave with every cluster resident.
 constexpr int kGqaStages = 3 * 128 / D;  // least stages: beside 256 stacked query rows

@@ -265,8 +265,8 @@ __global__ void __launch_bounds__(NTH, 3) approx_kernel(const T* __restrict__ K,
 // works on the current 8, and the 16 warps an SM holds keep about 64 KB in
 // flight.  (Gathering 128 rows into shared memory, then transforming them
 // level by level between barriers, left DRAM at 44 % at scale 3.)  Measured:
-// the db2 step of 64 units x 32K tokens 233.1 -> 218.1 us; its three
-// transforms read 537 MB in about 84 us of that, 99 us before.  Scales 6 to 10
+// the db2 step of 64 units x 32K tokens 233.1 -> 218.1 us (187.7 with one unit
+// a cluster); its three transforms read 537 MB in about 84 us, 99 us before.  Scales 6 to 10
 // (a long halo, few outputs) keep the shared-memory kernel below.
 template <typename T, int TAPS, int L>
 struct Cascade {
