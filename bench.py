@@ -5,8 +5,8 @@ wf_step, i.e. the skim + multi-scale scan filter (Eq. 7-11) and the sparse
 attention (final step of Algorithm 1) over every (batch, head) of the
 workload, with the Haar pyramid of the prompt keys already built (the paper
 computes it at the initial step; the 32-layer workload "c5" instead
-refreshes it every 8 steps inside the timed loop).  For bf16 / head_dim 128
-that is one fused kernel launch per layer.
+refreshes it every 8 steps inside the timed loop).  For bf16 and fp32 with one
+query head per key head that is one fused kernel launch per layer.
 
 value = algorithmic HBM bytes of the step / device time (GB/s): the bytes
 that must move are the query block, the candidate coefficient rows of every
@@ -95,23 +95,26 @@ def wavelet_unit_bytes(w: synth.Workload) -> int:
 
 
 def fused_eligible(w: synth.Workload) -> bool:
-    """wf_step runs its single fused kernel for bf16, head_dim 128, <= 32 query
-    rows and one query head per key head (the Haar pyramid path)."""
+    """wf_step runs its single fused bf16 kernel (the Haar pyramid path)."""
     return WAVELET is None and fused_shape(w)
 
 
 def fused_shape(w: synth.Workload) -> bool:
-    """Shapes the fused kernel serves: bf16, head_dim 128, <= 32 query rows,
-    one query head per key head."""
-    return w.dtype == "bf16" and w.head_dim == 128 and w.q <= 32 and w.group == 1
+    """Shapes the fused bf16 kernel serves: <= 32 query rows, one query head
+    per key head."""
+    return w.dtype == "bf16" and w.q <= 32 and w.group == 1
+
+
+def f32_fused(w: synth.Workload) -> bool:
+    """wf_step runs its single fp32 kernel (one query head per key head)."""
+    return WAVELET is None and w.dtype == "f32" and w.group == 1
 
 
 def grouped_fused(w: synth.Workload) -> bool:
-    """Grouped query heads that wf_step filters with the grouped filter kernel
-    (bf16, head_dim 128, <= 32 rows a query head, <= 256 stacked rows), then
-    attends with the per-stage tensor-core attention (split + combine)."""
-    return (WAVELET is None and w.dtype == "bf16" and w.head_dim == 128 and w.q <= 32 and w.group > 1
-            and w.group * w.q <= 256)
+    """Grouped query heads, or blocks of more than 32 rows, that wf_step
+    filters with the grouped filter kernel (bf16, <= 256 stacked rows), then
+    attends with the per-stage attention (split + combine)."""
+    return (WAVELET is None and w.dtype == "bf16" and (w.group > 1 or w.q > 32) and w.group * w.q <= 256)
 
 
 def recorded_traffic(w: synth.Workload):
@@ -134,7 +137,7 @@ def recorded_traffic(w: synth.Workload):
 
 
 def launches_per_step(w: synth.Workload) -> int:
-    if fused_eligible(w):
+    if fused_eligible(w) or f32_fused(w):
         return 1
     if grouped_fused(w):  # the grouped filter kernel, the attention split and its combine
         return 3
@@ -449,8 +452,10 @@ def kernel_name(w):
     """The kernels a step of workload w runs (the roofline's "kernel")."""
     if fused_eligible(w):
         return "wf_fused_kernel"
+    if f32_fused(w):
+        return "wf_f32_kernel"
     if WAVELET:
-        return ("approx_kernel + wf_fused_kernel (one launch per scale)" if fused_shape(w) else
+        return ("approx_stream_kernel + wf_fused_kernel (one launch per scale)" if fused_shape(w) else
                 "per-stage kernels (approx/score/weights/select/attn)")
     if grouped_fused(w):
         return "wf_gqa_filter_kernel + tc_attn_rows_kernel + attn_combine_kernel"
@@ -540,7 +545,8 @@ def main():
               "head_dim": w.head_dim,
               "context": w.n, "query_block": w.q, "generation_rows": w.ng, "levels": w.levels, "k": w.k,
               "keep": list(w.keep), "layers": w.layers, "storage": w.dtype,
-              "step": ("wf_step (one fused filter + sparse-attention kernel) per layer" if fused_eligible(w) else
+              "step": ("wf_step (one fused filter + sparse-attention kernel) per layer"
+                       if fused_eligible(w) or f32_fused(w) else
                        f"wf_step_wavelet ({WAVELET}, periodized; the gathered candidate blocks transformed at every "
                        "scale" + ("; one fused filter launch per scale, the last with the sparse attention)"
                                   if fused_shape(w) else "; per-stage kernels)") + " per layer" if WAVELET else
