@@ -180,8 +180,8 @@ wf_status wf_level0_schedule(int64_t n, int levels, int64_t k, int32_t* keep);
  * kernel, within those kernels' limits (see wf_step); other shapes run three
  * kernels a scale.
  * ws: device scratch of at least wf_filter_workspace_bytes() bytes,
- * 256-byte aligned.  Its first 4 bytes are a status word: for bf16 keys with
- * head_dim 128 the scores run on the tensor cores, and a kernel whose bounded
+ * 256-byte aligned.  Its first 4 bytes are a status word: for bf16 keys
+ * the scores run on the tensor cores, and a kernel whose bounded
  * wait gives up (it never should) sets the word and leaves the outputs
  * undefined; wf_workspace_status() reads and clears it.  Zero the word once
  * before the first call; the rest of ws may hold anything.
@@ -250,8 +250,8 @@ wf_status wf_filter_wavelet(const void* Q, const wf_tensor* q, const void* top, 
  * (descriptor o: same shape and dtype as Q), written rounded to that dtype.
  * ws: device scratch of at least wf_attn_workspace_bytes() bytes, 256-byte
  * aligned; as for wf_filter, its first 4 bytes are a status word set if a
- * tensor-core kernel's bounded wait gives up (bf16 keys with head_dim 128 run
- * on the tensor cores): zero it once, read it with wf_workspace_status().
+ * tensor-core kernel's bounded wait gives up (bf16 keys run on the tensor
+ * cores): zero it once, read it with wf_workspace_status().
  * Out-of-range idx entries are clamped to [0, n) (never read out of bounds).
  * bf16 with one query head per key head, q <= 32 and k <= 8192 runs as one
  * launch of wf_step's fused kernel (its attention alone).
