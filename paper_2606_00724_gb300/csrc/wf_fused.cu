@@ -1454,10 +1454,10 @@ __global__ void __launch_bounds__(NT, 1) wf_fused_kernel(const __grid_constant__
     // Global memory only after the grids this launch depends on are done (the
     // set-up above overlaps their tail when the launch is programmatic).
     grid_dep_wait();
-    grid_dep_launch();
     tc_fence_before();
     named_sync(kSetupSyncId, NS);
     tc_fence_after();
+    grid_dep_launch();  // after the barrier that publishes the tensor memory (see Launch)
     c.tmem = ms.tmem_base;
     cluster_sync();  // every CTA's barriers are armed before any remote arrival
     if (warp < MMA_WARP) {
@@ -2019,11 +2019,11 @@ __global__ void __launch_bounds__(NT, 1) wf_gqa_filter_kernel(const __grid_const
     for (int e = tid; e < (int)((sizeof(SelScratch) + 15) / 16); e += NS)
       *reinterpret_cast<uint4*>(smem + gl.sc + 16 * e) = make_uint4(0, 0, 0, 0);
     grid_dep_wait();
-    grid_dep_launch();
     if (warp < MMA_WARP) gqa_load_queries(c, p);
     tc_fence_before();
     named_sync(kSetupSyncId, NS);
     tc_fence_after();
+    grid_dep_launch();  // after the barrier that publishes the tensor memory (see Launch)
     c.tmem = ms.tmem_base;
     cluster_sync();  // every CTA's barriers are armed before any remote arrival
     if (warp < MMA_WARP) {

@@ -286,7 +286,11 @@ int sm_count();
 // placed as that kernel's leave, so its launch and set-up hide in the other's
 // tail; every kernel launched this way executes grid_dep_wait before its first
 // access to global memory, so it still starts after everything before it on
-// the stream, and grid_dep_launch to let the next one in.  Back-to-back steps:
+// the stream, and grid_dep_launch to let the next one in.  A kernel with tensor
+// memory does that behind the barrier that follows its tmem_alloc: one thread's
+// grid_dep_launch counts for its CTA, and a dependent CTA on the same SM takes
+// its own columns before it waits for this grid, so a CTA still without its
+// columns could wait for them for ever.  Back-to-back steps:
 // 32 heads x 8K tokens 54.8 -> 53.3 us, 128K 93.4 -> 91.2; a filter and its
 // attention at 20K 65.5 -> 59.7.  The pyramid build stays an ordinary kernel
 // (`plain`): its 16,000 short CTAs slowed down with the two instructions, 391

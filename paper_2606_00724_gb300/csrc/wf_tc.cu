@@ -437,7 +437,6 @@ __global__ void __launch_bounds__(NTH, 2) tc_attn_kernel(const __grid_constant__
     fence_mbar_init();
   }
   grid_dep_wait();
-  grid_dep_launch();
   for (int e = tid; e < 256; e += NTA) {
     cm[e] = -INFINITY;
     cl[e] = 0.f;
@@ -517,6 +516,7 @@ __global__ void __launch_bounds__(NTH, 2) tc_attn_kernel(const __grid_constant__
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (j == 0) grid_dep_launch();  // after the barrier that publishes the tensor memory (see Launch)
     tmem = *tbase;
     ocol = tmem + (uint32_t)a.nq;  // O^T columns after S^T
     const uint32_t ph = (uint32_t)j & 1u;
@@ -732,7 +732,6 @@ __global__ void __launch_bounds__(NTH, 1) tc_attn_rows_kernel(const __grid_const
     fence_mbar_init();
   }
   grid_dep_wait();
-  grid_dep_launch();
   for (int e = tid; e < nmt * 128 * (D / 8); e += NTH) {
     const int rr = e & 7, ch = (e >> 3) & (D / 8 - 1), g = e >> 7;
     const int i = g * 8 + rr;
@@ -798,6 +797,7 @@ __global__ void __launch_bounds__(NTH, 1) tc_attn_rows_kernel(const __grid_const
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (j == 0) grid_dep_launch();  // after the barrier that publishes the tensor memory (see Launch)
     tmem = *tbase;
     const uint32_t ph = (uint32_t)j & 1u;
     if (tid == 0) {
