@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(256) score_kernel(const T* __restrict__ Q, int
     float mx = valid ? s : -INFINITY;
 #pragma unroll
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float e = valid ? expf(s - mx) : 0.f;
+    float e = valid && mx > -INFINITY ? expf(s - mx) : 0.f;
 #pragma unroll
     for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
     if (lane == 0) pt[i] = make_float2(mx, e);
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(256) weights_kernel(const float* __restrict__ 
   float z = 0.f;
 #pragma unroll 8
   for (int i = 0; i < q; ++i) z += expf((lg[(int64_t)i * lg_row] - Ms[i]) - mx);
-  W[(int64_t)u * w_unit + j] = mx + logf(z);
+  W[(int64_t)u * w_unit + j] = fmaxf(mx + logf(z), -INFINITY);  // (a row of -inf logits, a NaN so far, ranks last)
 }
 
 __device__ __forceinline__ uint32_t order_key(float f) {

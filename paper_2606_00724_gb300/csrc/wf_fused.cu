@@ -861,6 +861,10 @@ __device__ __noinline__ void pass_keys(uint32_t rank, uint32_t cs, Misc& ms, int
   const uint32_t nr = aborted(ms) ? 0u : cs;
   auto emit = [&](int j, float key) {
     if (j < mc) {
+      // A row whose logits are all -inf has no weight: its key is a NaN here
+      // (-inf - -inf, or the zero rows that pad the queries times an infinity)
+      // and must be -inf, below every other.
+      key = fmaxf(key, -INFINITY);
       kmin = fminf(kmin, key);
       kmax = fmaxf(kmax, key);
       const uint32_t dst = keys_a + 4u * (uint32_t)(g0 + j);
@@ -1891,7 +1895,7 @@ __device__ void gqa_compute_role(const Ctx& c, const FusedParams& p, const GqaLa
       if (lane == 0) mbar_arrive(bar_addr(ms.rfree[reg]));
       const int j = t * TM + row;
       if (j < mc) {
-        const float key = rm + lg2(rs);
+        const float key = fmaxf(rm + lg2(rs), -INFINITY);  // (a row of -inf logits: see pass_keys)
         kmin = fminf(kmin, key);
         kmax = fmaxf(kmax, key);
         const uint32_t dst = keys_a + 4u * (uint32_t)(g0 + j);

@@ -4,6 +4,7 @@
 // last one is written and before the call.
 #pragma once
 
+#include <float.h>
 #include <stddef.h>
 #include <stdint.h>
 
@@ -287,6 +288,9 @@ __device__ __noinline__ void select_keys(uint32_t keys_a, int m, int kk, uint32_
   bool resolved = false;
 #pragma unroll 1
   for (int iter = 0; iter < 6; ++iter) {
+    // A key of -inf (a row of weight 0) does not stretch the buckets to an
+    // infinite width, which would put every key into the lowest one.
+    lo = fmaxf(lo, -FLT_MAX);
     if (!(hi > lo)) break;  // every undecided key is equal (or none is left)
     const float scale = (float)NB / (hi - lo);
     for_groups([&](int g, const float4& v) {
