@@ -7,6 +7,7 @@
 // partial output sum_t exp(s_t - m) V_t.  A combine kernel rescales the
 // partials to the global max and normalises.  fp32 logits, softmax and
 // accumulation; O is rounded once to the output dtype.
+#include <float.h>
 #include <math.h>
 
 #include "wf_internal.cuh"
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(256) attn_split_kernel(
     float mx = fmaxf(s0, s1);
 #pragma unroll
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    mx = fmaxf(mx, -FLT_MAX);  // finite, so that a chunk of logits -inf has P = 0, not exp(-inf + inf)
     const float p0 = lane < cnt ? expf(s0 - mx) : 0.f;
     const float p1 = lane + 32 < cnt ? expf(s1 - mx) : 0.f;
     float z = p0 + p1;

@@ -27,6 +27,7 @@
 // and two for the attention: 4 heads x 1K tokens (d 64) 64.9 -> 19.2 us a
 // step, 16 heads x 8K (d 128) 170.6 -> 73.2 us, the error against 64 bits
 // no larger (3.1e-7 and 2.3e-6; 5.6e-7 and 3.8e-6 before).
+#include <float.h>
 #include <math.h>
 #include <string.h>
 
@@ -389,7 +390,7 @@ __global__ void __launch_bounds__(NTH, 1) wf_f32_kernel(const __grid_constant__ 
     auto krow = [&](int j) { return row_of(p.K, p.Kg, j); };
     auto vrow = [&](int j) { return row_of(p.V, p.Vg, j); };
     if (tid < 64) {
-      st.ms[tid] = -INFINITY;
+      st.ms[tid] = -FLT_MAX;  // finite, so that a tile of logits -inf has P = 0, not exp(-inf + inf)
       st.l[tid] = 0.f;
     }
     // Output accumulators: a thread holds 4 channels of QG queries over one of
@@ -427,7 +428,7 @@ __global__ void __launch_bounds__(NTH, 1) wf_f32_kernel(const __grid_constant__ 
         if (lane == 0)
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const float a = mo[k] > -INFINITY ? expf(mo[k] - mx[k]) : 0.f;
+            const float a = expf(mo[k] - mx[k]);
             st.alpha[i + k] = a;
             st.ms[i + k] = mx[k];
             st.l[i + k] = fmaf(st.l[i + k], a, z[k]);

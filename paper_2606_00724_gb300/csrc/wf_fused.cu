@@ -37,6 +37,7 @@
 // Every wait is bounded (~1 s): on timeout the CTA records a status word,
 // stops issuing MMAs and skips the remaining waits, so every thread reaches
 // the final cluster barrier.
+#include <float.h>
 #include <math.h>
 #include <string.h>
 
@@ -1012,7 +1013,7 @@ __device__ __noinline__ void attn_online(Misc& ms, int* status, float sl2, uint8
         float m = -INFINITY;
 #pragma unroll
         for (int w = 0; w < NW; ++w) m = fmaxf(m, wslots<WIDE>(ms, pp, w).red[w & 3][tid]);
-        m *= sl2;
+        m = fmaxf(m * sl2, -FLT_MAX);  // finite also where every logit so far is -inf: P is 0 there, not 2^(-inf + inf)
         const float mn = j == 0 ? m : fmaxf(us.mloc[tid], m);
         us.alpha[tid] = j == 0 ? 1.f : ex2(us.mloc[tid] - mn);
         us.mloc[tid] = mn;

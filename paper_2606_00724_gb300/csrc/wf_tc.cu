@@ -21,6 +21,7 @@
 // chunk of the query columns.  The wait on the MMAs is bounded (~1 s): on a
 // timeout the CTA sets the status word, waits once more with the same
 // bound, frees its TMEM and leaves.
+#include <float.h>
 #include <math.h>
 
 #include <algorithm>
@@ -438,7 +439,7 @@ __global__ void __launch_bounds__(NTH, 2) tc_attn_kernel(const __grid_constant__
   }
   grid_dep_wait();
   for (int e = tid; e < 256; e += NTA) {
-    cm[e] = -INFINITY;
+    cm[e] = -FLT_MAX;  // finite, so that a tile of logits -inf has P = 0, not 2^(-inf + inf)
     cl[e] = 0.f;
   }
   for (int e = tid; e < a.nq * (D / 8); e += NTA) {
@@ -569,7 +570,7 @@ __global__ void __launch_bounds__(NTH, 2) tc_attn_kernel(const __grid_constant__
       const float* r = rw + ucw * 128 + lane;
       const float mo = cm[ucol];
       const float mn = fmaxf(mo, fmaxf(fmaxf(r[0], r[32]), fmaxf(r[64], r[96])) * a.sl2);
-      ca[ucol] = mo == mn ? 1.f : ex2(mo - mn);  // mo = -inf: nothing accumulated yet
+      ca[ucol] = mo == mn ? 1.f : ex2(mo - mn);  // (0 from the first finite logit's tile on: nothing accumulated yet)
       cm[ucol] = mn;
     }
     wg_sync(wg);
@@ -784,7 +785,7 @@ __global__ void __launch_bounds__(NTH, 1) tc_attn_rows_kernel(const __grid_const
   const uint32_t lq = (uint32_t)(quarter * 32) << 16;  // this warp's TMEM lane quarter
   const bool active = mt < nmt;                        // a warpgroup past the M tiles only copies
   uint32_t tmem = 0;
-  float mrun = -INFINITY, lrun = 0.f;  // the row's stabiliser (log2 units) and sum of P
+  float mrun = -FLT_MAX, lrun = 0.f;  // the row's stabiliser (log2 units; finite, as above) and sum of P
   // This thread's row of P: group r / 8 of its M tile, row r % 8 of the core matrices.
   const uint32_t prow = smem_u32(pq) + (uint32_t)(mt * 16 + (r >> 3)) * QGRP + (uint32_t)(r & 7) * 16u;
   bool ok = true;
@@ -844,7 +845,7 @@ __global__ void __launch_bounds__(NTH, 1) tc_attn_rows_kernel(const __grid_const
       const float mnew = mx * a.sl2;
       float alpha = 1.f;
       if (mnew > mrun + kLazy) {
-        alpha = ex2(mrun - mnew);  // 0 on the first tile (mrun = -inf)
+        alpha = ex2(mrun - mnew);  // 0 on the first tile
         mrun = mnew;
       }
       const float nm = -mrun;

@@ -6,7 +6,10 @@ both element types and head dims, the grouped one and the kernels per scale.
 
 Selections against the fp64 oracle, bit for bit; the inputs are random, and the
 oracle's smallest relative gap at a Top-K boundary is checked to exceed what
-fp32 sums of 64 terms can move (2^-17), so that no near-tie decides."""
+fp32 sums of 64 terms can move (2^-17), so that no near-tie decides.
+
+In the attention such a row adds nothing, also where it fills a whole tile or
+slice: outputs within the bounds of the other tests."""
 import dataclasses
 
 import numpy as np
@@ -14,7 +17,7 @@ import pytest
 import torch
 
 import oracle
-from helpers import LibRun, f64
+from helpers import LibRun, assert_close_out, f64
 from paper_2606_00724_gb300 import wf
 
 pytestmark = pytest.mark.gpu
@@ -89,3 +92,40 @@ def test_filter_ranks_rows_without_weight_last(dtype, H, group, d, n, q, L, k, m
         got = run.level_sets(u)
         for lev in range(L, -1, -1):
             assert np.array_equal(np.asarray(got[lev]), want[lev]), f"unit {u} scale {lev}"
+
+
+def _attention(Q, K, V, group):
+    """softmax(Q K^T / sqrt d) V in fp64, on the device."""
+    Q, K, V = Q.double(), K.double().repeat_interleave(group, 1), V.double().repeat_interleave(group, 1)
+    return torch.softmax(Q @ K.transpose(2, 3) / Q.shape[3] ** 0.5, -1) @ V
+
+
+@pytest.mark.parametrize("dtype,H,group,d,q,n,k,masked", [
+    ("bf16", 2, 1, 128, 9, 2048, 512, slice(120, 420)),    # the fused kernel's attention: whole slices masked
+    ("bf16", 2, 1, 64, 32, 2048, 512, slice(0, 300)),
+    ("bf16", 90, 1, 128, 32, 2048, 512, slice(0, 300)),    # the first tiles of a longer slice
+    ("bf16", 2, 1, 128, 32, 16384, 8200, slice(0, 4000)),  # the split kernels: keys on the TMEM lanes
+    ("bf16", 2, 4, 128, 32, 2048, 700, slice(0, 300)),     # query rows on the TMEM lanes
+    ("bf16", 2, 2, 64, 40, 2048, 512, slice(60, 300)),     # CUDA cores
+    ("f32", 2, 1, 128, 9, 2048, 512, slice(60, 300)),
+])
+def test_attention_ignores_rows_without_weight(dtype, H, group, d, q, n, k, masked):
+    Q, K = _inputs(dtype, H, group, d, n, q, masked, -float("inf"), seed=k + d + q)
+    V = torch.randn(1, H, n, d, generator=torch.Generator().manual_seed(k)).to(DT[dtype]).cuda()
+    idx = torch.arange(k, dtype=torch.int32, device="cuda").repeat(H, 1)
+    O = torch.empty_like(Q)
+    ws = torch.zeros(wf.wf_attn_workspace_bytes(Q, k, 0), dtype=torch.uint8, device="cuda")
+    wf.wf_sparse_attn(Q, K, V, idx, k, None, None, O, ws)
+    wf.wf_workspace_status(ws)
+    assert_close_out(f64(O), f64(_attention(Q, K[:, :, :k], V[:, :, :k], group)), DT[dtype])
+
+
+@pytest.mark.parametrize("dtype,d,q", [("f32", 64, 3), ("f32", 128, 40), ("bf16", 128, 3), ("bf16", 64, 32)])
+def test_step_that_keeps_rows_without_weight(dtype, d, q):
+    n, L, k = 512, 1, 500
+    Q, K = _inputs(dtype, 2, 1, d, n, q, slice(100, 300), -float("inf"), seed=d + q)
+    V = torch.randn(1, 2, n, d, generator=torch.Generator().manual_seed(q)).to(DT[dtype]).cuda()
+    run = LibRun(Q, K, V, None, None, L, wf.wf_default_schedule(n, L, k)).dwt().step(refresh=False)
+    wf.wf_workspace_status(run.ws_step)
+    at = run.idx.long().view(1, 2, k, 1).expand(-1, -1, -1, d)
+    assert_close_out(f64(run.O), f64(_attention(Q, K.gather(2, at), V.gather(2, at), 1)), DT[dtype])
