@@ -218,6 +218,30 @@ cudaError_t run(const AttnPlan& p, const void* Q, const wf_tensor& qd, const voi
   return combine<T>(p, p.nsplit, O, od, ws, s);
 }
 
+// Whether one launch of the fused kernel's attention is faster than the split
+// kernel and its combine (head_dim 128; the others have CUDA cores as the
+// alternative, at least 1.2 times slower everywhere).  It saves a launch and the
+// partials' way through memory, and after a filter its code is fetched already,
+// but an SM holds one CTA of it and two of the split kernel's.  Measured over 1
+// to 512 units, 1 to 32 query rows, lists of 32 to 8192, P in two bf16 terms on both
+// sides; alone (us, 32 rows) and after a filter (the pair):
+//   32 units, 1024 keys  13.9 / 16.1, pair 44.8 / 48.4
+//   64 units, 2048 keys  26.9 / 27.5, pair 81.6 / 91.9
+//   96 units, 1024 keys  25.4 / 20.2, pair 76.1 / 80.6
+//   32 units, 8192 keys  92.1 / 44.6;  64 units, 4096 keys  73.0 / 45.5
+//  160 units, 1024 keys  50.9 / 40.7; 256 units, 4096 keys 218.3 / 131.7
+// So: every cluster at once, and the tiles that a CTA takes one after the other
+// at most twice those of a split CTA and a few more where the split leaves many
+// partials to fold or many rows of them.  Long lists leave the ring three
+// stages, which costs a quarter: then only against a split of single tiles.
+bool fused_attn_pays(const FusedPlan& fp, const AttnPlan& p, int sms) {
+  constexpr int TM = 128;
+  const int total = p.k + p.ng, tiles = (total + TM - 1) / TM;
+  const int own = fp.P * (((total + fp.cs - 1) / fp.cs + TM - 1) / TM);
+  const int tps = tc_attn_split(p.U, tiles, 2 * (int64_t)sms), nsplit = (tiles + tps - 1) / tps;
+  return fp.resident && own <= 2 * tps + nsplit / 8 + (p.q > 16) && (fp.full_ring || fp.P == 2 || tps == 1);
+}
+
 }  // namespace
 
 AttnPlan plan_attn(const wf_tensor& q, int k, int ng, int group) {
@@ -246,16 +270,13 @@ cudaError_t launch_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd, c
                         const wf_tensor* g, void* O, const wf_tensor& od, float scale, void* ws, int* status,
                         cudaStream_t s) {
   // bf16, one query head per key head, at most 32 query rows: the attention of
-  // the fused step, one launch: the partials of a unit meet in the cluster's
-  // shared memory instead of going through memory to a second kernel, and the
-  // code is the filter's, fetched already (filter then attention, 32 heads, 1042
-  // keys out of 20K tokens: 57.2 us, 62 with the split kernels), with P in
-  // two bf16 terms where those round it to one (wf_fused_stages.cu).
+  // the fused step, where it pays.
   const int sms = sm_count();
+  bool two_terms = false;
   if (p.dtype == WF_BF16 && p.G == 1 && sms > 0) {
     const int32_t keep = p.k;
     const FusedPlan fp = plan_stage(qd, kv, 0, &keep, p.ng, sms);
-    if (fp.ok) {
+    if (fp.ok && (p.d == 64 || fused_attn_pays(fp, p, sms))) {
       FusedRange r{};
       r.lev_top = 0;
       r.lev_bot = 1;
@@ -264,11 +285,12 @@ cudaError_t launch_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd, c
       r.scale = scale;
       return launch_stage(fp, Q, qd, K, V, kv, Kg, Vg, g, nullptr, 0, &keep, nullptr, nullptr, O, od, status, s, &r);
     }
+    two_terms = fp.ok;
   }
   // Other bf16 with head_dim 128: tensor cores.
   if (tc_attn_supported(p, p.G * p.q)) {
     int nsplit = 0;
-    cudaError_t e = launch_tc_attn(p, Q, qd, K, V, kv, idx, Kg, Vg, g, scale, status, ws, &nsplit, s);
+    cudaError_t e = launch_tc_attn(p, Q, qd, K, V, kv, idx, Kg, Vg, g, scale, status, ws, &nsplit, two_terms, s);
     if (e != cudaSuccess) return e;
     return combine<bf16>(p, nsplit, O, od, ws, s);
   }

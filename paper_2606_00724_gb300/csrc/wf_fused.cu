@@ -2172,9 +2172,10 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   struct Choice {
     int P, cs, stages;
     size_t smem;
+    bool resident;
   };
   auto choose = [&](int P) {
-    Choice ch{P, 0, MAXS, 0};
+    Choice ch{P, 0, MAXS, 0, false};
     const int clusters = (U + P - 1) / P;
     if (smem_layout(MAXS, P, cmax, kmax, !filter).total > kMaxSmem) ch.stages = kStagesMin;
     ch.smem = smem_layout(ch.stages, P, cmax, kmax, !filter).total;
@@ -2183,6 +2184,7 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
       if (clusters * c <= num_sms && P * unit_cols(c) <= 512 &&
           clusters <= max_active_clusters(ch.stages, P == 1 && wide1, c, ch.smem))
         ch.cs = c;
+    ch.resident = ch.cs > 0;
     for (int c = 1; c <= MAXCS && ch.cs == 0; ++c)
       if (P * unit_cols(c) <= 512) ch.cs = c;
     return ch;
@@ -2197,7 +2199,7 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   // 23.6 us, x 8K of head_dim 64 46.1 -> 43.3; 96 units x 8K, 256 KB, 60.4
   // against 63.2).
   const bool one_unit = split || cmax * D <= 1 << 16;
-  const Choice c2 = U >= 2 ? choose(2) : Choice{2, 0, MAXS, 0};
+  const Choice c2 = U >= 2 ? choose(2) : Choice{2, 0, MAXS, 0, false};
   const Choice c1 = choose(1);
   Choice best = c2;
   if (c2.cs == 0 || (c1.cs > 0 && c2.cs < 2 * c1.cs + (one_unit ? 1 : 0))) best = c1;
@@ -2221,6 +2223,8 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   fp.cs = cs;
   fp.P = P;
   fp.wide = P == 1 && wide1;
+  fp.resident = best.resident;
+  fp.full_ring = stages == MAXS;
   fp.stages = stages;
   fp.smem = smem;
   fp.tmem_cols = cols;

@@ -128,12 +128,13 @@ cudaError_t launch_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd, c
                         cudaStream_t s);
 // The tensor-core split attention (bf16, head_dim 128, <= 256 query rows per
 // key unit): partials in the workspace's flash-decoding layout, split count
-// into *nsplit_out.
+// into *nsplit_out; two_terms: P keeps 16 bits (<= 32 rows per key unit).
 bool tc_attn_supported(const AttnPlan& p, int kv_group_rows);
+int tc_attn_split(int64_t units, int tiles, int64_t slots);  // key tiles a split
 cudaError_t launch_tc_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd, const void* K, const void* V,
                            const wf_tensor& kv, const int32_t* idx, const void* Kg, const void* Vg,
                            const wf_tensor* g, float scale, int* status, void* ws, int* nsplit_out,
-                           cudaStream_t s);
+                           bool two_terms, cudaStream_t s);
 
 // Fused step (bf16, <= 32 query rows): one cluster of cs CTAs
 // per P units.
@@ -143,6 +144,8 @@ struct FusedPlan {
   size_t smem;
   bool trim;
   bool wide;  // one unit per cluster served by both compute warpgroups
+  bool resident;   // every cluster at once
+  bool full_ring;  // the most stages of the instance
 };
 // Part of the chain in one launch (the literal-basis path runs one launch per
 // scale, with the transform of the candidates' blocks between launches):

@@ -403,14 +403,17 @@ __host__ __device__ constexpr size_t tc_attn_smem(int nq) {
   return 6 * (size_t)HALF + (size_t)(nq / 8) * QGRP + sizeof(float) * (NWG * 128 + 3 * 256) + 32;
 }
 
+// TWO: P in two bf16 terms, 16 of its bits (the second behind the first in the
+// K stage's place), as the fused attention keeps them.
+template <bool TWO>
 __global__ void __launch_bounds__(NTH, 2) tc_attn_kernel(const __grid_constant__ TcAttnArgs a) {
   constexpr int NTA = NTH, NW = NWG, CW = 1;  // CW: query chunks of 32 a warpgroup takes (nq = 32)
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* kst = smem;                         // K stages, 2 x (2 x HALF)
   uint8_t* vt = smem + 4 * HALF;               // V tile, 2 x HALF
   uint8_t* sq = smem + 6 * HALF;               // query block, nq / 8 groups of QGRP
-  // P^T (16 key groups of nq * 16 bytes) takes the current K stage's place:
-  // the K rows are dead once the S^T products have completed.
+  // P^T (16 key groups of nq * 16 bytes a term) takes the current K stage's
+  // place: the K rows are dead once the S^T products have completed.
   float* red = reinterpret_cast<float*>(sq + (a.nq / 8) * QGRP);  // [NW][CW][4][32]
   float* cm = red + NW * CW * 128;             // [256] running max per query (log2 units)
   float* cl = cm + 256;                        // [256] running row sums of P
@@ -579,7 +582,7 @@ __global__ void __launch_bounds__(NTH, 2) tc_attn_kernel(const __grid_constant__
     for (int cw = 0; cw < ncw; ++cw) {
       const int ch = wg + NW * cw;
       float v[32];
-      uint32_t pk[16];
+      uint32_t pk[16], pl[TWO ? 16 : 1];
       tmem_ld32(tmem + qoff + 32 * ch, v);
       const uint32_t cma = smem_u32(cm + ch * 32), caa = smem_u32(ca + ch * 32);
       bool rescale = false;
@@ -593,9 +596,16 @@ __global__ void __launch_bounds__(NTH, 2) tc_attn_kernel(const __grid_constant__
           const float p0 = valid ? ex2(fmaf(v[i], a.sl2, -m4[e])) : 0.f;
           const float p1 = valid ? ex2(fmaf(v[i + 1], a.sl2, -m4[e + 1])) : 0.f;
           const __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);
-          v[i] = __low2float(h2);
-          v[i + 1] = __high2float(h2);
           pk[i / 2] = *reinterpret_cast<const uint32_t*>(&h2);
+          if (TWO) {
+            v[i] = p0;
+            v[i + 1] = p1;
+            const __nv_bfloat162 l2 = __floats2bfloat162_rn(p0 - __low2float(h2), p1 - __high2float(h2));
+            pl[i / 2] = *reinterpret_cast<const uint32_t*>(&l2);
+          } else {
+            v[i] = __low2float(h2);
+            v[i + 1] = __high2float(h2);
+          }
         }
         if (j > 0) {
           const uint4 f = lds_v4(caa + 16u * k4);
@@ -607,6 +617,12 @@ __global__ void __launch_bounds__(NTH, 2) tc_attn_kernel(const __grid_constant__
       for (int c4 = 0; c4 < 4; ++c4)
         *reinterpret_cast<uint4*>(prow + (ch * 4 + c4) * 128) =
             make_uint4(pk[4 * c4], pk[4 * c4 + 1], pk[4 * c4 + 2], pk[4 * c4 + 3]);
+      if (TWO) {
+#pragma unroll
+        for (int c4 = 0; c4 < 4; ++c4)
+          *reinterpret_cast<uint4*>(prow + TM * 2 * a.nq + (ch * 4 + c4) * 128) =
+              make_uint4(pl[4 * c4], pl[4 * c4 + 1], pl[4 * c4 + 2], pl[4 * c4 + 3]);
+      }
       rw[(cw * 4 + quarter) * 32 + lane] = xpose_reduce32<false>(v, lane);
       if (rescale) {
         // The partial O^T of the tiles before (every PV product of them is
@@ -636,6 +652,12 @@ __global__ void __launch_bounds__(NTH, 2) tc_attn_kernel(const __grid_constant__
       for (int kq = 0; kq < TM / 16; ++kq)
         mma_bf16(ocol, smem_desc_sw128(smem_u32(vt) + kq * 2048, HALF, 1024),
                  smem_desc(smem_u32(pb) + kq * 2 * (a.nq * 16), a.nq * 16, 128), idesc, (j > 0 || kq > 0) ? 1u : 0u);
+      if (TWO) {
+#pragma unroll
+        for (int kq = 0; kq < TM / 16; ++kq)
+          mma_bf16(ocol, smem_desc_sw128(smem_u32(vt) + kq * 2048, HALF, 1024),
+                   smem_desc(smem_u32(pb) + TM * 2 * a.nq + kq * 2 * (a.nq * 16), a.nq * 16, 128), idesc, 1u);
+      }
       mma_commit(smem_u32(&bar[1]));
     }
     __syncwarp();
@@ -941,10 +963,18 @@ bool tc_attn_supported(const AttnPlan& p, int kv_group_rows) {
   return p.dtype == WF_BF16 && p.d == D && kv_group_rows <= 256;
 }
 
+// Splits of several key tiles (taken in a pipeline with a running max) so that
+// the grid fits one wave of `slots` CTAs: fewer partials to write and fold.
+int tc_attn_split(int64_t units, int tiles, int64_t slots) {
+  int tps = 1;
+  while (tps < tiles && units * ((tiles + tps - 1) / tps) > slots) ++tps;
+  return tps;
+}
+
 cudaError_t launch_tc_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd, const void* K, const void* V,
                            const wf_tensor& kv, const int32_t* idx, const void* Kg, const void* Vg,
                            const wf_tensor* g, float scale, int* status, void* ws, int* nsplit_out,
-                           cudaStream_t s) {
+                           bool two_terms, cudaStream_t s) {
   TcAttnArgs a;
   a.Q = static_cast<const bf16*>(Q);
   a.qsb = qd.stride_b; a.qsh = qd.stride_h; a.qss = qd.stride_s;
@@ -971,12 +1001,8 @@ cudaError_t launch_tc_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd
   int sms = sm_count();
   if (sms <= 0) sms = 148;
   const int64_t units = (int64_t)kv.batch * kv.heads;
-  // Splits of several key tiles (taken in a pipeline with a running max) so
-  // that the grid fits one wave of `occ` CTAs an SM: fewer partials to write
-  // and fold.
   auto split = [&](int occ) {
-    a.tps = 1;
-    while (a.tps < tiles && units * ((tiles + a.tps - 1) / a.tps) > (int64_t)occ * sms) ++a.tps;
+    a.tps = tc_attn_split(units, tiles, (int64_t)occ * sms);
     a.nsplit = (tiles + a.tps - 1) / a.tps;
   };
   cudaError_t e;
@@ -997,8 +1023,9 @@ cudaError_t launch_tc_attn(const AttnPlan& p, const void* Q, const wf_tensor& qd
     a.tcols = 64;
     const size_t smem = tc_attn_smem(a.nq);
     split(2);
-    if ((e = raise_smem_limit(reinterpret_cast<const void*>(tc_attn_kernel), smem)) != cudaSuccess) return e;
-    e = Launch(dim3((unsigned)a.nsplit, (unsigned)units), NTH, smem, s)(tc_attn_kernel, a);
+    const auto k = two_terms ? tc_attn_kernel<true> : tc_attn_kernel<false>;
+    if ((e = raise_smem_limit(reinterpret_cast<const void*>(k), smem)) != cudaSuccess) return e;
+    e = Launch(dim3((unsigned)a.nsplit, (unsigned)units), NTH, smem, s)(k, a);
   }
   *nsplit_out = a.nsplit;
   return e;

@@ -87,3 +87,34 @@ def test_attention_keeps_more_than_bf16_weights(d, q, k, ng, amp):
         Ks, Vs = torch.cat([Ks, Kg.double()], 2), torch.cat([Vs, Vg.double()], 2)
     R = torch.softmax(Q.double() @ Ks.transpose(2, 3) / d ** 0.5, -1) @ Vs
     assert ((O.double() - R).abs() <= 2.0 ** -8 * R.abs() + 2.0 ** -15 * Vs.abs().max()).all()
+
+
+@pytest.mark.parametrize("H,d,q,n,k,ng,bshd", [
+    (160, 128, 32, 1024, 300, 5, False),   # more units than clusters at once
+    (32, 128, 17, 16384, 8192, 18, True),  # the fused kernel's largest list
+    (96, 128, 32, 2048, 1024, 32, False),  # nine tiles a CTA against three of a split
+    (40, 128, 1, 4096, 2500, 0, True),     # one query row
+    (512, 128, 3, 256, 1, 0, False),       # one key
+])
+def test_split_attention_keeps_as_much(H, d, q, n, k, ng, bshd):
+    """The calls that the split kernels take over from the fused attention, to
+    the same bound (their P has the two terms too): unsorted and repeated
+    tokens, [B, rows, H, d] strides."""
+    g = torch.Generator().manual_seed(k)
+
+    def rn(rows, a=1.0):
+        t = (a * torch.randn(1, H, rows, d, generator=g)).to(torch.bfloat16).cuda()
+        return t.transpose(1, 2).contiguous().transpose(1, 2) if bshd else t
+
+    Q, K, V, Kg, Vg = rn(q, 2.0), rn(n), rn(n), rn(max(ng, 1)), rn(max(ng, 1))
+    idx = torch.randint(0, n, (H, k), generator=g, dtype=torch.int32).cuda()
+    O = torch.empty_like(Q)
+    ws = torch.zeros(wf.wf_attn_workspace_bytes(Q, k, ng), dtype=torch.uint8, device="cuda")
+    wf.wf_sparse_attn(Q, K, V, idx, k, Kg if ng else None, Vg if ng else None, O, ws)
+    wf.wf_workspace_status(ws)
+    at = idx.long().view(1, H, k, 1).expand(-1, -1, -1, d)
+    Ks, Vs = K.gather(2, at).double(), V.gather(2, at).double()
+    if ng:
+        Ks, Vs = torch.cat([Ks, Kg.double()], 2), torch.cat([Vs, Vg.double()], 2)
+    R = torch.softmax(Q.double() @ Ks.transpose(2, 3) / d ** 0.5, -1) @ Vs
+    assert ((O.double() - R).abs() <= 2.0 ** -8 * R.abs() + 2.0 ** -15 * Vs.abs().max()).all()
