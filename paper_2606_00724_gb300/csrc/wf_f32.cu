@@ -544,13 +544,11 @@ int resident_clusters(F32Kernel k, int cs, size_t smem) {
   return n;
 }
 
-}  // namespace
-
 // fp32, one query head per key head, candidate lists within the Top-K's 8192.
 // The largest cluster (up to 8) whose grid fits the SMs in one wave, all
 // clusters resident, and whose slice's logits and at least 64 rows fit shared
 // memory; else the smallest whose logits fit.
-F32Plan plan_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g, int num_sms) {
+F32Plan fit_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g, int num_sms) {
   F32Plan fp{};
   if (kv.dtype != WF_F32 || q.heads != kv.heads || q.seq > kMaxQ || levels > 10) return fp;
   const int D = kv.head_dim, QM = q.seq <= 32 ? 32 : 64;
@@ -573,6 +571,7 @@ F32Plan plan_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int3
     if (rest + 64 * row > kMaxSmem) return false;
     fp.trow = std::min(want, (int)((kMaxSmem - rest) / row)) / 8 * 8;
     fp.smem = f32_layout(D, QM, fp.trow, fp.srow, fp.bufw).total;
+    fp.tiles = (rows + fp.trow - 1) / fp.trow;
     return true;
   };
   for (int cs = MAXCS; cs >= 1 && fp.cs == 0; --cs)
@@ -580,8 +579,70 @@ F32Plan plan_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int3
   for (int cs = 1; cs <= MAXCS && fp.cs == 0; ++cs)
     if (fit(cs) && resident_clusters(k, cs, fp.smem) > 0) fp.cs = cs;
   if (fp.cs == 0) return fp;
+  const int at_once = resident_clusters(k, fp.cs, fp.smem);
+  fp.waves = (U + at_once - 1) / at_once;
   fp.U = U;
   fp.ok = true;
+  return fp;
+}
+
+// What the routes of an fp32 call take, in ns, for up to 32 query rows and
+// slices of several tiles or waves: fitted to 690 (head_dim 64) and 888 (128)
+// measured shapes of that kind, 1 to 304 units, lists of up to 4096, 1 to 32
+// query rows; each fit is within 5 % of half of them and 15 % of 95 in 100.
+struct F32Cost {
+  float f0, frow, fkey;        // one-launch filter: in all; a wave, per gathered row of a CTA, per candidate
+  float s0, srow, skey, scan;  // one-launch step: the same; per attended key of a CTA
+  float scale, cand, candq, sel;  // kernels per scale: a scale; a unit's candidate, the same per 32 query rows; Top-K
+  float a0, att, attq;         // split attention: in all; a unit's key, the same per 32 query rows
+};
+constexpr F32Cost kCost64 = {5100.f, 33.f, 1.9f, 3900.f, 36.f, 2.8f, 52.f, 17000.f, 0.19f, 0.21f, 1.3f, 12000.f, 0.40f, 0.041f};
+constexpr F32Cost kCost128 = {0.f, 63.f, 1.1f, 0.f, 71.f, 1.4f, 87.f, 19000.f, 0.38f, 0.26f, 0.44f, 16000.f, 1.0f, 0.11f};
+
+}  // namespace
+
+// The one launch where it is the faster route (on a near tie too: its sums
+// are the more accurate ones).  It always is above 32 query rows, and where all
+// clusters run at once with slices of at most two tiles.  Elsewhere (more units than
+// clusters at once, slices that do not fit the row buffer) its CTAs compute 32
+// query rows for any block, with one CTA an SM, and the kernels per scale catch
+// up for small blocks.  Head_dim 64, 8 query rows, 16K tokens, a step: two scales,
+// 40 units 219 us against 145, 16 units 67 against 91; four scales, 80 units 292
+// against 238, 128 units 296 against 326; with 32 rows 80 units 297 against 318.
+// So there the routes' costs are compared.
+F32Plan plan_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g, int num_sms) {
+  F32Plan fp = fit_f32(q, kv, levels, keep, n_g, num_sms);
+  auto at_once = [](const F32Plan& p) { return p.waves == 1 && p.tiles <= 2; };
+  if (!fp.ok || q.seq > 32 || at_once(fp)) return fp;
+  const F32Cost& c = kv.head_dim == 64 ? kCost64 : kCost128;
+  // The candidate lists: their number and lengths.
+  const int lists = levels + (fp.trim ? 1 : 0);
+  auto list = [&](int i) { return i == 0 ? kv.seq >> levels : 2 * keep[levels + 1 - i]; };
+  float cands = 0.f;
+  for (int i = 0; i < lists; ++i) cands += (float)list(i);
+  auto gathered = [&](int cs) {
+    int rows = 0;
+    for (int i = 0; i < lists; ++i) rows += (list(i) + cs - 1) / cs;
+    return (float)rows;
+  };
+  const float U = (float)std::max(fp.U, 6);  // (fewer units leave the kernels per scale without CTAs)
+  const float q32 = (float)q.seq / 32.f, near_tie = 1.03f;
+  const float per_scale = c.scale * lists + U * cands * (c.cand + c.candq * q32) + c.sel * cands;
+  auto filter_cost = [&](const F32Plan& p) {
+    return c.f0 + (float)p.waves * (c.frow * gathered(p.cs) + c.fkey * cands);
+  };
+  if (n_g < 0) {
+    fp.ok = filter_cost(fp) <= near_tie * per_scale;
+    return fp;
+  }
+  const F32Plan ff = fit_f32(q, kv, levels, keep, -1, num_sms);
+  const float one_filter = ff.ok ? filter_cost(ff) : per_scale;
+  const float filter = ff.ok && (at_once(ff) || one_filter <= near_tie * per_scale) ? one_filter : per_scale;
+  const float keys = (float)(keep[0] + n_g);
+  const float split = c.a0 + U * keys * (c.att + c.attq * q32);
+  const float one = c.s0 + (float)fp.waves * (c.srow * gathered(fp.cs) + c.skey * cands +
+                                              c.scan * (float)((keep[0] + n_g + fp.cs - 1) / fp.cs));
+  fp.ok = one <= near_tie * (filter + split);
   return fp;
 }
 

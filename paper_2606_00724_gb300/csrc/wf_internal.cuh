@@ -264,8 +264,9 @@ inline cudaError_t launch_gqa_filter(const GqaPlan& gp, const void* Q, const wf_
 // The fp32 step (one query head per key head): one cluster of cs CTAs a unit
 // (n_g as for plan_fused).
 struct F32Plan {
-  bool ok, trim;
+  bool ok, trim;  // ok: it applies and is the faster route
   int U, cs, trow, srow, bufw;
+  int waves, tiles;  // waves of clusters; tiles of the widest slice
   size_t smem;
 };
 F32Plan plan_f32(const wf_tensor& q, const wf_tensor& kv, int levels, const int32_t* keep, int n_g, int num_sms);

@@ -55,3 +55,32 @@ def test_step_f32(B, H, d, q, n, L, k, ng, bshd):
             assert np.array_equal(got[lev], sets[lev]), f"unit {u} scale {lev}"
         assert np.array_equal(run.idx[u].cpu().numpy(), mu0)
         assert_close_out(f64(run.O[i, h]), oracle.sparse_attn(Q, K, V, mu0, kg, vg), torch.float32)
+
+
+@pytest.mark.parametrize("H,d,q,n,L,k,ng,bshd", [
+    (153, 128, 5, 2048, 1, 205, 7, True),    # filter and attention leave the one launch
+    (153, 64, 17, 2048, 2, 205, 0, False),   # the attention alone does
+    (38, 64, 1, 8192, 1, 819, 32, False),    # one wave would do, its slices do not fit the row buffer
+    (100, 64, 32, 4096, 2, 411, 3, True),    # two waves of the one launch, token trim
+])
+def test_step_f32_routes(H, d, q, n, L, k, ng, bshd):
+    """Small query blocks where the one launch takes several waves or tiles:
+    the routes that the plan's costs choose between."""
+    w = synth.Workload("f32", 1, H, d, n, q, max(ng, 1), L, tuple(wf.wf_default_schedule(n, L, k)), "f32", "iid")
+    units = [0, H // 2, H - 1]
+    b = synth.make_batch(w, planted=True, device="cuda", cfg="f32", units=units)
+    if bshd:
+        b = synth.Batch(*(_bshd(t) for t in (b.Q, b.K, b.V, b.Kg, b.Vg)), b.targets)
+    Kg, Vg = (b.Kg, b.Vg) if ng else (None, None)
+    run = LibRun(b.Q, b.K, b.V, Kg, Vg, L, w.keep).dwt().step(refresh=False)
+    filt = LibRun(b.Q, b.K, b.V, Kg, Vg, L, w.keep).dwt().filter()
+    torch.cuda.synchronize()
+    for u in units:
+        got, alone = run.level_sets(u), filt.level_sets(u)
+        for lev in range(L, -1, -1):
+            want = b.targets[u][lev].cpu().numpy()
+            assert np.array_equal(np.asarray(got[lev]), want), f"unit {u} scale {lev}"
+            assert np.array_equal(np.asarray(alone[lev]), want), f"unit {u} scale {lev}, the filter alone"
+        Q, K, V = f64(b.Q[0, u]), f64(b.K[0, u]), f64(b.V[0, u])
+        kg, vg = (f64(Kg[0, u]), f64(Vg[0, u])) if ng else (None, None)
+        assert_close_out(f64(run.O[0, u]), oracle.sparse_attn(Q, K, V, run.idx[u].cpu().numpy(), kg, vg), torch.float32)
