@@ -19,7 +19,12 @@
 // issued before the first store (the row's source is chosen as an address, not
 // by a branch around the load), the next chunk's loads before this one's
 // arithmetic, and CTAs are small, to use more SMs (32 rows of 64 units at 32K,
-// four scales: 9.3 -> 3.2 us a launch).
+// four scales: 9.3 -> 3.2 us a launch).  Large updates are bound by HBM, and a
+// value CTA then copies up to eight slices a thread: with one, starting the CTAs took
+// longer than the copies (16K rows of 64 units of 128 fp32 channels, four
+// scales: 786 -> 375 us).
+#include <algorithm>
+
 #include "wf_internal.cuh"
 
 namespace wf {
@@ -34,9 +39,11 @@ struct Update {
   int64_t nsb, nsh, nss;  // strides of the update buffers
   int64_t pos, count;
   int64_t blk0;           // first block of the unit that holds a new row
+  uint32_t vctas;         // CTAs of a unit's value rows
+  int vper;               // 16-byte slices a thread of theirs copies, at most kMaxSlices
 };
 
-constexpr int kBuildThreads = 256, kUpdateThreads = 64;
+constexpr int kBuildThreads = 256, kUpdateThreads = 64, kMaxSlices = 8;
 
 template <typename T, int L, bool UPDATE>
 __global__ void __launch_bounds__(UPDATE ? kUpdateThreads : kBuildThreads) dwt_kernel(const T* K_in, T* K_out, int64_t sb, int64_t sh,
@@ -49,13 +56,25 @@ __global__ void __launch_bounds__(UPDATE ? kUpdateThreads : kBuildThreads) dwt_k
   constexpr int NP = L > LC ? L - LC : 1;
   const int lanes = D / VEC;
   if (UPDATE && blockIdx.x >= key_ctas) {
-    // A 16-byte slice of a new value row.
-    const int64_t e = ((int64_t)blockIdx.x - key_ctas) * blockDim.x + threadIdx.x;
-    const int64_t r = e / lanes % up.count, u = e / lanes / up.count;
-    if (u >= total_items / (nblk * lanes)) return;
-    const int64_t bb = u / H, hh = u % H, x = e % lanes * VEC;
-    const uint4 w = __ldg(reinterpret_cast<const uint4*>(up.Vn + bb * up.nsb + hh * up.nsh + r * up.nss + x));
-    *reinterpret_cast<uint4*>(up.V + bb * sb + hh * sh + (up.pos + r) * ss + x) = w;
+    // 16-byte slices of a unit's new value rows: every load before the first store.
+    const uint32_t vb = blockIdx.x - (uint32_t)key_ctas, u = vb / up.vctas;
+    const int64_t bb = u / (uint32_t)H, hh = u % (uint32_t)H;
+    const T* src = up.Vn + bb * up.nsb + hh * up.nsh;
+    T* dst = up.V + bb * sb + hh * sh + up.pos * ss;
+    const int64_t e0 = (int64_t)(vb - u * up.vctas) * (kUpdateThreads * up.vper) + threadIdx.x;
+    const int shift = __ffs(lanes) - 1;  // (8, 16 or 32 slices a row)
+    auto here = [&](int i) { return i < up.vper && (e0 + i * kUpdateThreads) >> shift < up.count; };
+    auto at = [&](int i, int64_t row_stride) {
+      const int64_t e = e0 + i * kUpdateThreads;
+      return (e >> shift) * row_stride + (e & (lanes - 1)) * VEC;
+    };
+    uint4 w[kMaxSlices];
+#pragma unroll
+    for (int i = 0; i < kMaxSlices; ++i)
+      if (here(i)) w[i] = __ldg(reinterpret_cast<const uint4*>(src + at(i, up.nss)));
+#pragma unroll
+    for (int i = 0; i < kMaxSlices; ++i)
+      if (here(i)) *reinterpret_cast<uint4*>(dst + at(i, ss)) = w[i];
     return;
   }
   const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -150,7 +169,15 @@ cudaError_t run(const void* K, void* K_out, const wf_tensor& kv, void* coeffs, c
   if (up.count > 0) {
     Update<T> u2 = up;
     u2.blk0 = up.pos >> L;
-    const int64_t vblocks = up.Vn ? ((int64_t)U * up.count * lanes + threads - 1) / threads : 0;
+    // Value rows: as many slices a thread as leave the SMs eight CTAs each.
+    const int64_t slices = up.Vn ? up.count * lanes : 0;
+    u2.vper = 1;
+    if (U * slices > 8 * 100 * threads) {
+      const int sms = sm_count();
+      if (sms > 0) u2.vper = (int)std::clamp<int64_t>(U * slices / (8 * (int64_t)sms * threads), 1, kMaxSlices);
+    }
+    u2.vctas = (uint32_t)((slices + threads * u2.vper - 1) / (threads * u2.vper));
+    const int64_t vblocks = (int64_t)U * u2.vctas;
     dwt_kernel<T, L, true><<<(unsigned)(blocks + vblocks), threads, 0, s>>>(
         static_cast<const T*>(K), static_cast<T*>(K_out), kv.stride_b, kv.stride_h, kv.stride_s, kv.heads, kv.seq,
         kv.head_dim, static_cast<T*>(coeffs), rows_total, nblk, items, blocks, u2);

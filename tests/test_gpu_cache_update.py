@@ -108,3 +108,31 @@ def test_update_rows_and_values(dtype, d, L, pos, count):
     wf.wf_cache_update(Kn, Vn, K, V, pos, L, coeffs)
     torch.cuda.synchronize()
     assert torch.equal(K, K2) and torch.equal(V, V2) and torch.equal(coeffs, want)
+
+
+@pytest.mark.parametrize("dtype,B,H,d,n,pos,count,bshd", [
+    (torch.float32, 4, 8, 64, 8192, 1001, 5003, True),    # eight value slices a thread, a ragged last CTA
+    (torch.bfloat16, 2, 60, 128, 2048, 3, 2045, False),   # the last token
+    (torch.bfloat16, 1, 37, 64, 4096, 0, 4095, True),     # a few slices a thread
+    (torch.float32, 3, 40, 128, 1024, 511, 129, False),
+])
+def test_large_update(dtype, B, H, d, n, pos, count, bshd):
+    """Updates that fill the chip: the value rows go several slices a thread.
+    Caches and coefficients equal the copies and a full build, bit for bit."""
+    L = 2
+    g = torch.Generator(device="cuda").manual_seed(count)
+
+    def rn(rows):
+        t = torch.randn(B, H, rows, d, generator=g, device="cuda").to(dtype)
+        return t.transpose(1, 2).contiguous().transpose(1, 2) if bshd else t
+
+    K, V, Kn, Vn = rn(n), rn(n), rn(count), rn(count)
+    coeffs = torch.empty(wf.wf_coeffs_bytes(K, L), dtype=torch.uint8, device="cuda")
+    wf.wf_dwt_build(K, L, coeffs)
+    K2, V2 = K.clone(), V.clone()
+    K2[:, :, pos:pos + count], V2[:, :, pos:pos + count] = Kn, Vn
+    want = torch.empty_like(coeffs)
+    wf.wf_dwt_build(K2, L, want)
+    wf.wf_cache_update(Kn, Vn, K, V, pos, L, coeffs)
+    torch.cuda.synchronize()
+    assert torch.equal(K, K2) and torch.equal(V, V2) and torch.equal(coeffs, want)
