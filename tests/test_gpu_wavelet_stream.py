@@ -27,6 +27,11 @@ if not torch.cuda.is_available():
     (torch.bfloat16, 128, 1, 1501, 70, False),
     (torch.bfloat16, 128, 3, 500, 200, True),
     (torch.bfloat16, 128, 2, 401, 650, False),  # more units than resident CTAs
+    (torch.bfloat16, 128, 5, 48, 38, True),     # half of 152 SMs: one output a thread
+    (torch.bfloat16, 128, 5, 49, 38, False),    # and just more, runs of 4
+    (torch.bfloat16, 64, 5, 23, 200, False),
+    (torch.float32, 128, 4, 3, 60, True),
+    (torch.bfloat16, 64, 1, 70, 4, False),      # two blocks a load group, a run of one
 ])
 def test_stream_edges(basis, dtype, d, level, m, heads, bshd):
     wv, ov = (wf.WF_WAVELET_HAAR, oracle.HAAR) if basis == "haar" else (wf.WF_WAVELET_DB2, oracle.DB2)
