@@ -139,13 +139,14 @@ wf_status check_attn_args(const wf_tensor* q, const wf_tensor* kv, int k, const 
   return WF_OK;
 }
 
-// The skim and scan of one layer: the fused kernel without its attention
-// where it applies (one launch; one query head per key head), else the grouped
-// filter kernel, else three kernels a scale.  wf_filter's scratch beyond the
-// status word is used by the last only.  The line lies where the kernels'
-// limits do, because one launch is faster over the whole range: 32 heads x
-// 20K tokens, filter then attention, 152 us with 13 launches for the filter
-// and two for the attention, 57 us with one each.
+// The skim and scan of one layer in one launch where a plan has it (the fused
+// kernel without its attention for one query head per key head, the fp32
+// kernel, the grouped filter kernel), else three kernels a scale; wf_filter's
+// scratch beyond the status word is used by these only.  The fp32 and the
+// grouped plan compare the routes where the kernels per scale catch up; the
+// fused kernel is faster wherever it applies: 32 heads x 20K tokens, filter then
+// attention, 152 us with 13 launches for the filter and two for the attention,
+// 57 us with one each.
 cudaError_t run_filter(const wf::FilterPlan& p, const void* Q, const wf_tensor& q, const void* coeffs, const void* K,
                        const wf_tensor& kv, int levels, const int32_t* keep, int32_t* idx, int32_t* level_sets,
                        void* scratch, int* status, int sms, cudaStream_t s) {

@@ -2383,6 +2383,24 @@ GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int3
     layout(1);
     if (smem > kMaxSmem) return gp;
   }
+  gp.trim = keep[0] < 2 * keep[1];
+  if (D == 128 && nch == 1 && cs == 1) {
+    // One CTA a unit and at most 32 stacked rows, on half-empty M tiles: in a
+    // last wave that is nearly empty the kernels per scale, spread over every
+    // SM, are faster on long lists (160 units x 16K tokens, one scale, 8 heads x 4
+    // rows: 242 us against 192; x 32K, four scales 263 against 247; 8K, three
+    // scales 141 against 154).  Both sides in us, fitted to 280 shapes of 80 to
+    // 384 units (within 4 % of half of them and 16 % of 95 in 100; the choice is at most
+    // 5 % slower than the better side).
+    const int lists = levels + (gp.trim ? 1 : 0), waves = (U + num_sms - 1) / num_sms;
+    float cands = (float)(kv.seq >> levels);
+    for (int l = levels; l > levels + 1 - lists; --l) cands += 2.f * (float)keep[l];
+    const float one = 6.1f * (float)lists + 0.0147f * (float)waves * cands;
+    const float rows32 = (float)(G * q.seq) / 32.f;
+    const float per_scale =
+        20.7f * (float)lists + 1e-3f * cands * ((float)U * (0.112f + 0.011f * rows32) + 0.6f);
+    if (one > per_scale) return gp;
+  }
   const int cols = 512;  // both passes' columns
   gp.ok = true;
   gp.cs = cs;
@@ -2393,7 +2411,6 @@ GqaPlan plan_gqa(const wf_tensor& q, const wf_tensor& kv, int levels, const int3
   gp.G = G;
   gp.cmax = cmax;
   gp.kmax = kmax;
-  gp.trim = keep[0] < 2 * keep[1];
   gp.U = U;
   return gp;
 }

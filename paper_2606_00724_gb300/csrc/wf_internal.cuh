@@ -178,7 +178,7 @@ struct FusedRange {
 // (batch, key head); the stacked query rows of the G query heads as MMA
 // columns): mu^0 and the level sets, for the per-stage attention after it.
 struct GqaPlan {
-  bool ok;
+  bool ok;  // it applies and is the faster route
   int cs, stages, tmem_cols, nch, G, cmax, kmax, U;
   size_t smem;
   bool trim;

@@ -78,3 +78,27 @@ def test_grouped_filter_streams_again(B, H, group, q, n, L, k):
         got = run.level_sets(u)
         for lev in range(L, -1, -1):
             assert np.array_equal(got[lev], b.targets[u][lev].cpu().numpy()), f"unit {u} scale {lev}"
+
+
+@pytest.mark.parametrize("B,H,group,q,n,L,k", [
+    (4, 40, 8, 4, 16384, 1, 2048),   # 160 units: a last wave of 8, a long list: the kernels per scale
+    (4, 40, 8, 4, 4096, 1, 512),     # a short one: the grouped kernel
+    (2, 40, 2, 3, 16384, 1, 2049),   # half a wave, token trim
+    (5, 61, 4, 5, 8192, 2, 819),     # three waves, nearly full
+])
+def test_grouped_filter_line(B, H, group, q, n, L, k):
+    # Up to 32 stacked rows and one CTA a unit: where the plan prefers the
+    # kernels per scale, and beside that line; the filter and the step.
+    w = synth.Workload("grouped_line", B, H, 128, n, q, 1, L, tuple(wf.wf_default_schedule(n, L, k)), "bf16", "iid",
+                       group=group)
+    units = [0, B * H // 2, B * H - 1]
+    b = synth.make_batch(w, planted=True, device="cuda", cfg="line", units=units)
+    run = LibRun(b.Q, b.K, b.V, None, None, L, w.keep).dwt().filter()
+    step = LibRun(b.Q, b.K, b.V, None, None, L, w.keep).dwt().step(refresh=False)
+    wf.wf_workspace_status(step.ws_step)
+    torch.cuda.synchronize()
+    for u in units:
+        got, again = run.level_sets(u), step.level_sets(u)
+        for lev in range(L, -1, -1):
+            assert np.array_equal(got[lev], b.targets[u][lev].cpu().numpy()), f"unit {u} scale {lev}"
+            assert np.array_equal(again[lev], got[lev]), f"unit {u} scale {lev} of the step"
