@@ -119,10 +119,17 @@ def _same_layout(a, b) -> bool:
     return a.shape == b.shape and a.stride() == b.stride()
 
 
+# The handle without a stream object, where this torch has the call (it is not
+# part of torch's public interface).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
-    if stream is None:
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
-    return stream.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())  # (initialises CUDA, or raises, as current_stream does)
 
 
 _KEEP_TYPES: dict = {}
