@@ -117,15 +117,27 @@ def grouped_fused(w: synth.Workload) -> bool:
     return (WAVELET is None and w.dtype == "bf16" and (w.group > 1 or w.q > 32) and w.group * w.q <= 256)
 
 
-def recorded_traffic(w: synth.Workload):
-    """DRAM bytes per launch of the fused kernel from the committed ncu record,
-    if it was taken on this workload with the current kernel source."""
+# What the fused kernel is compiled from: a traffic record holds for these.
+FUSED_SOURCES = ("wf_fused.cu", "wf_topk.cuh", "wf_sm100.cuh", "wf_internal.cuh")
+
+
+def fused_source_hash(csrc: str) -> str:
     import hashlib
-    rec = os.path.join(ROOT, "profiles", "wf_fused_kernel_traffic.md")
-    src = os.path.join(ROOT, "paper_2606_00724_gb300", "csrc", "wf_fused.cu")
-    if not (os.path.exists(rec) and os.path.exists(src)):
+    h = hashlib.sha256()
+    for f in FUSED_SOURCES:
+        with open(os.path.join(csrc, f), "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()[:16]
+
+
+def recorded_traffic(w: synth.Workload, root: str = ROOT):
+    """DRAM bytes per launch of the fused kernel from the committed ncu record,
+    if it was taken on this workload with the current kernel sources."""
+    rec = os.path.join(root, "profiles", "wf_fused_kernel_traffic.md")
+    csrc = os.path.join(root, "paper_2606_00724_gb300", "csrc")
+    if not os.path.exists(rec) or not all(os.path.exists(os.path.join(csrc, f)) for f in FUSED_SOURCES):
         return None
-    h = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
+    h = fused_source_hash(csrc)
     for ln in open(rec):
         cells = [c.strip() for c in ln.strip().strip("|").split("|")]
         if len(cells) == 6 and cells[0] == w.name and cells[5] == h:
