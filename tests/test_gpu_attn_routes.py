@@ -1,9 +1,10 @@
 """wf_sparse_attn on the fused kernel's attention (bf16, one query head a key
 head, at most 32 query rows) at its edges: fewer keys than CTAs in the
-cluster, ragged slices, two units a cluster, both warpgroups on a unit, lists
-of 8192 tokens (its largest) and beyond (the split kernels), unsorted,
-repeated and out-of-range tokens (clamped), an explicit scale, [B, rows, H, d]
-strides, both head dims.  Outputs against the fp64 oracle: O is rounded to
+cluster, ragged slices, clusters of one to eight CTAs, lists of 8192 tokens
+(its largest), and on the split kernels (longer lists, more units than
+clusters at once); unsorted, repeated and out-of-range tokens (clamped), an
+explicit scale, [B, rows, H, d] strides, both head dims.  (Two units a cluster:
+test_gpu_two_units.py.)  Outputs against the fp64 oracle: O is rounded to
 bf16 once, and the split kernels round P as well (relative 2^-8 each, the
 weights' errors averaging below their bound): the bf16 bound of the other
 tests.  The fused attention's own error is held to the rounding of O."""
@@ -25,11 +26,11 @@ if not torch.cuda.is_available():
     (1, 1, 128, 1, 64, 1, 0, 0.0, False),
     (1, 2, 64, 32, 256, 3, 2, 0.0, True),
     (2, 3, 128, 17, 2048, 333, 5, 0.25, True),
-    (2, 32, 128, 32, 4096, 517, 32, 0.0, False),   # two units a cluster
+    (2, 32, 128, 32, 4096, 517, 32, 0.0, False),   # one unit a cluster of two CTAs
     (1, 32, 64, 31, 8192, 1000, 7, 0.2, True),
-    (1, 2, 128, 32, 16384, 8192, 3, 0.0, False),   # both warpgroups, the largest list
-    (1, 1, 128, 32, 16384, 8193, 0, 0.0, False),   # the split kernels
-    (3, 60, 128, 5, 1024, 200, 0, 0.0, False),     # more clusters than fit at once
+    (1, 2, 128, 32, 16384, 8192, 3, 0.0, False),   # the largest list
+    (1, 1, 128, 32, 16384, 8193, 0, 0.0, False),   # the split kernels: a longer one
+    (3, 60, 128, 5, 1024, 200, 0, 0.0, False),     # and more units than clusters fit at once
 ])
 def test_attention_route(B, H, d, q, n, k, ng, scale, bshd):
     g = torch.Generator(device="cpu").manual_seed(k + d)

@@ -26,7 +26,7 @@ def _bshd(t):
 
 
 @pytest.mark.parametrize("B,H,group,q,n,L,k,bshd", [
-    (1, 3, 1, 1, 2048, 1, 301, False),    # one query row, one scale, an odd k (token trim), units that pair unevenly
+    (1, 3, 1, 1, 2048, 1, 301, False),    # one query row, one scale, an odd k (token trim)
     (1, 1, 1, 32, 256, 3, 8, True),       # one unit, fewer candidates than one tile
     (2, 3, 1, 32, 4104, 3, 512, True),    # ragged n, [B, rows, H, d] strides
     (1, 2, 1, 17, 16384, 1, 4096, False),  # 8192 candidates: the largest list of the fused kernel

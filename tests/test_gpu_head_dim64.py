@@ -1,6 +1,6 @@
 """The fused step and the grouped filter for bf16 with head_dim 64, at the
 edges of their plans: one query row, ragged lists, clusters of 8 down to 1,
-two units a cluster, both warpgroups on a unit, no generation rows, token
+both warpgroups on a unit, no generation rows, token
 trim, [B, rows, H, d] strides, blocks of 33 to 64 rows, grouped heads.
 
 Indices and level sets bit-exact against the fp64 oracle on planted inputs.
@@ -32,7 +32,7 @@ def _bshd(t):
     (1, 3, 1, 1, 2048, 2, 301, 0, False),    # one query row, token trim, no generation rows
     (1, 5, 1, 17, 4104, 3, 512, 7, True),    # ragged n, [B, rows, H, d] strides, an odd unit count
     (2, 16, 1, 32, 8200, 3, 821, 32, True),  # clusters of 4
-    (4, 40, 1, 32, 2048, 2, 256, 32, False),  # more units than SMs: two units a cluster of one or two CTAs
+    (4, 40, 1, 32, 2048, 2, 256, 32, False),  # more units than SMs: one unit a cluster of one CTA, two waves
     (1, 2, 1, 32, 65536, 4, 3277, 64, False),  # lists above 2048: both warpgroups on the unit
     (1, 3, 1, 40, 4104, 3, 513, 5, False),   # blocks of more than 32 rows: the grouped filter
     (1, 2, 4, 32, 4104, 3, 512, 32, True),   # grouped heads

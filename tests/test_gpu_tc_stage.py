@@ -1,10 +1,13 @@
-"""GPU parity of the tensor-core per-stage kernels (bf16, head_dim 128):
-the tcgen05 skim inside wf_filter and the tcgen05 split attention inside
-wf_sparse_attn, on shapes the workloads do not reach: query blocks that are
-not a multiple of 32 rows (1, 17, 40, and 3 grouped heads of 20), sparse
-key counts that leave ragged 128-key splits, no generation rows, BSHD
-strides, a non-default attention scale.  Indices bit-exact against the
-oracle on planted inputs; outputs within the bf16 bound."""
+"""GPU parity of the tensor-core kernels per stage (bf16, head_dim 128) on
+shapes the workloads do not reach.  The calls with up to 8192 candidates and
+tokens take the fused or the grouped filter and, with one query head a key
+head, the fused attention: query blocks that are not a multiple of 32 rows (1,
+17, 40, and 3 grouped heads of 20), sparse key counts that leave ragged
+128-key tiles, no generation rows, BSHD strides, a non-default attention
+scale.  The tcgen05 score kernel per scale serves longer lists, and the split
+attention with keys on the TMEM lanes grouped heads of at most 32 stacked rows
+and longer token lists: both with ragged query blocks.  Indices bit-exact
+against the oracle on planted inputs; outputs within the bf16 bound."""
 import dataclasses
 
 import numpy as np
@@ -74,3 +77,40 @@ def test_tc_attention_bshd_and_scale():
         p = np.exp(s - s.max(axis=1, keepdims=True))
         want = (p / p.sum(axis=1, keepdims=True)) @ Vs
         assert_close_out(f64(O[b, h]), want, torch.bfloat16)
+
+
+@pytest.mark.parametrize("q,group,n,k", [(40, 1, 16640, 2048), (17, 1, 17408, 3001), (5, 3, 16640, 1500),
+                                         (32, 7, 16640, 2048), (1, 1, 16640, 512)])
+def test_score_kernel_on_long_lists(q, group, n, k):
+    # One scale of 8320 or more candidates: the score kernel twice a scale.
+    w = synth.Workload("tc_long", 1, 2, 128, n, q, 1, 1, tuple(wf.wf_default_schedule(n, 1, k)), "bf16", "iid",
+                       group=group)
+    b = synth.make_batch(w, planted=True, device="cuda", cfg="tc_long")
+    run = LibRun(b.Q, b.K, b.V, None, None, 1, w.keep).dwt().filter()
+    torch.cuda.synchronize()
+    for u in range(w.units):
+        got = run.level_sets(u)
+        for lev in (1, 0):
+            assert np.array_equal(got[lev], b.targets[u][lev].cpu().numpy()), f"unit {u} scale {lev}"
+
+
+@pytest.mark.parametrize("q,group,n,k,ng,scale", [(5, 3, 2048, 333, 5, 0.0), (4, 8, 2048, 1000, 0, 0.05), (16, 2, 512, 1, 3, 0.0),
+                                                  (17, 1, 16384, 8200, 9, 0.0), (1, 1, 16384, 8193, 0, 0.11)])
+def test_split_attention_keys_on_lanes(q, group, n, k, ng, scale):
+    # Unsorted tokens, BSHD caches, ragged stacked rows.
+    B, H, d = 2, 3, 128
+    g = torch.Generator().manual_seed(k)
+    bshd = lambda rows, heads=H: torch.randn(B, rows, heads, d, generator=g).to(torch.bfloat16).cuda().transpose(1, 2)
+    Q, K, V, Kg, Vg = bshd(q, H * group), bshd(n), bshd(n), bshd(max(ng, 1)), bshd(max(ng, 1))
+    idx = torch.stack([torch.randperm(n, generator=g)[:k] for _ in range(B * H)]).int().cuda()
+    O = torch.empty(B, H * group, q, d, dtype=torch.bfloat16, device="cuda")
+    ws = torch.zeros(wf.wf_attn_workspace_bytes(O, k, ng), dtype=torch.uint8, device="cuda")
+    wf.wf_sparse_attn(Q, K, V, idx, k, Kg if ng else None, Vg if ng else None, O, ws, scale)
+    wf.wf_workspace_status(ws)
+    at = idx.long().view(B, H, k, 1).expand(-1, -1, -1, d)
+    Ks, Vs = K.gather(2, at).double(), V.gather(2, at).double()
+    if ng:
+        Ks, Vs = torch.cat([Ks, Kg.double()], 2), torch.cat([Vs, Vg.double()], 2)
+    Ks, Vs = Ks.repeat_interleave(group, 1), Vs.repeat_interleave(group, 1)
+    R = torch.softmax(Q.double() @ Ks.transpose(2, 3) * (scale or d ** -0.5), -1) @ Vs
+    assert_close_out(f64(O), f64(R), torch.bfloat16)

@@ -4,8 +4,7 @@ for bit (whole prompt and gathered candidate blocks), the Haar case against
 the stored pyramid and wf_filter, and wf_filter_wavelet's indices against
 the oracle's literal filter on planted inputs (every scale, bit-exact), and
 wf_step_wavelet's indices and output against the oracle.  For bf16 keys with
-head_dim 128 and one query head per key head both calls run the fused
-kernel once per scale."""
+one query head per key head both calls run the fused kernel once per scale."""
 import dataclasses
 
 import numpy as np
@@ -174,8 +173,7 @@ def test_step_wavelet_db2_matches_oracle(cfg, units):
 
 @pytest.mark.parametrize("basis", ["db2", "haar"])
 def test_step_wavelet_odd_units_no_generation_rows(basis):
-    # Three units (a two-unit cluster plan leaves its last cluster one unit)
-    # and no generation rows: every unit against the oracle's literal filter
+    # Three units and no generation rows: every unit against the oracle's literal filter
     # (indices at every scale) and attention over the selected rows only.
     wv, ov = BASES[basis]
     w = dataclasses.replace(synth.WORKLOADS["c3"], name="odd_units", batch=1, heads=3, n=4096, levels=3, ng=0,
