@@ -177,13 +177,14 @@ wf_status wf_level0_schedule(int64_t n, int levels, int64_t k, int32_t* keep);
  * [B*H][keep[L] + .. + keep[1] + keep[0]] = J_L, .., J_1, mu^0 per unit.
  * The whole filter is one launch of wf_step's fused kernel without its
  * attention (one query head per key head) or, for bf16, of its grouped filter
- * kernel, within those kernels' limits (see wf_step); other shapes run three
- * kernels a scale.
+ * kernel, within those kernels' limits (see wf_step) and where that is the
+ * faster route; other shapes run three kernels a scale.  bf16 scores run on the
+ * tensor cores, but for head_dim 64 in the kernels per scale (lists above 8192).
+ * A row whose logits are all -inf has weight 0: it ranks below every other.
  * ws: device scratch of at least wf_filter_workspace_bytes() bytes,
- * 256-byte aligned.  Its first 4 bytes are a status word: for bf16 keys
- * the scores run on the tensor cores, and a kernel whose bounded
- * wait gives up (it never should) sets the word and leaves the outputs
- * undefined; wf_workspace_status() reads and clears it.  Zero the word once
+ * 256-byte aligned.  Its first 4 bytes are a status word: a tensor-core kernel
+ * whose bounded wait gives up (it never should) sets the word and leaves the
+ * outputs undefined; wf_workspace_status() reads and clears it.  Zero the word once
  * before the first call; the rest of ws may hold anything.
  * ------------------------------------------------------------------------- */
 size_t wf_filter_workspace_bytes(const wf_tensor* q, const wf_tensor* kv, int levels, const int32_t* keep);
@@ -250,11 +251,15 @@ wf_status wf_filter_wavelet(const void* Q, const wf_tensor* q, const void* top, 
  * (descriptor o: same shape and dtype as Q), written rounded to that dtype.
  * ws: device scratch of at least wf_attn_workspace_bytes() bytes, 256-byte
  * aligned; as for wf_filter, its first 4 bytes are a status word set if a
- * tensor-core kernel's bounded wait gives up (bf16 keys run on the tensor
- * cores): zero it once, read it with wf_workspace_status().
+ * tensor-core kernel's bounded wait gives up: zero it once, read it with
+ * wf_workspace_status().
  * Out-of-range idx entries are clamped to [0, n) (never read out of bounds).
  * bf16 with one query head per key head, q <= 32 and k <= 8192 runs as one
- * launch of wf_step's fused kernel (its attention alone).
+ * launch of wf_step's fused kernel (its attention alone; head_dim 128 where that
+ * is the faster route).  Other bf16 with head_dim 128 and at most 256 rows of
+ * grouped heads (G q) runs on the tensor cores in two launches; everything else
+ * (fp32; bf16 with head_dim 64 and grouped heads, q > 32 or k > 8192) in two on the
+ * CUDA cores.
  * ------------------------------------------------------------------------- */
 size_t wf_attn_workspace_bytes(const wf_tensor* q, int k, int n_g);
 wf_status wf_sparse_attn(const void* Q, const wf_tensor* q, const void* K, const void* V, const wf_tensor* kv,
@@ -317,7 +322,9 @@ wf_status wf_noalloc_status(void* stream);
  * stacked rows as the MMA columns), then the attention of wf_sparse_attn.
  * fp32 with one query head per key head runs as one fused kernel in fp32
  * arithmetic throughout, one cluster per (batch, head).
- * All three take candidate lists of at most 8192 at every scale.
+ * All three take candidate lists of at most 8192 at every scale; the grouped and
+ * the fp32 one are left where the per-stage kernels are faster (many units or
+ * slices beyond shared memory, with small query blocks).
  * Other shapes run the per-stage kernels.  The bf16 fused kernels' waits
  * (on copies, tensor-core completion and the cluster's exchanges) are
  * bounded: if one gives up (it never should), the kernel returns early,

@@ -2160,10 +2160,11 @@ FusedPlan plan_fused(const wf_tensor& q, const wf_tensor& kv, int levels, const 
   // A one-unit plan runs both warpgroups on its unit unless the candidate lists
   // are too short for the halved per-thread work to outweigh the wider barriers
   // (32 heads, head_dim 128, a step: lists of 512 22.0 -> 22.5 us; of 1024 38.5
-  // -> 38.4, and 47 -> 35 where outlying keys leave more in the Top-K's boundary
-  // bucket than one warpgroup lists at once; of 1638 46.7 -> 45.2).  Filter and
-  // attention calls take the same instance at any size: alternating two costs
-  // 5 us of code fetches.
+  // -> 38.4; of 1638 46.7 -> 45.2).  Where outlying keys leave more in the
+  // Top-K's boundary bucket than one warpgroup lists at once, whatever the
+  // length, both save a second round (47 -> 35 us at 1024).  The one-unit plans of
+  // filter and attention calls take the same instance at any size: alternating
+  // two costs 5 us of code fetches.
   const bool wide1 = split || D == 64 || cmax >= 1024;
   // For P units per cluster (1, or 2 so that one unit's copies overlap the
   // other's exchanges and Top-K): the largest cluster (any size up to 8)

@@ -295,8 +295,8 @@ int sm_count();
 // grid_dep_launch counts for its CTA, and a dependent CTA on the same SM takes
 // its own columns before it waits for this grid, so a CTA still without its
 // columns could wait for them for ever.  Back-to-back steps:
-// 32 heads x 8K tokens 54.8 -> 53.3 us, 128K 93.4 -> 91.2; a filter and its
-// attention at 20K 65.5 -> 59.7.  The pyramid build stays an ordinary kernel
+// 32 heads x 8K tokens 51.1 -> 49.3 us, 128K 92.7 -> 89.1; a filter and its
+// attention at 20K 64.5 -> 58.4.  The pyramid build stays an ordinary kernel
 // (`plain`): its 16,000 short CTAs slowed down with the two instructions, 391
 // against 425 us for a build and a step.
 struct Launch {
