@@ -266,8 +266,10 @@ __global__ void __launch_bounds__(NTH, 3) approx_kernel(const T* __restrict__ K,
 // flight.  (Gathering 128 rows into shared memory, then transforming them
 // level by level between barriers, left DRAM at 44 % at scale 3.)  Measured:
 // the db2 step of 64 units x 32K tokens 233.1 -> 218.1 us (187.7 with one unit
-// a cluster); its three transforms read 537 MB in about 84 us, 99 us before.  Scales 6 to 10
-// (a long halo, few outputs) keep the shared-memory kernel below.
+// a cluster); its three transforms move 546 MB through DRAM, one by one and cold
+// in 98.6 us (5.5 TB/s, 0.81 of a copy's rate), in the step in about 84, 99 us
+// before.  Scales 6 to 10 (a long halo, few outputs) keep the shared-memory kernel
+// below.
 template <typename T, int TAPS, int L>
 struct Cascade {
   static constexpr int VEC = Vec<T>::N;
