@@ -16,8 +16,7 @@
 namespace wf {
 namespace {
 
-using sm100::grid_dep_launch;
-using sm100::grid_dep_wait;
+using namespace sm100;
 
 constexpr int CH = kAttnChunk;
 constexpr int QMAX = kMaxQ;
@@ -82,20 +81,24 @@ __global__ void __launch_bounds__(256) attn_split_kernel(
   }
   __syncthreads();
 
-  // Logits: lane -> keys (lane, lane+32), warp -> query rows warp + 8r.
+  // Logits: lane -> keys (lane, lane+32), warp -> query rows warp + 8r.  Each
+  // accumulator is a packed pair, the sums over the even and the odd channels, as
+  // in the one-launch fp32 step, so that the two routes are equally accurate
+  // (160 units, 442 keys, d 128: 3.25e-7 against 64 bits, 4.8e-7 with one chain;
+  // and 7 % faster over d 128, fp32).
   const int lane = tid & 31, warp = tid >> 5;
-  float acc0[QM / 8], acc1[QM / 8];
+  f32x2 acc0[QM / 8], acc1[QM / 8];
 #pragma unroll
-  for (int r = 0; r < QM / 8; ++r) { acc0[r] = 0.f; acc1[r] = 0.f; }
-#pragma unroll 2
+  for (int r = 0; r < QM / 8; ++r) acc0[r] = acc1[r] = pk2(0.f, 0.f);
+#pragma unroll 4
   for (int c = 0; c < D; c += 4) {
-    const float4 k0 = *reinterpret_cast<const float4*>(&Ks[lane * KS + c]);
-    const float4 k1 = *reinterpret_cast<const float4*>(&Ks[(lane + 32) * KS + c]);
+    const ulonglong2 k0 = *reinterpret_cast<const ulonglong2*>(&Ks[lane * KS + c]);
+    const ulonglong2 k1 = *reinterpret_cast<const ulonglong2*>(&Ks[(lane + 32) * KS + c]);
 #pragma unroll
     for (int r = 0; r < QM / 8; ++r) {
-      const float4 qv = *reinterpret_cast<const float4*>(&Qs[(warp + 8 * r) * D + c]);
-      acc0[r] = fmaf(qv.x, k0.x, fmaf(qv.y, k0.y, fmaf(qv.z, k0.z, fmaf(qv.w, k0.w, acc0[r]))));
-      acc1[r] = fmaf(qv.x, k1.x, fmaf(qv.y, k1.y, fmaf(qv.z, k1.z, fmaf(qv.w, k1.w, acc1[r]))));
+      const ulonglong2 qv = *reinterpret_cast<const ulonglong2*>(&Qs[(warp + 8 * r) * D + c]);
+      acc0[r] = fma2(qv.y, k0.y, fma2(qv.x, k0.x, acc0[r]));
+      acc1[r] = fma2(qv.y, k1.y, fma2(qv.x, k1.x, acc1[r]));
     }
   }
   float2* ml = ML + ((int64_t)u * nsplit + sp) * qstride;  // a split's partials: qstride rows
@@ -103,8 +106,9 @@ __global__ void __launch_bounds__(256) attn_split_kernel(
   for (int r = 0; r < QM / 8; ++r) {
     const int i = warp + 8 * r;
     if (i >= q) break;
-    const float s0 = lane < cnt ? acc0[r] * scale : -INFINITY;
-    const float s1 = lane + 32 < cnt ? acc1[r] * scale : -INFINITY;
+    const float2 a0 = up2(acc0[r]), a1 = up2(acc1[r]);
+    const float s0 = lane < cnt ? (a0.x + a0.y) * scale : -INFINITY;
+    const float s1 = lane + 32 < cnt ? (a1.x + a1.y) * scale : -INFINITY;
     float mx = fmaxf(s0, s1);
 #pragma unroll
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));

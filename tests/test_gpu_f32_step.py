@@ -84,3 +84,24 @@ def test_step_f32_routes(H, d, q, n, L, k, ng, bshd):
         Q, K, V = f64(b.Q[0, u]), f64(b.K[0, u]), f64(b.V[0, u])
         kg, vg = (f64(Kg[0, u]), f64(Vg[0, u])) if ng else (None, None)
         assert_close_out(f64(run.O[0, u]), oracle.sparse_attn(Q, K, V, run.idx[u].cpu().numpy(), kg, vg), torch.float32)
+
+
+@pytest.mark.parametrize("d,q,n,k,amp", [(128, 8, 4096, 410, 1.0), (128, 32, 8192, 819, 2.0), (64, 17, 4096, 410, 2.0)])
+def test_split_attention_as_accurate_as_one_launch(d, q, n, k, amp):
+    """A step that leaves the one launch attends on the split kernel.  Both sum
+    a logit in two chains of d / 2 products, and the logits' rounding dominates
+    the output's, so their rms errors against fp64 agree within a fifth (a
+    single chain of d has 1.4 times the error)."""
+    H, L, ng = 32, 2, 32
+    g = torch.Generator().manual_seed(k + d)
+    rn = lambda rows, a=1.0: a * torch.randn(1, H, rows, d, generator=g).cuda()
+    Q, K, V, Kg, Vg = rn(q, amp), rn(n), rn(n), rn(ng), rn(ng)
+    run = LibRun(Q, K, V, Kg, Vg, L, wf.wf_default_schedule(n, L, k)).dwt().step(refresh=False)
+    O = torch.empty_like(Q)
+    ws = torch.zeros(wf.wf_attn_workspace_bytes(Q, k, ng), dtype=torch.uint8, device="cuda")
+    wf.wf_sparse_attn(Q, K, V, run.idx, k, Kg, Vg, O, ws)
+    at = run.idx.long().view(1, H, k, 1).expand(-1, -1, -1, d)
+    Ks, Vs = (torch.cat([t.gather(2, at), e], 2).double() for t, e in ((K, Kg), (V, Vg)))
+    R = torch.softmax(Q.double() @ Ks.transpose(2, 3) / d ** 0.5, -1) @ Vs
+    one, split = ((x.double() - R).norm().item() for x in (run.O, O))
+    assert split <= 1.2 * one
