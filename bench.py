@@ -106,7 +106,8 @@ def fused_shape(w: synth.Workload) -> bool:
 
 
 def f32_fused(w: synth.Workload) -> bool:
-    """wf_step runs its single fp32 kernel (one query head per key head)."""
+    """wf_step runs its single fp32 kernel (one query head per key head; every
+    workload here is within that route)."""
     return WAVELET is None and w.dtype == "f32" and w.group == 1
 
 
