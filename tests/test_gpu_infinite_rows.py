@@ -10,7 +10,6 @@ fp32 sums of 64 terms can move (2^-17), so that no near-tie decides.
 
 In the attention such a row adds nothing, also where it fills a whole tile or
 slice: outputs within the bounds of the other tests."""
-import dataclasses
 
 import numpy as np
 import pytest
